@@ -46,67 +46,205 @@ struct Gas {
 constexpr int NN_HIDDEN = 32;
 constexpr int NN_PARAMS = 32 * 4 + 32 + 2 * (32 * 32 + 32) + 32 + 1;
 
-template <typename T> JF_HD T tsqrt(T x);
-template <> JF_HD float tsqrt<float>(float x) { return sqrtf(x); }
-template <> JF_HD double tsqrt<double>(double x) { return sqrt(x); }
-
-// Reciprocal of the point-wise numerics.  FP32 device code takes the
-// hardware approximate reciprocal (__fdividef: one MUFU operation, within
-// 2 ulp for |x| < 2^126); FP64 and host code divide exactly.
-template <typename T> JF_HD T trcp(T x) { return T(1) / x; }
+// Reciprocal and square roots of the point-wise numerics.  FP32 device code
+// takes the hardware approximations (rcp.approx.ftz: one MUFU operation,
+// within 1 ulp for |x| < 2^126; host code divides exactly).  FP64 device code
+// starts from the PTX approximations rcp / rsqrt.approx.ftz.f64 (about 20
+// bits, not on the FP64 pipe) and refines them with one third-order step,
+// Chebyshev's y + y (e + e^2) with e = 1 - x y and Halley's
+// s + s e (1/2 + 3/8 e) with e = 1 - x y^2: 3 and 5 FP64 operations, where an
+// IEEE division or square root takes about ten and the FP64 pipe (2 FMA per
+// clock and SM) is what bounds the FP64 kernels.  The results are within 1
+// ulp (measured over exponents -1000..1000).  FP32: against __fdividef, whose
+// multiplication it saves, the same bits, and the ROE step at 128^3 takes 903
+// instead of 941 us, the default one at 256^3 4.205 instead of 4.264 ms.
+template <typename T> JF_HD T trcp(T x);
 template <> JF_HD float trcp<float>(float x) {
 #ifdef __CUDA_ARCH__
-  return __fdividef(1.0f, x);
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 #else
   return 1.0f / x;
+#endif
+}
+template <> JF_HD double trcp<double>(double x) {
+#ifdef __CUDA_ARCH__
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+#else
+  return 1.0 / x;
+#endif
+}
+
+// 1 / sqrt(x) in FP64 (x > 0).
+JF_HD double trsqrt(double x) {
+#ifdef __CUDA_ARCH__
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+#else
+  return 1.0 / sqrt(x);
+#endif
+}
+
+template <typename T> JF_HD T tsqrt(T x);
+template <> JF_HD float tsqrt<float>(float x) { return sqrtf(x); }
+template <> JF_HD double tsqrt<double>(double x) {
+#ifdef __CUDA_ARCH__
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double r = x * y, e = fma(-r, y, 1.0);
+  const double s = fma(r * e, fma(0.375, e, 0.5), r);
+  return __double2hiint(x) == 0 ? 0.0 : s;  // sqrt(0) (a 32-bit compare)
+#else
+  return sqrt(x);
 #endif
 }
 
 template <typename T> JF_HD T tmin(T a, T b) { return b < a ? b : a; }
 template <typename T> JF_HD T tmax(T a, T b) { return a < b ? b : a; }
 
-// WENO5-JS: value at x_{i+1/2} biased to the left, from v[i-2..i+2].
-// Candidate stencils q_k, smoothness indicators beta_k, weights
+// WENO5-JS (Jiang & Shu 1996): value at x_{i+1/2} biased to the left, from
+// v[i-2..i+2]: candidate stencils q_k, smoothness indicators beta_k, weights
 // alpha_k = d_k / (eps + beta_k)^2 with d = (1/10, 6/10, 3/10),
-// omega_k = alpha_k / sum(alpha).
-// With z != 0 the WENO5-Z weights of Borges et al. (2008) replace the JS
-// ones: tau5 = |beta_0 - beta_2|, alpha_k = d_k (1 + tau5 / (eps + beta_k)).
+// omega_k = alpha_k / sum(alpha).  With z != 0 the WENO5-Z weights of Borges
+// et al. (2008) replace the JS ones: tau5 = |beta_0 - beta_2|,
+// alpha_k = d_k (1 + tau5 / (eps + beta_k)).
+//
+// Evaluated in differences, which takes the fewest operations (the kernels
+// are bound by the arithmetic pipes).  With D2 = v0 - v[-1], D3 = v[1] - v0
+// and the second differences d0, d1, d2 of the three sub-stencils,
+//   beta_0 = 4/3 d0^2 + d0 D2 + D2^2, beta_1 = 4/3 d1^2 + d1 D2 + D2^2,
+//   beta_2 = 4/3 d2^2 + d2 D3 + D3^2
+// (positive definite forms, no cancellation beyond a factor of 2), so that
+// D2^2 + eps serves two of them, and with the weights (1, 6, 3) r_k
+//   v^ = v0 + [a0 (d0/3 + D2/2) + a1 (d1/3 + D2/2) + a2 (d2/6 + D3/2)] / (a0 + a1 + a2).
+template <typename T>
+struct WenoTerms {
+  T d0, d1, d2;  // second differences of the sub-stencils
+  T h2, h3;      // D2 / 2, D3 / 2
+  T t0, t1, t2;  // eps + beta_k
+};
+
+template <typename T>
+JF_HD WenoTerms<T> weno5_terms(T vm2, T vm1, T v0, T vp1, T vp2, T eps) {
+  WenoTerms<T> w;
+  const T D2 = v0 - vm1, D3 = vp1 - v0;
+  w.d0 = D2 + (vm2 - vm1);
+  w.d1 = D3 - D2;
+  w.d2 = D3 + (vp1 - vp2);
+  const T q2 = D2 * D2 + eps, q3 = D3 * D3 + eps, k = T(4) / T(3);
+  w.t0 = w.d0 * (k * w.d0 + D2) + q2;
+  w.t1 = w.d1 * (k * w.d1 + D2) + q2;
+  w.t2 = w.d2 * (k * w.d2 + D3) + q3;
+  w.h2 = T(0.5) * D2;
+  w.h3 = T(0.5) * D3;
+  return w;
+}
+
+// The factors r_k of the weights, up to a common factor.  FP64: scaled by
+// (t0 t1 t2)^2 (JS; WENO5-Z: t0 t1 t2), so that no reciprocal is taken here
+// (the factors are >= eps, far inside the FP64 range).
+template <typename T>
+JF_HD void weno5_factors(const WenoTerms<T>& w, int z, T& r0, T& r1, T& r2) {
+  if constexpr (sizeof(T) == 8) {
+    if (z) {
+      const T tau = fabs(w.t0 - w.t2);
+      r0 = (w.t0 + tau) * (w.t1 * w.t2);
+      r1 = (w.t1 + tau) * (w.t0 * w.t2);
+      r2 = (w.t2 + tau) * (w.t0 * w.t1);
+    } else {
+      const T s0 = w.t0 * w.t0, s1 = w.t1 * w.t1, s2 = w.t2 * w.t2;
+      r0 = s1 * s2;
+      r1 = s0 * s2;
+      r2 = s0 * s1;
+    }
+  } else {
+    if (z) {
+      const T tau = fabs(w.t0 - w.t2);
+      r0 = (w.t0 + tau) * trcp(w.t0);
+      r1 = (w.t1 + tau) * trcp(w.t1);
+      r2 = (w.t2 + tau) * trcp(w.t2);
+    } else {
+      r0 = trcp(w.t0 * w.t0);
+      r1 = trcp(w.t1 * w.t1);
+      r2 = trcp(w.t2 * w.t2);
+    }
+  }
+}
+
 template <typename T>
 JF_HD T weno5(T vm2, T vm1, T v0, T vp1, T vp2, T eps, int z = 0) {
-  const T sixth = T(1) / T(6);
-  const T q0 = (T(2) * vm2 - T(7) * vm1 + T(11) * v0) * sixth;
-  const T q1 = (-vm1 + T(5) * v0 + T(2) * vp1) * sixth;
-  const T q2 = (T(2) * v0 + T(5) * vp1 - vp2) * sixth;
-  const T c13 = T(13) / T(12);
-  const T d0 = vm2 - T(2) * vm1 + v0, e0 = vm2 - T(4) * vm1 + T(3) * v0;
-  const T d1 = vm1 - T(2) * v0 + vp1, e1 = vm1 - vp1;
-  const T d2 = v0 - T(2) * vp1 + vp2, e2 = T(3) * v0 - T(4) * vp1 + vp2;
-  const T b0 = c13 * d0 * d0 + T(0.25) * e0 * e0;
-  const T b1 = c13 * d1 * d1 + T(0.25) * e1 * e1;
-  const T b2 = c13 * d2 * d2 + T(0.25) * e2 * e2;
-  const T t0 = eps + b0, t1 = eps + b1, t2 = eps + b2;
+  const WenoTerms<T> w = weno5_terms(vm2, vm1, v0, vp1, vp2, eps);
+  T a0, a1, a2;
+  weno5_factors(w, z, a0, a1, a2);
+  a1 = T(6) * a1;
+  a2 = T(3) * a2;
+  const T third = T(1) / T(3), sixth = T(1) / T(6);
+  const T num = a0 * (third * w.d0 + w.h2) + a1 * (third * w.d1 + w.h2) + a2 * (sixth * w.d2 + w.h3);
+  return v0 + num * trcp(a0 + a1 + a2);
+}
+
+// WENO5 per cell: both face values one cell j contributes, from the same
+// five values v[j-2..j+2]:
+//   right = v^-_{j+1/2} (left-biased, the weno5 formula above),
+//   left  = v^+_{j-1/2} (right-biased: the same formula on the mirrored
+//           stencil v[j+2..j-2]).
+// The mirrored stencil has the smoothness indicators in reverse order (the
+// three 3-cell sub-stencils are the same) and the differences reversed and
+// negated, so both values share the indicators and the factors r_k:
+//   left = v0 - [r2 (d2/3 + D3/2) + 6 r1 (d1/6 + D2/2) + 3 r0 (d0/6 + D2/2)] / (r2 + 6 r1 + 3 r0).
+template <typename T>
+JF_HD void weno5_cell_lean(T vm2, T vm1, T v0, T vp1, T vp2, T eps, T& right, T& left, int z = 0) {
+  const WenoTerms<T> w = weno5_terms(vm2, vm1, v0, vp1, vp2, eps);
+  T r0, r1, r2;
+  weno5_factors(w, z, r0, r1, r2);
+  const T a1 = T(6) * r1, a2 = T(3) * r2, c0 = T(3) * r0;
+  const T third = T(1) / T(3), sixth = T(1) / T(6);
+  const T Sr = r0 + a1 + a2, Sl = c0 + a1 + r2;
+  const T nr = r0 * (third * w.d0 + w.h2) + a1 * (third * w.d1 + w.h2) + a2 * (sixth * w.d2 + w.h3);
+  const T nl = c0 * (sixth * w.d0 + w.h2) + a1 * (sixth * w.d1 + w.h2) + r2 * (third * w.d2 + w.h3);
   if constexpr (sizeof(T) == 8) {
-    // alpha_k scaled by a common product of the (eps + beta_j) terms: one
-    // division instead of four (the factors are >= eps, far inside the FP64
-    // range).  JS: alpha_k ~ d_k / t_k^2, scaled by (t0 t1 t2)^2; Z:
-    // alpha_k ~ d_k (t_k + tau5) / t_k, scaled by t0 t1 t2.
-    T a0, a1, a2;
-    if (z) {
-      const T tau = fabs(b0 - b2);
-      a0 = T(0.1) * (t0 + tau) * t1 * t2;
-      a1 = T(0.6) * (t1 + tau) * t0 * t2;
-      a2 = T(0.3) * (t2 + tau) * t0 * t1;
-    } else {
-      const T s0 = t0 * t0, s1 = t1 * t1, s2 = t2 * t2;
-      a0 = T(0.1) * s1 * s2;
-      a1 = T(0.6) * s0 * s2;
-      a2 = T(0.3) * s0 * s1;
-    }
-    return (a0 * q0 + a1 * q1 + a2 * q2) / (a0 + a1 + a2);
+    // one reciprocal for both values: 1/S_r = S_l / (S_r S_l) and the converse
+    // (S >= 1e-23 as every s_k >= eps^2; the product stays far inside the
+    // FP64 range)
+    const T inv = trcp(Sr * Sl);
+    right = v0 + nr * (Sl * inv);
+    left = v0 - nl * (Sr * inv);
   } else {
+    right = v0 + nr * trcp(Sr);
+    left = v0 - nl * trcp(Sl);
+  }
+}
+
+// The FP32 tile kernels (1D, 2D, 3D) keep an earlier grouping of the same
+// formulas, with three independent indicators: their states enter numbers
+// that are reported in FP64 (the CFL step, the loss at the end of a
+// trajectory), which another FP32 rounding moves by 1e-9 to 1e-7.  The lean
+// form above serves the row tiles and FP64 (see cell_recon).
+template <typename T>
+JF_HD void weno5_cell(T vm2, T vm1, T v0, T vp1, T vp2, T eps, T& right, T& left, int z = 0) {
+  if constexpr (sizeof(T) == 8) {
+    weno5_cell_lean(vm2, vm1, v0, vp1, vp2, eps, right, left, z);
+  } else {
+    const T D1 = vm2 - vm1, D2 = v0 - vm1, D3 = vp1 - v0, D4 = vp1 - vp2;
+    const T c13 = T(13) / T(12);
+    const T d0 = D2 + D1, e0 = T(3) * D2 + D1;
+    const T d1 = D3 - D2, e1 = D2 + D3;
+    const T d2 = D3 + D4, e2 = T(3) * D3 + D4;
+    const T t0 = eps + (c13 * d0 * d0 + T(0.25) * e0 * e0);
+    const T t1 = eps + (c13 * d1 * d1 + T(0.25) * e1 * e1);
+    const T t2 = eps + (c13 * d2 * d2 + T(0.25) * e2 * e2);
+    // candidate offsets q_k - v0 (times 6) of both reconstructions
+    const T g0 = T(5) * D2 + T(2) * D1, g1 = D2 + T(2) * D3, g2 = T(4) * D3 + D4;
+    const T h0 = -(T(5) * D3 + T(2) * D4), h1 = -(D3 + T(2) * D2), h2 = -(T(4) * D2 + D1);
     T r0, r1, r2;
     if (z) {
-      const T tau = fabs(b0 - b2);
+      const T tau = fabs(t0 - t2);
       r0 = (t0 + tau) * trcp(t0);
       r1 = (t1 + tau) * trcp(t1);
       r2 = (t2 + tau) * trcp(t2);
@@ -116,9 +254,14 @@ JF_HD T weno5(T vm2, T vm1, T v0, T vp1, T vp2, T eps, int z = 0) {
       r2 = trcp(t2 * t2);
     }
     const T a0 = T(0.1) * r0, a1 = T(0.6) * r1, a2 = T(0.3) * r2;
-    return (a0 * q0 + a1 * q1 + a2 * q2) * trcp(a0 + a1 + a2);
+    const T b0 = T(0.1) * r2, b2 = T(0.3) * r0;
+    right = v0 + (a0 * g0 + a1 * g1 + a2 * g2) * trcp(T(6) * (a0 + a1 + a2));
+    left = v0 + (b0 * h0 + a1 * h1 + b2 * h2) * trcp(T(6) * (b0 + a1 + b2));
   }
 }
+
+__device__ __forceinline__ float2 splat2(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 rcp2(float2 x) { return make_float2(trcp(x.x), trcp(x.y)); }
 
 // The left and right WENO5-JS states of one face component in packed FP32x2
 // arithmetic (sm_100+ FFMA2 / FADD2 / FMUL2): lane x reconstructs
@@ -152,7 +295,6 @@ __device__ __forceinline__ float2 weno5_pair(float2 vm2, float2 vm1, float2 v0, 
   const float2 t1 = __ffma2_rn(d1, d1, __ffma2_rn(__fmul2_rn(k3, e1), e1, ke));
   const float2 t2 = __ffma2_rn(d2, d2, __ffma2_rn(__fmul2_rn(k3, e2), e2, ke));
   // approximate reciprocals (t_k^2 >= (12/13 eps)^2 > 0, so the sum is > 0)
-  auto rcp2 = [](float2 x) { return make_float2(__fdividef(1.0f, x.x), __fdividef(1.0f, x.y)); };
   float2 r0, r1, r2;
   if (z) {
     const float2 d02 = __ffma2_rn(m1, t2, t0);
@@ -173,83 +315,6 @@ __device__ __forceinline__ float2 weno5_pair(float2 vm2, float2 vm1, float2 v0, 
   return __ffma2_rn(num, rcp2(den), v0);
 }
 
-// WENO5-JS per cell: both face values one cell j contributes, from the same
-// five values v[j-2..j+2]:
-//   right = v^-_{j+1/2} (left-biased, the weno5 formula above),
-//   left  = v^+_{j-1/2} (right-biased: the same formula on the mirrored
-//           stencil v[j+2..j-2]).
-// The mirrored stencil has the smoothness indicators in reverse order
-// (beta'_k = beta_{2-k}: the three 3-cell sub-stencils are the same), so
-// both values share the indicators and their reciprocals; only the linear
-// weights and candidates differ.  With the differences D1..D4 of weno5_pair
-// the mirrored ones are D1' = -D4, D2' = -D3, D3' = -D2, D4' = -D1.
-// Equal to two weno5 calls up to rounding.  z = 1: WENO5-Z (Table 2; alpha_k
-// = d_k (1 + tau5 / (eps + beta_k)), tau5 = |beta_0 - beta_2|, the same for
-// the mirrored stencil, so the two values share the weights' factors too).
-template <typename T>
-JF_HD void weno5_cell(T vm2, T vm1, T v0, T vp1, T vp2, T eps, T& right, T& left, int z = 0) {
-  const T D1 = vm2 - vm1, D2 = v0 - vm1, D3 = vp1 - v0, D4 = vp1 - vp2;
-  const T c13 = T(13) / T(12);
-  const T d0 = D2 + D1, e0 = T(3) * D2 + D1;
-  const T d1 = D3 - D2, e1 = D2 + D3;
-  const T d2 = D3 + D4, e2 = T(3) * D3 + D4;
-  const T t0 = eps + (c13 * d0 * d0 + T(0.25) * e0 * e0);
-  const T t1 = eps + (c13 * d1 * d1 + T(0.25) * e1 * e1);
-  const T t2 = eps + (c13 * d2 * d2 + T(0.25) * e2 * e2);
-  // candidate offsets q_k - v0 (times 6) of both reconstructions
-  const T g0 = T(5) * D2 + T(2) * D1, g1 = D2 + T(2) * D3, g2 = T(4) * D3 + D4;
-  const T h0 = -(T(5) * D3 + T(2) * D4), h1 = -(D3 + T(2) * D2), h2 = -(T(4) * D2 + D1);
-  if constexpr (sizeof(T) == 8) {
-    // alpha_k scaled by the common product (t0 t1 t2)^2 (one division per
-    // value; the factors are >= eps, far inside the FP64 range):
-    // right: (0.1 s1 s2, 0.6 s0 s2, 0.3 s0 s1); left (mirrored t):
-    // (0.1 s0 s1, 0.6 s0 s2, 0.3 s1 s2), s_k = t_k^2.  WENO5-Z: the factors
-    // 1 + tau5 / t_k scaled by t0 t1 t2: u_k = (t_k + tau5) t_i t_j, the left
-    // value taking them in reverse order
-    T a0, a1, a2, b0, b2;
-    if (z) {
-      const T tau = fabs(t0 - t2);
-      const T u0 = (t0 + tau) * (t1 * t2), u1 = (t1 + tau) * (t0 * t2), u2 = (t2 + tau) * (t0 * t1);
-      a0 = T(0.1) * u0;
-      a1 = T(0.6) * u1;
-      a2 = T(0.3) * u2;
-      b0 = T(0.1) * u2;
-      b2 = T(0.3) * u0;
-    } else {
-      const T s0 = t0 * t0, s1 = t1 * t1, s2 = t2 * t2;
-      const T p12 = s1 * s2, p02 = s0 * s2, p01 = s0 * s1;
-      a0 = T(0.1) * p12;
-      a1 = T(0.6) * p02;
-      a2 = T(0.3) * p01;
-      b0 = T(0.1) * p01;
-      b2 = T(0.3) * p12;
-    }
-    // one division for both values: 1/D_r = D_l / (D_r D_l) and the converse
-    // (D >= 6e-25 as every s_k >= eps^2; the product stays far inside the
-    // FP64 range)
-    const T Dr = T(6) * (a0 + a1 + a2), Dl = T(6) * (b0 + a1 + b2);
-    const T inv = T(1) / (Dr * Dl);
-    right = v0 + (a0 * g0 + a1 * g1 + a2 * g2) * (Dl * inv);
-    left = v0 + (b0 * h0 + a1 * h1 + b2 * h2) * (Dr * inv);
-  } else {
-    T r0, r1, r2;
-    if (z) {
-      const T tau = fabs(t0 - t2);
-      r0 = (t0 + tau) * trcp(t0);
-      r1 = (t1 + tau) * trcp(t1);
-      r2 = (t2 + tau) * trcp(t2);
-    } else {
-      r0 = trcp(t0 * t0);
-      r1 = trcp(t1 * t1);
-      r2 = trcp(t2 * t2);
-    }
-    const T a0 = T(0.1) * r0, a1 = T(0.6) * r1, a2 = T(0.3) * r2;
-    const T b0 = T(0.1) * r2, b2 = T(0.3) * r0;
-    right = v0 + (a0 * g0 + a1 * g1 + a2 * g2) * trcp(T(6) * (a0 + a1 + a2));
-    left = v0 + (b0 * h0 + a1 * h1 + b2 * h2) * trcp(T(6) * (b0 + a1 + b2));
-  }
-}
-
 // weno5_cell for two components of one cell in the lanes of packed FP32x2
 // operations (the arithmetic of weno5_pair: indicators scaled by 12/13,
 // linear weights scaled by 10/3; z = 1: WENO5-Z as in weno5_cell).
@@ -268,7 +333,6 @@ __device__ __forceinline__ void weno5_cell_pair(float2 vm2, float2 vm1, float2 v
   const float2 t0 = __ffma2_rn(d0, d0, __ffma2_rn(__fmul2_rn(k3, e0), e0, ke));
   const float2 t1 = __ffma2_rn(d1, d1, __ffma2_rn(__fmul2_rn(k3, e1), e1, ke));
   const float2 t2 = __ffma2_rn(d2, d2, __ffma2_rn(__fmul2_rn(k3, e2), e2, ke));
-  auto rcp2 = [](float2 x) { return make_float2(__fdividef(1.0f, x.x), __fdividef(1.0f, x.y)); };
   float2 r0, r1, r2;
   if (z) {
     const float2 d02 = __ffma2_rn(m1, t2, t0);
@@ -297,6 +361,44 @@ __device__ __forceinline__ void weno5_cell_pair(float2 vm2, float2 vm1, float2 v
   left = __ffma2_rn(numl, rcp2(denl), v0);
 }
 
+// weno5_cell_lean for two components of one cell in the lanes: 41 packed
+// operations and 10 reciprocals where weno5_cell_pair takes 46 and 10.
+__device__ __forceinline__ void weno5_cell_pair_lean(float2 vm2, float2 vm1, float2 v0, float2 vp1, float2 vp2,
+                                                     float eps, float2& right, float2& left, int z = 0) {
+  const float2 m1 = splat2(-1.0f), k = splat2(4.0f / 3.0f), ke = splat2(eps);
+  const float2 D2 = __ffma2_rn(m1, vm1, v0), D3 = __ffma2_rn(m1, v0, vp1);
+  const float2 d0 = __fadd2_rn(D2, __ffma2_rn(m1, vm1, vm2));
+  const float2 d1 = __ffma2_rn(m1, D2, D3);
+  const float2 d2 = __fadd2_rn(D3, __ffma2_rn(m1, vp2, vp1));
+  const float2 q2 = __ffma2_rn(D2, D2, ke), q3 = __ffma2_rn(D3, D3, ke);
+  const float2 t0 = __ffma2_rn(d0, __ffma2_rn(k, d0, D2), q2);
+  const float2 t1 = __ffma2_rn(d1, __ffma2_rn(k, d1, D2), q2);
+  const float2 t2 = __ffma2_rn(d2, __ffma2_rn(k, d2, D3), q3);
+  float2 r0, r1, r2;
+  // approximate reciprocals (t_k^2 >= eps^2 > 0, so the sums are > 0)
+  if (z) {
+    const float2 d02 = __ffma2_rn(m1, t2, t0);
+    const float2 tau = make_float2(fabsf(d02.x), fabsf(d02.y));
+    r0 = __fmul2_rn(__fadd2_rn(t0, tau), rcp2(t0));
+    r1 = __fmul2_rn(__fadd2_rn(t1, tau), rcp2(t1));
+    r2 = __fmul2_rn(__fadd2_rn(t2, tau), rcp2(t2));
+  } else {
+    r0 = rcp2(__fmul2_rn(t0, t0));
+    r1 = rcp2(__fmul2_rn(t1, t1));
+    r2 = rcp2(__fmul2_rn(t2, t2));
+  }
+  const float2 a1 = __fmul2_rn(splat2(6.0f), r1), a2 = __fmul2_rn(splat2(3.0f), r2), c0 = __fmul2_rn(splat2(3.0f), r0);
+  const float2 h2 = __fmul2_rn(splat2(0.5f), D2), h3 = __fmul2_rn(splat2(0.5f), D3);
+  const float2 third = splat2(1.0f / 3.0f), sixth = splat2(1.0f / 6.0f);
+  const float2 nr = __ffma2_rn(a2, __ffma2_rn(sixth, d2, h3),
+                               __ffma2_rn(a1, __ffma2_rn(third, d1, h2), __fmul2_rn(r0, __ffma2_rn(third, d0, h2))));
+  const float2 nl = __ffma2_rn(r2, __ffma2_rn(third, d2, h3),
+                               __ffma2_rn(a1, __ffma2_rn(sixth, d1, h2), __fmul2_rn(c0, __ffma2_rn(sixth, d0, h2))));
+  const float2 Sr = __fadd2_rn(__fadd2_rn(r0, a1), a2), Sl = __fadd2_rn(__fadd2_rn(c0, a1), r2);
+  right = __ffma2_rn(nr, rcp2(Sr), v0);
+  left = __ffma2_rn(nl, make_float2(trcp(-Sl.x), trcp(-Sl.y)), v0);
+}
+
 // WENO3-JS (Table 2): value at x_{i+1/2} biased to the left from
 // v[i-1], v[i], v[i+1]: q0 = (3 v[i] - v[i-1]) / 2, q1 = (v[i] + v[i+1]) / 2,
 // beta0 = (v[i] - v[i-1])^2, beta1 = (v[i+1] - v[i])^2,
@@ -322,9 +424,10 @@ __device__ __forceinline__ float2 weno3_pair(float2 vm1, float2 v0, float2 vp1, 
 //   Toro (1994): PVRS pressure p* = max(0, (p_L + p_R)/2 - (u_R - u_L)(rho_L + rho_R)(c_L + c_R)/8);
 //     q_K = 1 if p* <= p_K else sqrt(1 + (gamma + 1)/(2 gamma)(p*/p_K - 1));
 //     S_L = u_L - c_L q_L, S_R = u_R + c_R q_R.
+// q = sqrt(rho_R / rho_L), read by Einfeldt's estimate.
 template <typename T, int D>
-JF_HD void signal_speeds(const T WL[5], const T WR[5], const Gas<T>& g, int speeds, T EL, T ER, T irL, T irR, T cL,
-                         T cR, T& SL, T& SR) {
+JF_HD void signal_speeds(const T WL[5], const T WR[5], const Gas<T>& g, int speeds, T EL, T ER, T irL, T irR, T q,
+                         T cL, T cR, T& SL, T& SR) {
   const T rL = WL[0], rR = WR[0], pL = WL[4], pR = WR[4];
   const T unL = WL[1 + D], unR = WR[1 + D];
   if (speeds == 1) {
@@ -338,9 +441,8 @@ JF_HD void signal_speeds(const T WL[5], const T WR[5], const Gas<T>& g, int spee
     SL = unL - cL * qL;
     SR = unR + cR * qR;
   } else {
-    // Roe weights sqrt(rho_K) / (sqrt(rho_L) + sqrt(rho_R)) from the ratio
-    // q = sqrt(rho_R / rho_L): w_L = 1 / (1 + q), w_R = q w_L
-    const T q = tsqrt(rR * irL);
+    // Roe weights sqrt(rho_K) / (sqrt(rho_L) + sqrt(rho_R)):
+    // w_L = 1 / (1 + q), w_R = q w_L
     const T wL = trcp(T(1) + q), wR = q * wL;
     const T HL = (EL + pL) * irL, HR = (ER + pR) * irR;
     const T u0 = wL * WL[1] + wR * WR[1];
@@ -362,15 +464,17 @@ JF_HD void side_state(const T W[5], const Gas<T>& g, T& E, T& ir, T& c) {
   c = tsqrt(g.gamma * W[4] * ir);
 }
 
-// Both sides' E, 1/rho and c; FP64 forms the two reciprocals from one
-// division, 1/rho_L = rho_R / (rho_L rho_R) and the converse.
+// Both sides' E, 1/rho and c, and q = sqrt(rho_R / rho_L); FP64 forms the
+// reciprocals and q from one inverse square root y = (rho_L rho_R)^(-1/2):
+// q = rho_R y, 1/rho_L = q y, 1/rho_R = rho_L y^2.
 template <typename T>
-JF_HD void side_states(const T WL[5], const T WR[5], const Gas<T>& g, T& EL, T& ER, T& irL, T& irR, T& cL,
+JF_HD void side_states(const T WL[5], const T WR[5], const Gas<T>& g, T& EL, T& ER, T& irL, T& irR, T& q, T& cL,
                        T& cR) {
   if constexpr (sizeof(T) == 8) {
-    const T inv = T(1) / (WL[0] * WR[0]);
-    irL = WR[0] * inv;
-    irR = WL[0] * inv;
+    const T y = trsqrt(WL[0] * WR[0]);
+    q = WR[0] * y;
+    irL = q * y;
+    irR = WL[0] * y * y;
     EL = WL[4] * g.inv_gm1 + T(0.5) * WL[0] * (WL[1] * WL[1] + WL[2] * WL[2] + WL[3] * WL[3]);
     ER = WR[4] * g.inv_gm1 + T(0.5) * WR[0] * (WR[1] * WR[1] + WR[2] * WR[2] + WR[3] * WR[3]);
     cL = tsqrt(g.gamma * WL[4] * irL);
@@ -378,6 +482,7 @@ JF_HD void side_states(const T WL[5], const T WR[5], const Gas<T>& g, T& EL, T& 
   } else {
     side_state(WL, g, EL, irL, cL);
     side_state(WR, g, ER, irR, cR);
+    q = tsqrt(WR[0] * irL);
   }
 }
 
@@ -412,10 +517,10 @@ JF_HD void hllc(const T WL[5], const T WR[5], const Gas<T>& g, T F[5], int speed
   const T rL = WL[0], rR = WR[0], pL = WL[4], pR = WR[4];
   const T unL = WL[1 + D], unR = WR[1 + D];
   // every division goes through a reciprocal (1/rho of each side shared)
-  T EL, ER, irL, irR, cL, cR;
-  side_states(WL, WR, g, EL, ER, irL, irR, cL, cR);
+  T EL, ER, irL, irR, q, cL, cR;
+  side_states(WL, WR, g, EL, ER, irL, irR, q, cL, cR);
   T SL, SR;
-  signal_speeds<T, D>(WL, WR, g, speeds, EL, ER, irL, irR, cL, cR, SL, SR);
+  signal_speeds<T, D>(WL, WR, g, speeds, EL, ER, irL, irR, q, cL, cR, SL, SR);
   const T mL = rL * (SL - unL), mR = rR * (SR - unR);
   const T Ss = (pR - pL + mL * unL - mR * unR) * trcp(mL - mR);
   // side selection: F_L if 0 <= S_L; F*_L if S_L < 0 <= S*; F*_R if S* < 0 < S_R; F_R if S_R <= 0
@@ -438,7 +543,7 @@ JF_HD void hllc(const T WL[5], const T WR[5], const Gas<T>& g, T F[5], int speed
     // S_L < u_L - c_L, S_L < 0 <= S*, and the mirror image)
     T fac, p_m;
     if constexpr (sizeof(T) == 8) {
-      const T d = S - Ss, x = T(1) / (m * d);
+      const T d = S - Ss, x = trcp(m * d);
       fac = m * m * x;
       p_m = p * d * x;
     } else {
@@ -461,10 +566,10 @@ JF_HD void hllc(const T WL[5], const T WR[5], const Gas<T>& g, T F[5], int speed
 // else (S_R F_L - S_L F_R + S_L S_R (U_R - U_L)) / (S_R - S_L).
 template <typename T, int D>
 JF_HD void hll(const T WL[5], const T WR[5], const Gas<T>& g, T F[5], int speeds = 0) {
-  T EL, ER, irL, irR, cL, cR;
-  side_states(WL, WR, g, EL, ER, irL, irR, cL, cR);
+  T EL, ER, irL, irR, q, cL, cR;
+  side_states(WL, WR, g, EL, ER, irL, irR, q, cL, cR);
   T SL, SR;
-  signal_speeds<T, D>(WL, WR, g, speeds, EL, ER, irL, irR, cL, cR, SL, SR);
+  signal_speeds<T, D>(WL, WR, g, speeds, EL, ER, irL, irR, q, cL, cR, SL, SR);
   T FL[5], FR[5], UL[5], UR[5];
   side_flux<T, D>(WL, EL, FL, UL);
   side_flux<T, D>(WR, ER, FR, UR);
@@ -485,8 +590,8 @@ JF_HD void hll(const T WL[5], const T WR[5], const Gas<T>& g, T F[5], int speeds
 // F = (F_L + F_R)/2 - a (U_R - U_L)/2.
 template <typename T, int D>
 JF_HD void rusanov(const T WL[5], const T WR[5], const Gas<T>& g, T F[5]) {
-  T EL, ER, irL, irR, cL, cR;
-  side_states(WL, WR, g, EL, ER, irL, irR, cL, cR);
+  T EL, ER, irL, irR, q, cL, cR;
+  side_states(WL, WR, g, EL, ER, irL, irR, q, cL, cR);
   const T a = tmax(fabs(WL[1 + D]) + cL, fabs(WR[1 + D]) + cR);
   T FL[5], FR[5], UL[5], UR[5];
   side_flux<T, D>(WL, EL, FL, UL);
@@ -605,8 +710,8 @@ JF_HD void nn_inputs(const T WL[5], const T WR[5], const Gas<T>& g, T cL, T cR, 
 // with alpha = exp(NN(x)).
 template <typename T, int D>
 JF_HD void rusanov_nn(const T WL[5], const T WR[5], const Gas<T>& g, T F[5]) {
-  T EL, ER, irL, irR, cL, cR;
-  side_states(WL, WR, g, EL, ER, irL, irR, cL, cR);
+  T EL, ER, irL, irR, q, cL, cR;
+  side_states(WL, WR, g, EL, ER, irL, irR, q, cL, cR);
   T x[4];
   nn_inputs<T, D>(WL, WR, g, cL, cR, x);
   const T a = nn_alpha(g.nn, x);
