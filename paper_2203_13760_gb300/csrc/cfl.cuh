@@ -17,8 +17,21 @@ struct CflChunk {
   long long begin, end;
 };
 
+// CTAs of a single-grid pass over N cells: one vector of cells per thread,
+// at most two CTAs per SM.  Their atomics on one address, not the loads, took
+// most of the pass on mid-size grids: with up to eight CTAs of 256 threads
+// per SM (and the CTA count set by cells, so that three quarters of them had
+// no vector) it took 18 us at 1024^2 FP32.
 template <typename T>
-__global__ void __launch_bounds__(256) cfl_kernel(const T* __restrict__ U0, CflArgs a0, ReduceScratch* sc0,
+inline unsigned cfl_blocks(long long N, int sms) {
+  constexpr int V = 16 / (int)sizeof(T);
+  const long long units = N % V == 0 ? N / V : N;
+  const long long b = (units + kCflThreads - 1) / kCflThreads, cap = 2LL * sms;
+  return (unsigned)(b < 1 ? 1 : (b > cap ? cap : b));
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kCflThreads) cfl_kernel(const T* __restrict__ U0, CflArgs a0, ReduceScratch* sc0,
                                                   double* dt0, double* dt0b, int* flag,
                                                   const SimDesc<T>* __restrict__ sims,
                                                   const CflChunk* __restrict__ chunks,
@@ -86,7 +99,7 @@ __global__ void __launch_bounds__(256) cfl_kernel(const T* __restrict__ U0, CflA
     for (long long q = q0; q < end; q += stride) cell_rates(U, q, a.N, a.nactive, gamma, gm1, kdiff, conv, diff, bad);
   }
   if (bad) atomicOr(flag, 1);
-  finish_cfl((double)conv, (double)diff, sc, nblocks, a.hmin, a.cfl, dto, dto2);
+  finish_cfl(conv, diff, sc, nblocks, a.hmin, a.cfl, dto, dto2);
 }
 
 }  // namespace jf

@@ -354,7 +354,7 @@ jf_status rhs_impl(jf_ctx* h, const void* U, void* dUdt, cudaStream_t s) {
 template <typename T>
 jf_status cfl_impl(jf_ctx* h, const void* U, double* dt_out, double* dt_out2, cudaStream_t s) {
   const CflArgs a = make_cfl(h->grid, h->gas, h->scheme);
-  cfl_kernel<T><<<reduce_blocks(a.N, h->sms), 256, 0, s>>>(static_cast<const T*>(U), a, h->red_cfl, dt_out, dt_out2,
+  cfl_kernel<T><<<cfl_blocks<T>(a.N, h->sms), kCflThreads, 0, s>>>(static_cast<const T*>(U), a, h->red_cfl, dt_out, dt_out2,
                                                             h->flag, nullptr, nullptr, nullptr, nullptr, nullptr);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(h, e, "cfl kernel launch");

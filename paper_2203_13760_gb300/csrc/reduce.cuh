@@ -6,7 +6,8 @@
 // shared memory) and folds its result into a global accumulator with one
 // atomic; the last CTA to finish (ticket counter) finalises the result and
 // resets the accumulator and counter for the next launch.  No CTA waits for
-// another.
+// another.  The CTAs' atomics meet on one address, so the CFL pass runs at
+// most two CTAs per SM (cfl_blocks).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -32,10 +33,19 @@ struct ReduceScratch {
   double sum;
 };
 
+// Maximum over a warp of values >= 0, whose bit patterns order like the
+// values: integer operations, which leave the FP64 pipe alone.
+__device__ __forceinline__ float warp_max(float v) {
+  return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+}
 __device__ __forceinline__ double warp_max(double v) {
+  long long m = __double_as_longlong(v);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long x = __shfl_xor_sync(0xffffffffu, m, o);
+    m = x > m ? x : m;
+  }
+  return __longlong_as_double(m);
 }
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -51,7 +61,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 template <typename T>
 __device__ __forceinline__ void cell_rates_of(T r, T ru, T rv, T rw, T E, int nactive, T gamma, T gm1, T kdiff,
                                               T& conv, T& diff, bool& bad) {
-  const T inv = T(1) / r;
+  T inv;
+  if constexpr (sizeof(T) == 8) inv = trcp(r); else inv = T(1) / r;
   const T u = ru * inv;
   const T v = rv * inv;
   const T w = rw * inv;
@@ -78,37 +89,50 @@ template <typename T> struct Vec16;
 template <> struct Vec16<float> { using type = float4; };
 template <> struct Vec16<double> { using type = double2; };
 
-// Block-wide FP64 maxima of (conv, diff) folded into sc; the CTA that takes
-// the last of `nblocks` tickets forms dt = CFL min(hmin / C, 3/14 hmin^2 / D)
-// and resets sc.  blockDim.x <= 256, a multiple of 32.
-__device__ __forceinline__ void finish_cfl(double conv, double diff, ReduceScratch* sc, unsigned int nblocks,
-                                           double hmin, double cfl, double* dt_out, double* dt_out2) {
-  __shared__ double s_conv[8], s_diff[8];
+// dt = CFL min(hmin / C, 3/14 hmin^2 / D)
+__device__ __forceinline__ void write_dt(double C, double Dm, double hmin, double cfl, double* dt_out,
+                                         double* dt_out2) {
+  double dt = hmin / C;
+  if (Dm > 0.0) dt = fmin(dt, (3.0 / 14.0) * hmin * hmin / Dm);
+  dt *= cfl;
+  *dt_out = dt;
+  if (dt_out2) *dt_out2 = dt;
+}
+
+// Block-wide maxima of (conv, diff), folded into sc; the CTA that takes the
+// last of `nblocks` tickets forms dt and resets sc.  A single CTA (small
+// grids) forms dt without the round trips of the accumulators.
+// blockDim.x <= kCflThreads, a multiple of 32.
+constexpr int kCflThreads = 512;
+template <typename T>
+__device__ __forceinline__ void finish_cfl(T conv, T diff, ReduceScratch* sc, unsigned int nblocks, double hmin,
+                                           double cfl, double* dt_out, double* dt_out2) {
+  __shared__ T s_conv[kCflThreads / 32], s_diff[kCflThreads / 32];
   conv = warp_max(conv);
   diff = warp_max(diff);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   if (lane == 0) { s_conv[wid] = conv; s_diff[wid] = diff; }
   __syncthreads();
   if (wid == 0) {
-    conv = lane < (int)(blockDim.x >> 5) ? s_conv[lane] : 0.0;
-    diff = lane < (int)(blockDim.x >> 5) ? s_diff[lane] : 0.0;
+    conv = lane < (int)(blockDim.x >> 5) ? s_conv[lane] : T(0);
+    diff = lane < (int)(blockDim.x >> 5) ? s_diff[lane] : T(0);
     conv = warp_max(conv);
     diff = warp_max(diff);
     if (lane == 0) {
+      if (nblocks == 1) {
+        write_dt((double)conv, (double)diff, hmin, cfl, dt_out, dt_out2);
+        return;
+      }
       // NaN never wins fmax; a NaN state is reported through the flag
-      atomicMax(&sc->acc[0], (unsigned long long)__double_as_longlong(conv));
-      atomicMax(&sc->acc[1], (unsigned long long)__double_as_longlong(diff));
+      atomicMax(&sc->acc[0], (unsigned long long)__double_as_longlong((double)conv));
+      if (diff > T(0)) atomicMax(&sc->acc[1], (unsigned long long)__double_as_longlong((double)diff));
       __threadfence();
       const unsigned int t = atomicAdd(&sc->ticket, 1u);
       if (t == nblocks - 1) {
         __threadfence();
         const double C = __longlong_as_double((long long)atomicMax(&sc->acc[0], 0ull));
         const double Dm = __longlong_as_double((long long)atomicMax(&sc->acc[1], 0ull));
-        double dt = hmin / C;
-        if (Dm > 0.0) dt = fmin(dt, (3.0 / 14.0) * hmin * hmin / Dm);
-        dt *= cfl;
-        *dt_out = dt;
-        if (dt_out2) *dt_out2 = dt;
+        write_dt(C, Dm, hmin, cfl, dt_out, dt_out2);
         sc->acc[0] = 0ull;
         sc->acc[1] = 0ull;
         sc->ticket = 0u;
