@@ -19,7 +19,7 @@
 
 namespace jf {
 
-constexpr long long kChunk = 8192;  // cells per CFL CTA (a whole number of vectors)
+constexpr long long kChunk = 16384;  // cells per CFL CTA (a whole number of vectors)
 
 // Euler steps of a batch: U = U1 for every simulation (blockIdx.y), the
 // pointers read from the device descriptors so that rebinding stays valid.

@@ -29,6 +29,13 @@ inline unsigned cfl_blocks(long long N, int sms) {
   const long long b = (units + kCflThreads - 1) / kCflThreads, cap = 2LL * sms;
   return (unsigned)(b < 1 ? 1 : (b > cap ? cap : b));
 }
+// Threads of its CTAs: whole warps with a vector each (one CTA for tiny grids).
+template <typename T>
+inline unsigned cfl_threads(long long N) {
+  constexpr int V = 16 / (int)sizeof(T);
+  const long long units = N % V == 0 ? N / V : N;
+  return units >= kCflThreads ? kCflThreads : (unsigned)((units + 31) / 32 * 32);
+}
 
 template <typename T>
 __global__ void __launch_bounds__(kCflThreads) cfl_kernel(const T* __restrict__ U0, CflArgs a0, ReduceScratch* sc0,

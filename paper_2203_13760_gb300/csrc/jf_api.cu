@@ -251,15 +251,36 @@ bool rows_preferred(const jf_grid* grids, int n, int rows_bx, int rows_ctas_per_
   return rows <= 1.08 * tiles && row_tiles >= 12.0 * sms * (rows_ctas_per_sm > 0 ? rows_ctas_per_sm : 1);
 }
 
+// 2D FP64 grids: the FP64 pipe is shared by an SM's warps, so a launch takes
+// the busiest SM's tiles times the warp tasks of a tile (2 BY + 3
+// reconstructions and 2 BY + 2 faces).  The tile shape with the fewest: small
+// grids are spread over the SMs with 32 x 3 or 32 x 4 tiles, large ones take
+// 32 x 8.  Measured, walled WENO3 stage: 128^2 31.0 us with 32 x 4 (rule: 21
+// tasks), 46.9 with 32 x 8 (37); 256^2 99.1 (84) and 93.0 (74).
+template <typename T>
+int f64_tile(const jf_ctx* h, const std::vector<std::pair<int, int>>& list) {
+  int count = 0, best = 0;
+  const StageVariant<T>* tab = stage_variants<T>(&count);
+  long long least = -1;
+  for (int i = 0; i < (int)list.size(); ++i) {
+    const StageVariant<T>& t = tab[list[i].first];
+    if (t.ymarch) continue;
+    const long long tiles = (long long)((h->grid.nx + t.bx - 1) / t.bx) * ((h->grid.ny + t.by - 1) / t.by);
+    const long long cost = ((tiles + h->sms - 1) / h->sms) * (4 * t.by + 5);
+    if (least < 0 || cost < least) { least = cost; best = i; }
+  }
+  return best;
+}
+
 template <typename T>
 jf_status select_variant(jf_ctx* h, int v, bool prepare) {
   const bool visc = dissipative(h->gas, h->scheme);
   auto list = variant_list<T>(h->dim, visc, scheme_kind(h));
   if (list.empty()) { set_error(h, "no compiled kernel variant for this configuration"); return JF_ERR_UNSUPPORTED; }
   if (v < 0) {  // the first variant, or the first row-tile one (automatic chunk) where rows_preferred says so
-    v = 0;
     int count = 0;
     const StageVariant<T>* tab = stage_variants<T>(&count);
+    v = sizeof(T) == 8 && h->dim == 2 ? f64_tile<T>(h, list) : 0;
     for (int i = 0; i < (int)list.size(); ++i)
       if (tab[list[i].first].ymarch && list[i].second == 0) {
         const StageVariant<T>& r = tab[list[i].first];
@@ -354,8 +375,8 @@ jf_status rhs_impl(jf_ctx* h, const void* U, void* dUdt, cudaStream_t s) {
 template <typename T>
 jf_status cfl_impl(jf_ctx* h, const void* U, double* dt_out, double* dt_out2, cudaStream_t s) {
   const CflArgs a = make_cfl(h->grid, h->gas, h->scheme);
-  cfl_kernel<T><<<cfl_blocks<T>(a.N, h->sms), kCflThreads, 0, s>>>(static_cast<const T*>(U), a, h->red_cfl, dt_out, dt_out2,
-                                                            h->flag, nullptr, nullptr, nullptr, nullptr, nullptr);
+  cfl_kernel<T><<<cfl_blocks<T>(a.N, h->sms), cfl_threads<T>(a.N), 0, s>>>(
+      static_cast<const T*>(U), a, h->red_cfl, dt_out, dt_out2, h->flag, nullptr, nullptr, nullptr, nullptr, nullptr);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(h, e, "cfl kernel launch");
   return JF_OK;

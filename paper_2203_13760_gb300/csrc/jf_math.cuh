@@ -410,6 +410,36 @@ JF_HD T weno3(T vm1, T v0, T vp1, T eps) {
   const T a0 = T(1.0 / 3.0) * trcp(t0 * t0), a1 = T(2.0 / 3.0) * trcp(t1 * t1);
   return (a0 * q0 + a1 * q1) * trcp(a0 + a1);
 }
+// Both WENO3-JS face values of one cell from v[j-1..j+1] (as weno5_cell):
+// with e0 = v0 - v[-1], e1 = v[1] - v0 and r_k = 1 / (eps + e_k^2)^2,
+//   right = v0 + (r0 e0 + 2 r1 e1) / (2 (r0 + 2 r1)),
+//   left  = v0 - (r1 e1 + 2 r0 e0) / (2 (r1 + 2 r0)).
+// FP64: r0, r1 scaled by (eps + e0^2)^2 (eps + e1^2)^2, and one reciprocal
+// for both values.
+template <typename T>
+JF_HD void weno3_cell(T vm1, T v0, T vp1, T eps, T& right, T& left) {
+  const T e0 = v0 - vm1, e1 = vp1 - v0;
+  const T t0 = eps + e0 * e0, t1 = eps + e1 * e1;
+  T r0, r1;
+  if constexpr (sizeof(T) == 8) {
+    r0 = t1 * t1;
+    r1 = t0 * t0;
+  } else {
+    r0 = trcp(t0 * t0);
+    r1 = trcp(t1 * t1);
+  }
+  const T Sr = r0 + T(2) * r1, Sl = r1 + T(2) * r0;
+  const T p0 = r0 * e0, p1 = r1 * e1;
+  const T nr = p0 + T(2) * p1, nl = p1 + T(2) * p0;
+  if constexpr (sizeof(T) == 8) {
+    const T inv = trcp(T(2) * Sr * Sl);
+    right = v0 + nr * (Sl * inv);
+    left = v0 - nl * (Sr * inv);
+  } else {
+    right = v0 + nr * trcp(T(2) * Sr);
+    left = v0 - nl * trcp(T(2) * Sl);
+  }
+}
 __device__ __forceinline__ float2 weno3_pair(float2 vm1, float2 v0, float2 vp1, float eps) {
   return make_float2(weno3(vm1.x, v0.x, vp1.x, eps), weno3(vm1.y, v0.y, vp1.y, eps));
 }

@@ -146,7 +146,7 @@ struct Geo {
   static constexpr int NFX = (BX + 1) * BY;          // x faces per plane
   static constexpr int NFY = plane_dims(DIM) == 2 ? BX * (BY + 1) : 0;
   static constexpr int NCELL = BX * BY;              // cell threads
-  static constexpr int NT = plane_dims(DIM) == 2 ? BX * (BY + 1) : BX + 32;  // threads
+  static constexpr int NT = plane_dims(DIM) == 2 ? BX * (BY + 1) : (BX <= 30 ? 160 : BX + 32);  // threads
   static_assert(plane_dims(DIM) == 1 || BX == 32, "2D/3D tiles are one warp wide");
   static_assert(plane_dims(DIM) == 2 || BY == 1, "row tiles are one row");
 };
@@ -325,8 +325,8 @@ constexpr bool sch_roe(int s) { return s == SCH_ROE || s == SCH_ROE_EXT; }
 constexpr bool sch_ext(int s) { return s == SCH_GENERAL_EXT || s == SCH_ROE_EXT || s == SCH_NN; }
 // Families whose kernels reconstruct once per cell and direction (the face
 // values of a plane in shared memory): the default scheme and the run-time
-// Godunov schemes with WENO5-JS / WENO5-Z.
-constexpr bool sch_pc(int s) { return s == SCH_DEFAULT || s == SCH_GENERAL; }
+// Godunov schemes.
+constexpr bool sch_pc(int s) { return s == SCH_DEFAULT || sch_general(s); }
 
 // Flux-splitting face flux of the ROE setup (Section 3.3, Flux-Splitting
 // approach; Section 5): Roe average of the two cells beside the face, the
@@ -453,30 +453,63 @@ __device__ __forceinline__ void face_riemann(const RingView<T, BX, BY, DIM, VISC
 }
 
 // Cell-centre C4 tangential derivative sums of the z faces of one column
-// (FP32, z-marching kernels): h[t][j] for tangent t (0: x, 1: y) at the
+// (z-marching kernels): h[t][j] for tangent t (0: x, 1: y) at the
 // planes k, k + 1, k + 2 of the face k + 1/2 (j = 0, 1, 2), the packed pair
 // (w, u_t) as in face_visc_add.  The face k + 3/2 reuses them and computes
 // only plane k + 3.
+// FP64: h[t][j][0] for w and h[t][j][1] for u_t.
+template <typename T>
 struct ZTangents {
   float2 h[2][3];
 };
+template <>
+struct ZTangents<double> {
+  double h[2][3][2];
+};
+
+// FP64 x and y faces of a marching tile: the interpolation along the normal,
+// 9 (v0 + v1) - (v_-1 + v2), of u_D (s = 0) and u_z (s = 1) in the planes
+// k - 2 .. k + 1 of the face at plane k (j = 0 .. 3).  The tangential stencil
+// along the march is the product of that interpolation and the C4 derivative
+// in either order; taken first, the interpolation is one plane per face
+// instead of four derivatives.
+template <typename T>
+struct FaceCarry {
+  T f[2][4];
+};
+template <typename T, int D, typename Ring>
+__device__ __forceinline__ T normal_interp(const Ring& R, int x0, int y0, int c, int e) {
+  auto val = [&](int n) { return D == 0 ? R.at(c, x0 + n, y0, e) : R.at(c, x0, y0 + n, e); };
+  return fma(T(9), val(0) + val(1), -(val(-1) + val(2)));
+}
+// The planes `first` .. `first` + 3 of the ring view.
+template <typename T, int D, typename Ring>
+__device__ __forceinline__ void face_carry_init(const Ring& R, int x0, int y0, int first, FaceCarry<T>& fc) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    fc.f[0][j] = normal_interp<T, D>(R, x0, y0, 1 + D, first + j);
+    fc.f[1][j] = normal_interp<T, D>(R, x0, y0, 3, first + j);
+  }
+}
 
 // Dissipative part of the net flux (Sections 2 and 3.4) through the face
 // between the cell at shared-memory position (x0, y0, plane 0) and its
 // neighbour along D, added to NF.
-// ZC (FP32, D == 2 only): 0 computes every tangential stencil; 1 computes
-// them and keeps those of planes 0..2 in *zc; 2 takes planes -1..1 from *zc,
-// computes plane 2 and shifts *zc to planes 0..2.
+// ZC, D == 2: 0 computes every tangential stencil; 1 computes them and keeps
+// those of planes 0..2 in *zc; 2 takes planes -1..1 from *zc, computes plane 2
+// and shifts *zc to planes 0..2.  D < 2 (FP64): 2 takes the tangential
+// stencils along the march from *fc, computes plane 2 and shifts *fc.
 template <typename T, int D, int BX, int BY, int DIM, bool VISC, int ZC = 0>
 __device__ __forceinline__ void face_visc_add(const RingView<T, BX, BY, DIM, VISC>& R, int x0, int y0,
                                               const Gas<T>& g, const T inv_h[3], T NF[5],
-                                              ZTangents* zc = nullptr) {
-  static_assert(ZC == 0 || (D == 2 && sizeof(T) == 4), "carried tangential stencils: FP32 z faces only");
+                                              ZTangents<T>* zc = nullptr, FaceCarry<T>* fc = nullptr) {
+  static_assert(ZC == 0 || D == 2 || (ZC == 2 && sizeof(T) == 8), "carried stencils of x and y faces: FP64 only");
   using Ro = Roles<D>;
+  const auto& ring = R;
   auto val = [&](int c, int n, int t1, int t2) -> T {
     int x, y, e;
     Ro::map(n, t1, t2, x, y, e);
-    return R.at(c, x0 + x, y0 + y, e);
+    return ring.at(c, x0 + x, y0 + y, e);
   };
   // Dissipative flux (Sections 2 and 3.4).  G[a][b] = du_a/dx_b at the face.
   T G[3][3];
@@ -547,43 +580,63 @@ __device__ __forceinline__ void face_visc_add(const RingView<T, BX, BY, DIM, VIS
     if constexpr (axis_on(DIM, Ro::T1)) tang(std::integral_constant<int, 1>{});
     if constexpr (axis_on(DIM, Ro::T2)) tang(std::integral_constant<int, 2>{});
   } else {
+    // FP64: the weights of each stencil grouped by equal factors, and their
+    // products with 1/h formed once per face, so that a normal derivative or
+    // face value takes 4 operations, a cell-centre tangential derivative 3
+    // and its interpolation 4 (5, 5, 5 and 6 term by term)
+    const T kd0 = T(27.0 / 24.0) * hn, kd1 = T(1.0 / 24.0) * hn;
+    auto df = [&](int c) {
+      return fma(kd0, val(c, 1, 0, 0) - val(c, 0, 0, 0), kd1 * (val(c, -1, 0, 0) - val(c, 2, 0, 0)));
+    };
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
-    G[a][D] = df4(val(1 + a, -1, 0, 0), val(1 + a, 0, 0, 0), val(1 + a, 1, 0, 0), val(1 + a, 2, 0, 0)) * hn;
-  dTdn = df4(val(5, -1, 0, 0), val(5, 0, 0, 0), val(5, 1, 0, 0), val(5, 2, 0, 0)) * hn;
-  // tangential derivatives: cell-centre C4 at cells -1..2 along the normal,
-  // then fourth-order interpolation to the face
-  if (axis_on(DIM, Ro::T1)) {
-    constexpr int e = Ro::T1;
-    const T he = inv_h[e];
+    for (int a = 0; a < 3; ++a) G[a][D] = df(1 + a);
+    dTdn = df(5);
+    constexpr bool carried = ZC == 2 && D < 2;  // tangent T2 (the march) from *fc
+    // tangential derivatives along e of (u_D, u_e): cell-centre C4 at cells
+    // -1..2 along the normal, then fourth-order interpolation to the face
+    auto tang = [&](auto role) {
+      constexpr int R = decltype(role)::value;  // 1: tangent T1, 2: tangent T2
+      constexpr int e = R == 1 ? Ro::T1 : Ro::T2;
+      const T he = inv_h[e], k0 = T(9.0 / 192.0) * he, k1 = T(-1.0 / 192.0) * he;
 #pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const int a = s == 0 ? D : e;
-      T cen[4];
+      for (int s = 0; s < 2; ++s) {
+        const int a = s == 0 ? D : e, c = 1 + a;
+        if constexpr (carried && R == 2) {
+          T* f = fc->f[s];
+          const T f4 = normal_interp<T, D>(ring, x0, y0, c, 2);
+          G[a][e] = fma(T(8), f[3] - f[1], f[0] - f4) * (T(1.0 / 192.0) * he);
+          uf[a] = T(1.0 / 16.0) * f[2];
+          f[0] = f[1];
+          f[1] = f[2];
+          f[2] = f[3];
+          f[3] = f4;
+        } else {
+          T h[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        cen[q] = dc4(val(1 + a, q - 1, -2, 0), val(1 + a, q - 1, -1, 0), val(1 + a, q - 1, 1, 0),
-                     val(1 + a, q - 1, 2, 0));
-      G[a][e] = rc4(cen[0], cen[1], cen[2], cen[3]) * he;
+          for (int q = 0; q < 4; ++q) {
+            if (ZC == 2 && D == 2 && q < 3) {
+              h[q] = zc->h[R - 1][q][s];
+              continue;
+            }
+            auto at = [&](int j) { return R == 1 ? val(c, q - 1, j, 0) : val(c, q - 1, 0, j); };
+            h[q] = fma(T(8), at(1) - at(-1), at(-2) - at(2));
+          }
+          if constexpr (ZC != 0 && D == 2) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) zc->h[R - 1][q][s] = h[q + 1];
+          }
+          G[a][e] = fma(k0, h[1] + h[2], k1 * (h[0] + h[3]));
+        }
+      }
+    };
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      if (carried && (a == D || a == Ro::T2)) continue;  // with the carried stencil
+      uf[a] = fma(T(9.0 / 16.0), val(1 + a, 0, 0, 0) + val(1 + a, 1, 0, 0),
+                  T(-1.0 / 16.0) * (val(1 + a, -1, 0, 0) + val(1 + a, 2, 0, 0)));
     }
-  }
-  if (axis_on(DIM, Ro::T2)) {
-    constexpr int e = Ro::T2;
-    const T he = inv_h[e];
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-      const int a = s == 0 ? D : e;
-      T cen[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        cen[q] = dc4(val(1 + a, q - 1, 0, -2), val(1 + a, q - 1, 0, -1), val(1 + a, q - 1, 0, 1),
-                     val(1 + a, q - 1, 0, 2));
-      G[a][e] = rc4(cen[0], cen[1], cen[2], cen[3]) * he;
-    }
-  }
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-    uf[a] = rc4(val(1 + a, -1, 0, 0), val(1 + a, 0, 0, 0), val(1 + a, 1, 0, 0), val(1 + a, 2, 0, 0));
+    if constexpr (axis_on(DIM, Ro::T1)) tang(std::integral_constant<int, 1>{});
+    if constexpr (axis_on(DIM, Ro::T2)) tang(std::integral_constant<int, 2>{});
   }
   const T div = G[0][0] + G[1][1] + G[2][2];
   T tau[3];
@@ -658,14 +711,15 @@ __device__ __forceinline__ void face_flux(const RingView<T, BX, BY, DIM, VISC>& 
   if constexpr (VISC) face_visc_add<T, D, BX, BY, DIM, VISC>(R, x0, y0, g, inv_h, NF);
 }
 
-// WENO5 face values of one cell along D (per-cell families, weno5_cell; z:
-// the WENO5-Z weights): the cell sits `shift` cells along D from ring
+// Face values of one cell along D (per-cell families, weno5_cell; z = 1: the
+// WENO5-Z weights; z = 2, W3 kernels only: WENO3-JS): the cell sits `shift`
+// cells along D from ring
 // position (x0, y0, plane 0);
 // right[c] = v^-_{+1/2}, its value at the face to its right (the left state
 // of that face), left[c] = v^+_{-1/2} (the right state of the face to its
 // left).  FP32: (rho, p) and (u, v) in packed lanes, w alone (or, NOW, not
 // at all: the caller pairs it with another cell's w).
-template <typename T, int D, int BX, int BY, int DIM, bool VISC, bool NOW = false>
+template <typename T, int D, int BX, int BY, int DIM, bool VISC, bool W3, bool NOW = false>
 __device__ __forceinline__ void cell_recon(const RingView<T, BX, BY, DIM, VISC>& R, int x0, int y0, int shift, T eps,
                                            T right[5], T left[5], int z = 0) {
   using Ro = Roles<D>;
@@ -674,6 +728,12 @@ __device__ __forceinline__ void cell_recon(const RingView<T, BX, BY, DIM, VISC>&
     Ro::map(n + shift, 0, 0, x, y, e);
     return R.at(c, x0 + x, y0 + y, e);
   };
+  if (W3 && z == 2) {
+#pragma unroll
+    for (int c = 0; c < 5; ++c)
+      if (!(NOW && c == 3)) weno3_cell<T>(val(c, -1), val(c, 0), val(c, 1), eps, right[c], left[c]);
+    return;
+  }
   if constexpr (sizeof(T) == 4) {
     // row tiles: the lean form (5 % less time per stage: 1024^2 62.5 -> 59.1 us,
     // 64 uneven grids 261 -> 248 us); the tiles keep their rounding (weno5_cell)
@@ -700,6 +760,14 @@ __device__ __forceinline__ void cell_recon(const RingView<T, BX, BY, DIM, VISC>&
   }
 }
 
+// The same for one component of a cell of a 1D tile.
+template <typename T, bool W3, typename Ring>
+__device__ __forceinline__ void component_recon(const Ring& R, int x, int c, T eps, T& right, T& left, int z) {
+  auto val = [&](int n) { return R.at(c, x + n, 0, 0); };
+  if (W3 && z == 2) weno3_cell<T>(val(-1), val(0), val(1), eps, right, left);
+  else weno5_cell<T>(val(-2), val(-1), val(0), val(1), val(2), eps, right, left, z);
+}
+
 // The stage kernel.  blockDim.x == Geo::NT.
 // grid = (ceil(nx/BX), ceil(ny/BY), ceil(nz/zchunk)) (3D), (.., .., 1) otherwise.
 // One tile (tile column (bx, by), z chunk bz) of one grid: the whole stage
@@ -718,9 +786,12 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
   const int gx0 = bx * BX;
   const int gy0 = by * BY;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const bool cell_thread = threadIdx.x < G::NCELL;
-  const int tx = threadIdx.x % BX;
-  const int ty = threadIdx.x / BX;
+  // 1D tiles of at most 30 cells (FP64): five warps, of which warp c takes
+  // component c of the reconstruction and of the update, lane by lane
+  constexpr bool SPLIT = DIM == 1 && BX <= 30;
+  const bool cell_thread = SPLIT ? lane < BX : threadIdx.x < G::NCELL;
+  const int tx = SPLIT ? lane : threadIdx.x % BX;
+  const int ty = SPLIT ? 0 : threadIdx.x / BX;
   const int gx = gx0 + tx, gy = gy0 + ty;
   const bool own = cell_thread && gx < A.nx && gy < A.ny;
   const T dt = A.rhs_only ? T(0) : T(*A.dt);
@@ -762,24 +833,33 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
   // face values of a plane kept in shared memory (x, y; along z only the
   // current cell's value at its upper face, zl, is kept, by its column)
   constexpr bool PC = sch_pc(SCH);
-  const int wz = SCH == SCH_DEFAULT ? 0 : g.recon;  // per-cell WENO5: 0 JS, 1 Z
+  constexpr bool W3 = sch_ext(SCH);
+  const int wz = SCH == SCH_DEFAULT ? 0 : g.recon;  // 0 WENO5-JS, 1 WENO5-Z, 2 WENO3-JS (W3)
   constexpr int SX = BY * (BX + 2), SY = plane_dims(DIM) == 2 ? (BY + 2) * BX : 0;
   T* EX = Fy + 5 * G::NFY;  // [2][5][BY][BX+2] (PC only)
   T* EY = EX + 2 * 5 * SX;  // [2][5][BY+2][BX] (PC, tiles spanning y)
-  // per-cell families, 3D: the net fluxes of a column's z faces in shared
+  // per-cell families, 3D, FP32: the net fluxes of a column's z faces in shared
   // memory, [2][5][NCELL] (face k + 1/2 in slot k & 1), written and read by
   // the column's own thread, so that they hold no registers across the phases
-  constexpr bool ZS = PC && marches(DIM);
+  // (FP64 runs one CTA of at most eight warps per SM: registers are free and
+  // shared memory is short)
+  constexpr bool ZS = PC && marches(DIM) && sizeof(T) == 4;
   T* ZF = EY + 2 * 5 * SY;
   auto zf = [&](int k, int c) -> T& { return ZF[((k & 1) * 5 + c) * G::NCELL + threadIdx.x]; };
   // and the WENO5 value of the column's cell k at k + 1/2 (the left state of
   // the next z face), [5][NCELL]
-  auto zl = [&](int c) -> T& { return ZF[(10 + c) * G::NCELL + threadIdx.x]; };
-  T NFz_lo[5] = {T(0), T(0), T(0), T(0), T(0)};  // other schemes: the lower z face's net flux
-  ZTangents ztan;  // FP32 z faces: the tangential stencils of the planes k .. k + 2
+  T zl_r[5];
+  auto zl = [&](int c) -> T& {
+    if constexpr (ZS) return ZF[(10 + c) * G::NCELL + threadIdx.x];
+    else return zl_r[c];
+  };
+  T NFz_lo[5] = {T(0), T(0), T(0), T(0), T(0)};  // without ZS: the lower z face's net flux
+  ZTangents<T> ztan;  // z faces: the tangential stencils of the planes k .. k + 2
+  constexpr bool FC = PC && VISC && marches(DIM) && sizeof(T) == 8;
+  FaceCarry<T> xcar, ycar;  // FC: this thread's x and y face
   PlaneRegs<T, BX, BY, DIM, VISC> next;  // plane k + 4, in flight while plane k is computed
   PlaneMap<T, BX, BY, DIM, VISC> pmap;    // per-cell families (no walls): the in-plane offsets of its cells
-  if constexpr (PC && marches(DIM)) plane_map<T, BX, BY, DIM, VISC>(A, pmap, gx0, gy0);
+  if constexpr (PC && !WALLS && marches(DIM)) plane_map<T, BX, BY, DIM, VISC>(A, pmap, gx0, gy0);
   if (marches(DIM)) {
 #pragma unroll 1
     for (int q = 0; q < 6; ++q) load_plane<T, BX, BY, DIM, VISC, WALLS>(A, g, ring + q * G::PLANE, gx0, gy0, z0 - 3 + q);
@@ -791,23 +871,27 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
       if constexpr (PC) {
         // face z0 - 1/2 from the values of cells z0 - 1 and z0; zl: cell z0 at z0 + 1/2
         T r[5], l[5], rz[5], lz[5];
-        cell_recon<T, 2, BX, BY, DIM, VISC>(R, HALO + tx, G::HY + ty, 0, g.eps, r, l, wz);
-        cell_recon<T, 2, BX, BY, DIM, VISC>(R, HALO + tx, G::HY + ty, 1, g.eps, rz, lz, wz);
+        cell_recon<T, 2, BX, BY, DIM, VISC, W3>(R, HALO + tx, G::HY + ty, 0, g.eps, r, l, wz);
+        cell_recon<T, 2, BX, BY, DIM, VISC, W3>(R, HALO + tx, G::HY + ty, 1, g.eps, rz, lz, wz);
 #pragma unroll
         for (int c = 0; c < 5; ++c) zl(c) = rz[c];
         T F[5], NF[5];
         face_riemann<T, 2, BX, BY, DIM, VISC, SCH>(R, HALO + tx, G::HY + ty, g, r, lz, F);
 #pragma unroll
         for (int c = 0; c < 5; ++c) NF[c] = -F[c];
-        if constexpr (VISC && sizeof(T) == 4)
-          face_visc_add<T, 2, BX, BY, DIM, VISC, 1>(R, HALO + tx, G::HY + ty, g, inv_h, NF, &ztan);
-        else if constexpr (VISC)
-          face_visc_add<T, 2, BX, BY, DIM, VISC>(R, HALO + tx, G::HY + ty, g, inv_h, NF);
+        if constexpr (VISC) face_visc_add<T, 2, BX, BY, DIM, VISC, 1>(R, HALO + tx, G::HY + ty, g, inv_h, NF, &ztan);
 #pragma unroll
-        for (int c = 0; c < 5; ++c) zf(z0 - 1, c) = NF[c];
+        for (int c = 0; c < 5; ++c) {
+          if constexpr (ZS) zf(z0 - 1, c) = NF[c];
+          else NFz_lo[c] = NF[c];
+        }
       } else {
         face_flux<T, 2, BX, BY, DIM, VISC, SCH>(R, HALO + tx, G::HY + ty, g, inv_h, NFz_lo);
       }
+    }
+    if constexpr (FC) {  // planes z0 - 2 .. z0 + 1
+      if (xf_x >= 0) face_carry_init<T, 0>(R, HALO + xf_x - 1, G::HY + xf_y, -1, xcar);
+      if constexpr (plane_dims(DIM) == 2) face_carry_init<T, 1>(R, HALO + yf_x, G::HY + yf_y - 1, -1, ycar);
     }
     __syncthreads();  // slot 0 (plane z0 - 3) is overwritten next
     load_plane<T, BX, BY, DIM, VISC, WALLS>(A, g, ring, gx0, gy0, z0 + 3);
@@ -831,6 +915,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
       if (own && !A.rhs_only) {
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
+          if (SPLIT && c != warp) continue;
           const bool ok = JF_CHECK(qc >= 0 && qc < A.N, "JFDBG cell qc=%lld N=%lld\n", qc, A.N);
           us[c] = ok ? __ldg(A.Us + qc + gcomp(DIM, c) * A.N) : T(1);
           un[c] = A.Un && ok ? A.Un[qc + gcomp(DIM, c) * A.N] : T(0);
@@ -846,7 +931,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
       // -1 .. BX) and y (rows -1 .. BY), and the z face of each column
       auto put_x = [&](int row, int j) {
         T r[5], l[5];
-        cell_recon<T, 0, BX, BY, DIM, VISC>(R, HALO + j, G::HY + row, 0, g.eps, r, l, wz);
+        cell_recon<T, 0, BX, BY, DIM, VISC, W3>(R, HALO + j, G::HY + row, 0, g.eps, r, l, wz);
         const int i = row * (BX + 2) + j + 1;
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
@@ -858,7 +943,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
       };
       auto put_y = [&](int row, int x) {
         T r[5], l[5];
-        cell_recon<T, 1, BX, BY, DIM, VISC>(R, HALO + x, G::HY + row, 0, g.eps, r, l, wz);
+        cell_recon<T, 1, BX, BY, DIM, VISC, W3>(R, HALO + x, G::HY + row, 0, g.eps, r, l, wz);
         const int i = (row + 1) * BX + x;
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
@@ -868,7 +953,14 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
           }
         }
       };
-      if (plane_dims(DIM) == 1) {
+      if constexpr (SPLIT) {
+        if (lane < BX + 2) {
+          T r, l;
+          component_recon<T, W3>(R, HALO + lane - 1, warp, g.eps, r, l, wz);
+          EX[warp * SX + lane] = r;
+          EX[(5 + warp) * SX + lane] = l;
+        }
+      } else if (plane_dims(DIM) == 1) {
         if (threadIdx.x < BX + 2) put_x(0, (int)threadIdx.x - 1);
       } else if constexpr (sizeof(T) == 4) {
         // the same cells as below; the w components of a thread's x cell and
@@ -879,7 +971,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
         const int xcol = warp < BY ? lane - 1 : (hx ? BX - 1 + (lane & 1) : 0);
         const int yrow0 = warp < BY ? warp - 1 : BY - 1;
         T r[5], l[5];
-        cell_recon<T, 0, BX, BY, DIM, VISC, true>(R, HALO + xcol, G::HY + xrow, 0, g.eps, r, l, wz);
+        cell_recon<T, 0, BX, BY, DIM, VISC, W3, true>(R, HALO + xcol, G::HY + xrow, 0, g.eps, r, l, wz);
         const int ix = xrow * (BX + 2) + xcol + 1;
         if (hx) {
 #pragma unroll
@@ -891,7 +983,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
             }
           }
         }
-        cell_recon<T, 1, BX, BY, DIM, VISC, true>(R, HALO + lane, G::HY + yrow0, 0, g.eps, r, l, wz);
+        cell_recon<T, 1, BX, BY, DIM, VISC, W3, true>(R, HALO + lane, G::HY + yrow0, 0, g.eps, r, l, wz);
         const int iy = (yrow0 + 1) * BX + lane;
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
@@ -906,7 +998,12 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
         for (int n = 0; n < 5; ++n)
           wv[n] = make_float2(R.at(3, HALO + xcol + n - 2, G::HY + xrow, 0), R.at(3, HALO + lane, G::HY + yrow0 + n - 2, 0));
         float2 wr, wl;
-        weno5_cell_pair(wv[0], wv[1], wv[2], wv[3], wv[4], g.eps, wr, wl, wz);
+        if (W3 && wz == 2) {
+          weno3_cell(wv[1].x, wv[2].x, wv[3].x, g.eps, wr.x, wl.x);
+          weno3_cell(wv[1].y, wv[2].y, wv[3].y, g.eps, wr.y, wl.y);
+        } else {
+          weno5_cell_pair(wv[0], wv[1], wv[2], wv[3], wv[4], g.eps, wr, wl, wz);
+        }
         if (hx && JF_CHECK(ix >= 0 && ix < SX, "JFDBG EX i=%d\n", ix)) {
           EX[3 * SX + ix] = wr.x;
           EX[8 * SX + ix] = wl.x;
@@ -931,7 +1028,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
       if (marches(DIM) && cell_thread) {
         // face k + 1/2: the stored value of cell k (zl) and the lower value of cell k + 1
         T r[5], l[5], F[5], NF[5], zl0[5];
-        cell_recon<T, 2, BX, BY, DIM, VISC>(R, HALO + tx, G::HY + ty, 1, g.eps, r, l, wz);
+        cell_recon<T, 2, BX, BY, DIM, VISC, W3>(R, HALO + tx, G::HY + ty, 1, g.eps, r, l, wz);
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
           zl0[c] = zl(c);
@@ -940,18 +1037,21 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
         face_riemann<T, 2, BX, BY, DIM, VISC, SCH>(R, HALO + tx, G::HY + ty, g, zl0, l, F);
 #pragma unroll
         for (int c = 0; c < 5; ++c) NF[c] = -F[c];
-        if constexpr (VISC && sizeof(T) == 4)
-          face_visc_add<T, 2, BX, BY, DIM, VISC, 2>(R, HALO + tx, G::HY + ty, g, inv_h, NF, &ztan);
-        else if constexpr (VISC)
-          face_visc_add<T, 2, BX, BY, DIM, VISC>(R, HALO + tx, G::HY + ty, g, inv_h, NF);
+        if constexpr (VISC) face_visc_add<T, 2, BX, BY, DIM, VISC, 2>(R, HALO + tx, G::HY + ty, g, inv_h, NF, &ztan);
 #pragma unroll
-        for (int c = 0; c < 5; ++c) zf(k, c) = NF[c];
+        for (int c = 0; c < 5; ++c) {
+          if constexpr (ZS) zf(k, c) = NF[c];
+          else NFz_hi[c] = NF[c];
+        }
       }
       __syncthreads();
       // plane k + 4 in flight during the faces and the update (committed at
       // the end of this plane); its registers are free during the
       // reconstruction phase
-      if (marches(DIM) && k + 1 < z1) fetch_plane_mapped<T, BX, BY, DIM, VISC>(A, next, pmap, k + 4);
+      if (marches(DIM) && k + 1 < z1) {
+        if constexpr (WALLS) fetch_plane<T, BX, BY, DIM, VISC, true>(A, next, gx0, gy0, k + 4);
+        else fetch_plane_mapped<T, BX, BY, DIM, VISC>(A, next, pmap, k + 4);
+      }
       // phase 2: the x and y faces from the stored values
       if (xf_x >= 0) {
         T Wm[5], Wp[5], F[5], NF[5];
@@ -964,7 +1064,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
         face_riemann<T, 0, BX, BY, DIM, VISC, SCH>(R, HALO + xf_x - 1, G::HY + xf_y, g, Wm, Wp, F);
 #pragma unroll
         for (int c = 0; c < 5; ++c) NF[c] = -F[c];
-        if constexpr (VISC) face_visc_add<T, 0, BX, BY, DIM, VISC>(R, HALO + xf_x - 1, G::HY + xf_y, g, inv_h, NF);
+        if constexpr (VISC)
+          face_visc_add<T, 0, BX, BY, DIM, VISC, FC ? 2 : 0>(R, HALO + xf_x - 1, G::HY + xf_y, g, inv_h, NF, nullptr, &xcar);
         const int t = xf_y * (BX + 1) + xf_x;
 #pragma unroll
         for (int c = 0; c < 5; ++c)
@@ -982,7 +1083,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
         face_riemann<T, 1, BX, BY, DIM, VISC, SCH>(R, HALO + yf_x, G::HY + yf_y - 1, g, Wm, Wp, F);
 #pragma unroll
         for (int c = 0; c < 5; ++c) NF[c] = -F[c];
-        if constexpr (VISC) face_visc_add<T, 1, BX, BY, DIM, VISC>(R, HALO + yf_x, G::HY + yf_y - 1, g, inv_h, NF);
+        if constexpr (VISC)
+          face_visc_add<T, 1, BX, BY, DIM, VISC, FC ? 2 : 0>(R, HALO + yf_x, G::HY + yf_y - 1, g, inv_h, NF, nullptr, &ycar);
         const int t = yf_y * BX + yf_x;
 #pragma unroll
         for (int c = 0; c < 5; ++c)
@@ -1048,6 +1150,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
     } else if (own) {
 #pragma unroll
       for (int c = 0; c < 5; ++c) {
+        if (SPLIT && c != warp) continue;
         const int fx = ty * (BX + 1) + tx;
         T rhs = (Fx[c * G::NFX + fx + 1] - Fx[c * G::NFX + fx]) * inv_h[0];
         if (plane_dims(DIM) == 2) {
@@ -1160,10 +1263,11 @@ constexpr size_t stage_smem_elems() {
 // (rows -1 .. BY); index 0 the value at the cell's right face, 1 at its left.
 // 3D: then the z-face net fluxes [2][5][NCELL] and the upper WENO5 values of
 // the columns' current cells [5][NCELL].
-template <int DIM, int BX, int BY>
+// (FP64: without that z state, which lives in registers.)
+template <int DIM, int BX, int BY, typename T = float>
 constexpr size_t recon_smem_elems() {
   return (size_t)2 * 5 * (BY * (BX + 2) + (plane_dims(DIM) == 2 ? (BY + 2) * BX : 0)) +
-         (marches(DIM) ? 3 * 5 * BX * BY : 0);
+         (marches(DIM) && sizeof(T) == 4 ? 3 * 5 * BX * BY : 0);
 }
 
 // Element offset of the Rusanov-NN parameters in the dynamic shared memory:
@@ -1198,7 +1302,7 @@ __global__ void __launch_bounds__(Geo<BX, BY, DIM, VISC>::NT, MINB)
     asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
     const size_t need = sizeof(T) * (SCH == SCH_NN ? nn_smem_offset<T, DIM, VISC, BX, BY>() + NN_PARAMS
                                                    : stage_smem_elems<T, DIM, VISC, BX, BY>() +
-                                                         (sch_pc(SCH) ? recon_smem_elems<DIM, BX, BY>() : 0));
+                                                         (sch_pc(SCH) ? recon_smem_elems<DIM, BX, BY, T>() : 0));
     if (!JF_CHECK(dyn >= need, "JFDBG smem %u < %llu\n", dyn, (unsigned long long)need)) return;
     if (work && threadIdx.x == 0)
       for (int i = blockIdx.x; i < nwork; i += gridDim.x) {

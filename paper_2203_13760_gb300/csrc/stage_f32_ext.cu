@@ -10,10 +10,12 @@ namespace jf {
 
 const StageVariant<float>* ext_variants_f32(int* count) {
   static const StageVariant<float> table[] = {
-      make_variant<float, 3, true, 32, 8, 2, SCH_GENERAL_EXT>(),
-      make_variant<float, 3, false, 32, 8, 2, SCH_GENERAL_EXT>(),
-      make_variant<float, 2, true, 32, 8, 2, SCH_GENERAL_EXT>(),
-      make_variant<float, 2, false, 32, 8, 2, SCH_GENERAL_EXT>(),
+      make_variant<float, 3, true, 32, 7, 2, SCH_GENERAL_EXT>(),
+      make_variant<float, 3, false, 32, 7, 2, SCH_GENERAL_EXT>(),
+      make_variant<float, 2, true, 32, 7, 2, SCH_GENERAL_EXT>(),
+      make_variant<float, 2, true, 32, 4, 4, SCH_GENERAL_EXT>(),
+      make_variant<float, 2, false, 32, 7, 2, SCH_GENERAL_EXT>(),
+      make_variant<float, 2, false, 32, 4, 4, SCH_GENERAL_EXT>(),
       make_variant<float, 1, true, 128, 1, 2, SCH_GENERAL_EXT>(),
       make_variant<float, 1, false, 128, 1, 2, SCH_GENERAL_EXT>(),
       make_variant<float, 3, true, 32, 7, 2, SCH_ROE_EXT>(),

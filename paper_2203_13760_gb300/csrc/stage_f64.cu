@@ -16,20 +16,22 @@ const StageVariant<double>* stage_variants<double>(int* count) {
       // CTA of 7 warps per SM (208 KB of shared memory), measured at TGV 256^3
       // 82.2 M cell-updates/s against 68.8 M for 32 x 4 (5 warps) and 49.1 M
       // for 32 x 2 at two CTAs per SM
-      make_variant<double, 3, true, 32, 6, 1, SCH_DEFAULT>(),
+      make_variant<double, 3, true, 32, 7, 1, SCH_DEFAULT>(),
       make_variant<double, 3, true, 32, 4, 1, SCH_DEFAULT>(),
       make_variant<double, 3, true, 32, 2, 2, SCH_DEFAULT>(),
-      make_variant<double, 3, false, 32, 6, 1, SCH_DEFAULT>(),
+      make_variant<double, 3, false, 32, 7, 1, SCH_DEFAULT>(),
       make_variant<double, 3, false, 32, 4, 1, SCH_DEFAULT>(),
       make_variant<double, 3, false, 32, 2, 2, SCH_DEFAULT>(),
       // 2D
       make_variant<double, 2, true, 32, 8, 1, SCH_DEFAULT>(),
       make_variant<double, 2, true, 32, 4, 2, SCH_DEFAULT>(),
+      make_variant<double, 2, true, 32, 3, 3, SCH_DEFAULT>(),
       make_variant<double, 2, false, 32, 8, 1, SCH_DEFAULT>(),
       make_variant<double, 2, false, 32, 4, 2, SCH_DEFAULT>(),
+      make_variant<double, 2, false, 32, 3, 3, SCH_DEFAULT>(),
       // 1D
-      make_variant<double, 1, true, 128, 1, 1, SCH_DEFAULT>(),
-      make_variant<double, 1, false, 128, 1, 1, SCH_DEFAULT>(),
+      make_variant<double, 1, true, 30, 1, 8, SCH_DEFAULT>(),
+      make_variant<double, 1, false, 30, 1, 8, SCH_DEFAULT>(),
     };
     int ng = 0;
     const StageVariant<double>* gen = general_variants_f64(&ng);

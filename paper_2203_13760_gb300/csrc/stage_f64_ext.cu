@@ -11,15 +11,19 @@ const StageVariant<double>* ext_variants_f64(int* count) {
       make_variant<double, 3, true, 32, 4, 1, SCH_GENERAL_EXT>(),
       make_variant<double, 3, false, 32, 4, 1, SCH_GENERAL_EXT>(),
       make_variant<double, 2, true, 32, 8, 1, SCH_GENERAL_EXT>(),
+      make_variant<double, 2, true, 32, 4, 2, SCH_GENERAL_EXT>(),
+      make_variant<double, 2, true, 32, 3, 3, SCH_GENERAL_EXT>(),
       make_variant<double, 2, false, 32, 8, 1, SCH_GENERAL_EXT>(),
-      make_variant<double, 1, true, 128, 1, 1, SCH_GENERAL_EXT>(),
-      make_variant<double, 1, false, 128, 1, 1, SCH_GENERAL_EXT>(),
+      make_variant<double, 2, false, 32, 4, 2, SCH_GENERAL_EXT>(),
+      make_variant<double, 2, false, 32, 3, 3, SCH_GENERAL_EXT>(),
+      make_variant<double, 1, true, 30, 1, 8, SCH_GENERAL_EXT>(),
+      make_variant<double, 1, false, 30, 1, 8, SCH_GENERAL_EXT>(),
       make_variant<double, 3, true, 32, 4, 1, SCH_ROE_EXT>(),
       make_variant<double, 3, false, 32, 4, 1, SCH_ROE_EXT>(),
       make_variant<double, 2, true, 32, 8, 1, SCH_ROE_EXT>(),
       make_variant<double, 2, false, 32, 8, 1, SCH_ROE_EXT>(),
-      make_variant<double, 1, true, 128, 1, 1, SCH_ROE_EXT>(),
-      make_variant<double, 1, false, 128, 1, 1, SCH_ROE_EXT>(),
+      make_variant<double, 1, true, 30, 1, 8, SCH_ROE_EXT>(),
+      make_variant<double, 1, false, 30, 1, 8, SCH_ROE_EXT>(),
   };
   *count = (int)(sizeof(table) / sizeof(table[0]));
   return table;

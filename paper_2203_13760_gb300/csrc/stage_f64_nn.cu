@@ -10,8 +10,8 @@ const StageVariant<double>* nn_variants_f64(int* count) {
       make_variant<double, 3, false, 32, 7, 1, SCH_NN>(),
       make_variant<double, 2, true, 32, 7, 1, SCH_NN>(),
       make_variant<double, 2, false, 32, 7, 1, SCH_NN>(),
-      make_variant<double, 1, true, 128, 1, 1, SCH_NN>(),
-      make_variant<double, 1, false, 128, 1, 1, SCH_NN>(),
+      make_variant<double, 1, true, 30, 1, 8, SCH_NN>(),
+      make_variant<double, 1, false, 30, 1, 8, SCH_NN>(),
   };
   *count = (int)(sizeof(table) / sizeof(table[0]));
   return table;

@@ -20,8 +20,8 @@ const StageVariant<double>* roe_variants_f64(int* count) {
       make_variant<double, 2, true, 32, 4, 2, SCH_ROE>(),
       make_variant<double, 2, false, 32, 8, 1, SCH_ROE>(),
       make_variant<double, 2, false, 32, 4, 2, SCH_ROE>(),
-      make_variant<double, 1, true, 128, 1, 1, SCH_ROE>(),
-      make_variant<double, 1, false, 128, 1, 1, SCH_ROE>(),
+      make_variant<double, 1, true, 30, 1, 8, SCH_ROE>(),
+      make_variant<double, 1, false, 30, 1, 8, SCH_ROE>(),
   };
   *count = (int)(sizeof(table) / sizeof(table[0]));
   return table;
