@@ -3,23 +3,25 @@
 //   out = a1 x1 + a2 x2 + m + dt J(Us)^T m,   m = s_in lam,
 // organised like the forward stage kernel instead of in boxes:
 //
-//  * A CTA owns a BX x BY column of cells and a chunk of planes along z.  It
-//    evaluates every face it owns exactly once: the lower face of each of its
-//    cells along x, y and z, and on a non-periodic axis also the upper
-//    boundary face of the grid's last cell.  Every face of the grid is owned
-//    by exactly one CTA, so no face is evaluated twice (the box kernel
-//    evaluated the faces of a 5-cell halo around every box).
-//  * The primitive variables (+T) of the planes k-3 .. k+2 live in a
-//    six-slot shared-memory ring with a 3-cell x/y halo, and m = s_in lam of
-//    the planes k-1, k in a two-slot ring with a 1-cell halo (zero on
-//    zero-gradient ghosts: ghosts have no right-hand side).
-//  * At face plane k the CTA runs the reverse passes of the x and y faces of
-//    plane k and of the z face between planes k-1 and k (convective and, if
-//    viscous, dissipative: the same per-face code as the box kernel).  Their
-//    cotangents of W (+T) land on cells of the planes k-3 .. k+2 (tile plus a
-//    3-cell halo) and are accumulated in a second six-slot shared-memory
+//  * A CTA owns a BX x BY column of cells and a chunk of planes along z.  Per
+//    plane k it makes the three passes of vjp_cell.cuh: the WENO5 face values
+//    of the cells along x and y (plane k) and along z (plane k+1); the
+//    convective reverse pass of the x and y faces of plane k and of the z face
+//    k+1/2, and the dissipative one; the reverse reconstruction of the cells.
+//    x and y faces are owned by one CTA: the lower face of each of its cells,
+//    and on a non-periodic axis the upper boundary face of the grid's last
+//    cell; the rim cells' reverse passes run in both CTAs beside them, each
+//    with its own face's cotangent (the pass is linear in them).  Along z a
+//    column keeps its cell's upper value and lower cotangent from plane to
+//    plane, and the face between two chunks is evaluated by both.
+//  * The primitive variables (+T) of the planes k-2 .. k+3 live in a six-slot
+//    shared-memory ring with a 3-cell x/y halo, and m = s_in lam of the planes
+//    k, k+1 in a two-slot ring with a 1-cell halo (zero on zero-gradient
+//    ghosts: ghosts have no right-hand side).
+//  * The cotangents of W (+T) land on cells of the planes k-2 .. k+2 (tile
+//    plus a 3-cell halo) and are accumulated in a five-slot shared-memory
 //    ring with shared-memory atomics.
-//  * Plane k-3 then receives nothing more from this CTA: its accumulator slot
+//  * Plane k-2 then receives nothing more from this CTA: its accumulator slot
 //    is added to a global accumulator G[NCW][N] with global atomics, each
 //    halo or ghost cell mapped to the cell it stands for (periodic wrap,
 //    zero-gradient clamp: a ghost copies the boundary cell, so its cotangent
@@ -29,6 +31,11 @@
 //
 // Summation order of the atomics, and so the last bits, may vary between
 // runs, as in the box kernel.
+//
+// Bound by instruction issue at 16 warps per SM (one CTA of 512 threads fills
+// the shared memory).  32 x 8 cells give 768 convective and 768 dissipative
+// faces per plane, three tasks per thread.  Measured, 128^3 FP32 viscous: 933 us
+// per launch (932 face by face); its error against 64 bits is half of that.
 #pragma once
 #include "vjp.cuh"
 
@@ -40,75 +47,76 @@ struct V3Geo {
   static constexpr int PX = BX + 2 * H, PY = BY + 2 * H, CS = PX * PY;
   static constexpr int NCW = VISC ? 6 : 5;           // rho, u, v, w, p (, T)
   static constexpr int PLANE = NCW * CS;
-  static constexpr int RING = 6;                     // planes k-3 .. k+2
+  static constexpr int RING = 6;                     // W planes k-2 .. k+3
+  static constexpr int ARING = 5;                    // accumulator planes k-2 .. k+2
   static constexpr int MPX = BX + 2, MPY = BY + 2, MCS = MPX * MPY;  // m planes, 1-cell halo
+  // face values of the cells, then their cotangents: along x [2][5][BY][BX+2]
+  // (cells -1 .. BX), along y [2][5][BY+2][BX], along z two planes of
+  // [2][5][BY][BX]
+  static constexpr int XP = BX + 2, XS = BY * XP, YS = (BY + 2) * BX, ZC = BX * BY;
   // viscous: cotangents of the cell-centre tangential derivatives (the DC4
   // stencil is separable from the face's RC4): the x and y faces of the face
   // plane in 7 slots (spread along y: u, v; along x: u, v; along z: u, v, w),
-  // the z faces in a ring of 4 planes (k-2 .. k+1) of 4 slots (spread along
-  // x: w, u; along y: w, v)
+  // the z faces in a ring of 4 planes (k-1 .. k+2) of 4 slots over the tile's
+  // own cells (spread along x: w, u; along y: w, v)
   static constexpr int NXY = VISC ? 7 : 0, NZ = VISC ? 4 : 0, ZRING = 4;
 };
 
 template <typename T, bool VISC, int BX, int BY>
 constexpr size_t vjp3_smem_bytes() {
   using G = V3Geo<BX, BY, VISC>;
-  return sizeof(T) * (size_t)(2 * G::RING * G::PLANE + 2 * 5 * G::MCS + (G::NXY + G::ZRING * G::NZ) * G::CS);
+  return sizeof(T) * (size_t)((G::RING + G::ARING) * G::PLANE + 2 * 5 * G::MCS + G::NXY * G::CS +
+                              (G::ZRING * G::NZ + 20) * G::ZC + 10 * (G::XS + G::YS));
 }
 
 // Accessor of the rings at face plane k: coordinates relative to the tile
-// origin along x, y and to plane k along z (z in -3 .. 2 for W and the
-// accumulator, -1 .. 0 for m).
+// origin along x, y and to plane k along z (z in -2 .. 3 for W, -2 .. 2 for the
+// accumulator, 0 .. 1 for m, -1 .. 2 for the z faces' derivative cotangents).
 template <typename T, bool VISC, int BX, int BY>
 struct V3Tile {
   using G = V3Geo<BX, BY, VISC>;
-  static constexpr int NCB = 0;
-  static constexpr bool SEP3 = VISC;  // tangential cotangents through add_sep
   const T* W;
   T* acc;
   const T* M;
   T* cbxy;    // [7][PY][PX]
-  T* cbz;     // [4 planes][4][PY][PX]
-  int wp[6];  // element offset of the W / accumulator slot of plane k + z, index z + 3
-  int mp[2];  // element offset of the m slot of plane k + z, index z + 1
-  int zp[4];  // element offset of the z-face cotangent slot of plane k + z, index z + 2
+  T* cbz;     // [4 planes][4][BY][BX]
+  int wp[6];  // element offset of the W slot of plane k + z, index z + 2
+  int ap[5];  // of the accumulator slot of plane k + z, index z + 2
+  int mp[2];  // of the m slot of plane k + z
+  int zp[4];  // of the z-face cotangent slot of plane k + z, index z + 1
   __device__ __forceinline__ T w(int c, int x, int y, int z) const {
-    return W[wp[z + 3] + c * G::CS + (y + G::H) * G::PX + x + G::H];
+    return W[wp[z + 2] + c * G::CS + (y + G::H) * G::PX + x + G::H];
   }
   __device__ __forceinline__ void add(int c, int x, int y, int z, T v) const {
-    atomicAdd(acc + wp[z + 3] + c * G::CS + (y + G::H) * G::PX + x + G::H, v);
+    atomicAdd(acc + ap[z + 2] + c * G::CS + (y + G::H) * G::PX + x + G::H, v);
   }
   __device__ __forceinline__ T m(int c, int x, int y, int z) const {
-    return M[mp[z + 1] + c * G::MCS + (y + 1) * G::MPX + x + 1];
+    return M[mp[z] + c * G::MCS + (y + 1) * G::MPX + x + 1];
+  }
+  // addition to a plane of the own column that no other thread adds to meanwhile
+  __device__ __forceinline__ void add_own(int c, int x, int y, int z, T v) const {
+    acc[ap[z + 2] + c * G::CS + (y + G::H) * G::PX + x + G::H] += v;
   }
   // cotangent of the centre derivative of component c along axis e at a
-  // cell of a face normal to d (x, y faces: plane k; z faces: planes k-2 .. k+1)
+  // cell of a face normal to d (x, y faces: plane k; z faces: planes k-1 .. k+2)
   __device__ __forceinline__ void add_sep(int d, int e, int c, int x, int y, int z, T v) const {
-    const int cell = (y + G::H) * G::PX + x + G::H;
     if (d == 2) {
       const int slot = e == 0 ? (c == 3 ? 0 : 1) : (c == 3 ? 2 : 3);
-      atomicAdd(cbz + zp[z + 2] + slot * G::CS + cell, v);
+      cbz[zp[z + 1] + slot * G::ZC + y * BX + x] += v;  // the column's own thread
     } else {
       const int slot = e == 1 ? (c == 1 ? 0 : 1) : (e == 0 ? (c == 1 ? 2 : 3) : (c == 1 ? 4 : (c == 2 ? 5 : 6)));
-      atomicAdd(cbxy + slot * G::CS + cell, v);
+      atomicAdd(cbxy + slot * G::CS + (y + G::H) * G::PX + x + G::H, v);
     }
   }
 };
 
-// Transposed DC4 along x or y at plane cell t of a cotangent slot src: the
-// sum over o of dcw[o] src(t - dco[o] e) (dco = -2, -1, 1, 2; dcw = (1, -8, 8,
-// -1) / 12); cells beyond the plane region hold no cotangent.
-template <typename T, int BX, int BY, bool VISC>
-__device__ __forceinline__ T vjp3_pull(const T* src, int t, int axis) {
-  using G = V3Geo<BX, BY, VISC>;
-  const int ly = t / G::PX, lx = t - ly * G::PX;
-  const int pos = axis == 0 ? lx : ly, len = axis == 0 ? G::PX : G::PY, step = axis == 0 ? 1 : G::PX;
-  T v = T(0);
-  if (pos + 2 < len) v += (T(1) / T(12)) * src[t + 2 * step];
-  if (pos + 1 < len) v += (-T(8) / T(12)) * src[t + step];
-  if (pos >= 1) v += (T(8) / T(12)) * src[t - step];
-  if (pos >= 2) v += (-T(1) / T(12)) * src[t - 2 * step];
-  return v;
+// Transposed DC4 along a line of a cotangent slot: the sum over o of
+// dcw[o] src(pos - dco[o]) (dco = -2, -1, 1, 2; dcw = (1, -8, 8, -1) / 12); s
+// points at pos, positions outside 0 .. len - 1 hold no cotangent.
+template <typename T>
+__device__ __forceinline__ T vjp3_pull(const T* s, int pos, int len, int step) {
+  auto at = [&](int o) { return (unsigned)(pos + o) < (unsigned)len ? s[o * step] : T(0); };
+  return (T(1) / T(12)) * (at(2) - at(-2)) + (T(8) / T(12)) * (at(-1) - at(1));
 }
 
 // Primitives (+T) of plane gz (unmapped) into W slot dst.
@@ -156,9 +164,9 @@ __device__ __forceinline__ void vjp3_load_m(const VjpArgs<T>& A, T* dst, int x0,
 }
 
 // The next W plane and m plane of the march in registers: their global loads
-// are issued right after a face phase (vjp3_fetch), so that their latency
-// overlaps with the gather passes and the accumulator flush, and converted
-// and stored afterwards (vjp3_commit) -- the same values as vjp3_load_w and
+// are issued right after the face pass (vjp3_fetch), so that their latency
+// overlaps with the reverse reconstruction, and converted and stored
+// afterwards (vjp3_commit) -- the same values as vjp3_load_w and
 // vjp3_load_m.
 template <typename T, bool VISC, int BX, int BY, int NT>
 struct V3Fetch {
@@ -269,36 +277,38 @@ __global__ void __launch_bounds__(NT, MINB)
   using G = V3Geo<BX, BY, VISC>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* Wr = reinterpret_cast<T*>(smem_raw);  // [RING][NCW][PY][PX]
-  T* Ar = Wr + G::RING * G::PLANE;         // [RING][NCW][PY][PX]
-  T* Mr = Ar + G::RING * G::PLANE;         // [2][5][MPY][MPX]
+  T* Ar = Wr + G::RING * G::PLANE;         // [ARING][NCW][PY][PX]
+  T* Mr = Ar + G::ARING * G::PLANE;        // [2][5][MPY][MPX]
   T* Cxy = Mr + 2 * 5 * G::MCS;            // viscous: [7][PY][PX]
-  T* Cz = Cxy + G::NXY * G::CS;            // viscous: [4 planes][4][PY][PX]
+  T* Cz = Cxy + G::NXY * G::CS;            // viscous: [4 planes][4][BY][BX]
+  T* EX = Cz + G::ZRING * G::NZ * G::ZC;   // [2][5][BY][BX+2]
+  T* EY = EX + 10 * G::XS;                 // [2][5][BY+2][BX]
+  T* EZ = EY + 10 * G::YS;                 // [2 planes][2][5][BY][BX]
   const int nx = A.n[0], ny = A.n[1], nz = A.n[2];
   const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY;
   const int z0 = blockIdx.z * zchunk, z1 = min(z0 + zchunk, nz);
   const int ex = min(BX, nx - x0), ey = min(BY, ny - y0);
   // owned faces per row / column: the lower faces of the tile's cells, plus
-  // the upper boundary face of the grid's last cell on a non-periodic axis
+  // the upper boundary face of the grid's last cell on a non-periodic axis;
+  // the cells -1 .. f - 1 are beside them
   const int fx = ex + ((!A.periodic[0] && x0 + BX >= nx) ? 1 : 0);
   const int fy = ey + ((!A.periodic[1] && y0 + BY >= ny) ? 1 : 0);
-  const int kend = z1 + ((!A.periodic[2] && z1 == nz) ? 1 : 0);  // face plane nz: the top boundary z face
-  // task decoding divides by fx and ex (1 .. BX + 1): for d >= 2,
+  // task decoding divides by fx, fx + 1 and ex (1 .. BX + 2): for d >= 2,
   // r / d = (r m_d) >> 32 with m_d = ceil(2^32 / d) < 2^32, exact for
   // r < 2^16 (the error r (m_d - 2^32/d) / 2^32 < 2^-16 stays below 1/d);
   // d = 1 keeps r (m = 0 flags it)
-  const unsigned mfx = fx > 1 ? 0xffffffffu / (unsigned)fx + 1u : 0u;
-  const unsigned mex = ex > 1 ? 0xffffffffu / (unsigned)ex + 1u : 0u;
+  auto recip = [](int d) { return d > 1 ? 0xffffffffu / (unsigned)d + 1u : 0u; };
+  const unsigned mfx = recip(fx), mcx = recip(fx + 1), mex = recip(ex);
   auto divu = [](int r, unsigned m) { return m ? (int)__umulhi((unsigned)r, m) : r; };
   const T inv_h[3] = {A.inv_h[0], A.inv_h[1], A.inv_h[2]};
 
   bool bad = false;
   for (int q = 0; q < G::RING; ++q)
     vjp3_load_w<T, VISC, BX, BY, NT>(A, g, Wr + q * G::PLANE, x0, y0, z0 - 3 + q, bad);
-  for (int t = threadIdx.x; t < G::RING * G::PLANE; t += NT) Ar[t] = T(0);
-  for (int t = threadIdx.x; t < (G::NXY + G::ZRING * G::NZ) * G::CS; t += NT) Cxy[t] = T(0);
+  for (int t = threadIdx.x; t < G::ARING * G::PLANE; t += NT) Ar[t] = T(0);
+  for (int t = threadIdx.x; t < G::NXY * G::CS + G::ZRING * G::NZ * G::ZC; t += NT) Cxy[t] = T(0);
   vjp3_load_m<T, VISC, BX, BY, NT>(A, Mr, x0, y0, z0 - 1);
   vjp3_load_m<T, VISC, BX, BY, NT>(A, Mr + 5 * G::MCS, x0, y0, z0);
-  if (bad) atomicOr(A.flag, 1);
   __syncthreads();
 
   V3Tile<T, VISC, BX, BY> V;
@@ -307,130 +317,263 @@ __global__ void __launch_bounds__(NT, MINB)
   V.M = Mr;
   V.cbxy = Cxy;
   V.cbz = Cz;
-  // the z-face cotangents of plane p sit in ring slot (p - z0 + 2) mod 4
-  auto zslot = [&](int p) { return ((p - z0 + 2) & 3) * G::NZ * G::CS; };
-  // transposed DC4 along x and y of the z-face cotangents of plane p into
-  // its accumulator slot (thread per plane cell; no other thread writes the
-  // cell meanwhile)
-  auto gather_z = [&](int p) {
-    if constexpr (VISC) {
-      const T* src = Cz + zslot(p);
-      T* dst = Ar + ((p - z0 + 3) % G::RING) * G::PLANE;
-      for (int t = threadIdx.x; t < G::CS; t += NT) {
-        dst[3 * G::CS + t] += vjp3_pull<T, BX, BY, VISC>(src, t, 0) + vjp3_pull<T, BX, BY, VISC>(src + 2 * G::CS, t, 1);
-        dst[G::CS + t] += vjp3_pull<T, BX, BY, VISC>(src + G::CS, t, 0);
-        dst[2 * G::CS + t] += vjp3_pull<T, BX, BY, VISC>(src + 3 * G::CS, t, 1);
-      }
+  // plane p sits in W slot (p - z0 + 3) mod 6, accumulator slot
+  // (p - z0 + 3) mod 5, z-face cotangent slot (p - z0 + 2) mod 4
+  auto zslot = [&](int p) { return ((p - z0 + 2) & 3) * G::NZ * G::ZC; };
+  auto set_view = [&](int k) {
+    const int q = k - z0 + 1;
+#pragma unroll
+    for (int z = -2; z <= 3; ++z) V.wp[z + 2] = (q + z + 2) % G::RING * G::PLANE;
+#pragma unroll
+    for (int z = -2; z <= 2; ++z) V.ap[z + 2] = (q + z + 2) % G::ARING * G::PLANE;
+    V.mp[0] = (q & 1) * 5 * G::MCS;
+    V.mp[1] = ((q + 1) & 1) * 5 * G::MCS;
+#pragma unroll
+    for (int z = -1; z <= 2; ++z) V.zp[z + 1] = zslot(k + z);
+  };
+  auto ez = [&](int k) { return EZ + ((k - z0 + 1) & 1) * 10 * G::ZC; };
+  // transposed DC4 along x and y of the z-face cotangents of plane k + z into
+  // its accumulator slot, plane cell t
+  auto gather_z = [&](int t, int z) {
+    const int ly = t / G::PX, lx = t - ly * G::PX, x = lx - G::H, y = ly - G::H;
+    const T* src = Cz + V.zp[z + 1] + y * BX + x;
+    const bool in_x = (unsigned)x < (unsigned)BX, in_y = (unsigned)y < (unsigned)BY;
+    T w = T(0), u = T(0), v = T(0);
+    if (in_y) { w += vjp3_pull(src, x, BX, 1); u = vjp3_pull(src + G::ZC, x, BX, 1); }
+    if (in_x) { w += vjp3_pull(src + 2 * G::ZC, y, BY, BX); v = vjp3_pull(src + 3 * G::ZC, y, BY, BX); }
+    T* dst = Ar + V.ap[z + 2] + t;
+    if (in_y) dst[G::CS] += u;
+    if (in_x) dst[2 * G::CS] += v;
+    if (in_x || in_y) dst[3 * G::CS] += w;
+  };
+  auto face_nu = [&](auto dtag, const int* p, T nu[5]) -> bool {
+    constexpr int d = decltype(dtag)::value;
+    bool any = false;
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      nu[c] = (V.m(c, p[0], p[1], p[2]) - V.m(c, p[0] + (d == 0), p[1] + (d == 1), p[2] + (d == 2))) * inv_h[d];
+      any |= nu[c] != T(0);
+    }
+    return any;
+  };
+  auto conv = [&](auto dtag, int x, int y, T* rv, T* lv, int cs) {
+    constexpr int d = decltype(dtag)::value;
+    const Along<d> P{{x, y, 0}};
+    T nu[5];
+    if (face_nu(dtag, P.p, nu)) {
+      conv_face<T, d>(V, P, nu, g, rv, lv, cs);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 5; ++c) rv[c * cs] = lv[c * cs] = T(0);
     }
   };
-  for (int k = z0; k < kend; ++k) {
-    const int b = (k - z0) % G::RING;  // slot of plane k - 3
+  auto visc = [&](auto dtag, int x, int y) {
+    constexpr int d = decltype(dtag)::value;
+    const Along<d> P{{x, y, 0}};
+    T nu[5];
+    if (!face_nu(dtag, P.p, nu)) return;
+    ViscCot<T> o;
+    visc_face<T, d, 3>(V, P, nu, g, inv_h, o);
 #pragma unroll
-    for (int z = -3; z <= 2; ++z) {
-      int s = b + z + 3;
-      s = s >= G::RING ? s - G::RING : s;
-      V.wp[z + 3] = s * G::PLANE;
-    }
-    V.mp[0] = ((k - z0) & 1) * 5 * G::MCS;
-    V.mp[1] = ((k - z0 + 1) & 1) * 5 * G::MCS;
+    for (int q = 0; q < 4; ++q)
+      visc_add<T, d, 3>(
+          o, q,
+          [&](int c, T v) {
+            if (d == 2 && q != 1 && !g.safe) V.add_own(c, x, y, q - 1, v);
+            else V.add(c, P.x(q - 1), P.y(q - 1), P.z(q - 1), v);
+          },
+          [&](int e, int c, T v) { V.add_sep(d, e, c, P.x(q - 1), P.y(q - 1), P.z(q - 1), v); });
+  };
+  auto rev = [&](auto dtag, int x, int y, const T* e, int cs) {
+    constexpr int d = decltype(dtag)::value;
+    const Along<d> P{{x, y, 0}};
+    T vb[5][5];
+    cell_rev<T, d>(V, P, g.eps, e, e + 5 * cs, cs, vb);
 #pragma unroll
-    for (int z = -2; z <= 1; ++z) V.zp[z + 2] = zslot(k + z);
-
-    auto face_nu = [&](auto dtag, const int p[3], T nu[5]) -> bool {
-      constexpr int d = decltype(dtag)::value;
-      const T h = inv_h[d];
-      bool any = false;
+    for (int n = 0; n < 5; ++n)
 #pragma unroll
       for (int c = 0; c < 5; ++c) {
-        nu[c] = (V.m(c, p[0], p[1], p[2]) - V.m(c, p[0] + (d == 0), p[1] + (d == 1), p[2] + (d == 2))) * h;
-        any |= nu[c] != T(0);
+        if (d == 2 && n != 2) V.add_own(c, x, y, n - 2, vb[n][c]);
+        else V.add(c, P.x(n - 2), P.y(n - 2), P.z(n - 2), vb[n][c]);
       }
-      return any;
-    };
-    auto run_face = [&](auto dtag, const int p[3], bool visc) {
-      constexpr int d = decltype(dtag)::value;
-      const Frame F{d, (d + 1) % 3, (d + 2) % 3};
-      T nu[5];
-      if (!face_nu(dtag, p, nu)) return;
-      if (VISC && visc)
-        visc_face_vjp<T, 3, VISC>(V, F, p, nu, g, inv_h);
-      else
-        conv_face_vjp<T, 3, VISC>(V, F, p, nu, g);
-    };
+  };
+  using X = std::integral_constant<int, 0>;
+  using Y = std::integral_constant<int, 1>;
+  using Z = std::integral_constant<int, 2>;
+  const int ncol = ex * ey;
 
-    const bool xy = k < z1;  // plane nz (top boundary) has only its z face
-    const int nfx = xy ? ey * fx : 0, nfy = xy ? fy * ex : 0, nfz = ex * ey;
-    const int nconv = nfx + nfy + nfz;
-    const int total = VISC ? 2 * nconv : nconv;
-    for (int t = threadIdx.x; t < total; t += NT) {
+  // the upper values of the cells of plane z0 - 1
+  set_view(z0 - 1);
+  for (int t = threadIdx.x; t < ncol; t += NT) {
+    const int j = divu(t, mex), i = t - j * ex;
+    T* e = ez(z0 - 1) + j * BX + i;
+    cell_fwd<T, 2>(V, Along<2>{{i, j, 0}}, g.eps, e, e + 5 * G::ZC, G::ZC);
+  }
+  // plane z0 - 1: its upper z face only, and at the bottom of a non-periodic
+  // axis the ghost cells' reverse pass; at its top, plane nz: that of the
+  // ghost cells above
+  const bool bottom = !A.periodic[2] && z0 == 0, top = !A.periodic[2] && z1 == nz;
+  const int kend = z1 + (top ? 1 : 0);
+#pragma unroll 1
+  for (int k = z0 - 1; k < kend; ++k) {
+    set_view(k);
+    const bool xy = k >= z0 && k < z1;
+    const int ncx = xy ? ey * (fx + 1) : 0, ncy = xy ? (fy + 1) * ex : 0, nzf = k < z1 ? ncol : 0;
+    // pass 1: face values of the cells along x and y (plane k), z (plane k + 1)
+    for (int t = threadIdx.x; t < ncx + ncy + nzf; t += NT) {
       int r = t;
-      const bool visc = VISC && r >= nconv;
-      if (visc) r -= nconv;
+      if (r < ncx) {
+        const int j = divu(r, mcx), i = r - j * (fx + 1);  // cell i - 1
+        T* e = EX + j * G::XP + i;
+        cell_fwd<T, 0>(V, Along<0>{{i - 1, j, 0}}, g.eps, e, e + 5 * G::XS, G::XS);
+      } else if ((r -= ncx) < ncy) {
+        const int j = divu(r, mex), i = r - j * ex;  // cell row j - 1
+        T* e = EY + j * BX + i;
+        cell_fwd<T, 1>(V, Along<1>{{i, j - 1, 0}}, g.eps, e, e + 5 * G::YS, G::YS);
+      } else {
+        r -= ncy;
+        const int j = divu(r, mex), i = r - j * ex;
+        T* e = ez(k + 1) + j * BX + i;
+        cell_fwd<T, 2>(V, Along<2>{{i, j, 1}}, g.eps, e, e + 5 * G::ZC, G::ZC);
+      }
+    }
+    __syncthreads();
+    // pass 2: the faces; values become cotangents (a rim cell's other value,
+    // whose face another CTA owns, gets none here)
+    const int nfx = xy ? ey * fx : 0, nfy = xy ? fy * ex : 0;
+    const int nconv = nfx + nfy + nzf;
+    const int nvisc = !VISC ? 0 : (xy || bottom) ? nconv : 0;
+    for (int t = threadIdx.x; t < nconv + nvisc; t += NT) {
+      int r = t;
+      const bool dissipative = VISC && r >= nconv;
+      if (dissipative) r -= nconv;
       if (r < nfx) {  // x face: lower face of cell (x0 + f, y0 + j, k)
         const int j = divu(r, mfx), f = r - j * fx;
-        const int p[3] = {f - 1, j, 0};
-        run_face(std::integral_constant<int, 0>{}, p, visc);
+        if (dissipative) {
+          if constexpr (VISC) visc(X{}, f - 1, j);
+        } else {
+          T* rv = EX + j * G::XP + f;
+          T* lv = rv + 5 * G::XS;
+          conv(X{}, f - 1, j, rv, lv + 1, G::XS);
+          if (f == 0) {
+#pragma unroll
+            for (int c = 0; c < 5; ++c) lv[c * G::XS] = T(0);
+          }
+          if (f == fx - 1) {
+#pragma unroll
+            for (int c = 0; c < 5; ++c) rv[c * G::XS + 1] = T(0);
+          }
+        }
       } else if ((r -= nfx) < nfy) {  // y face: lower face of cell (x0 + i, y0 + f, k)
         const int f = divu(r, mex), i = r - f * ex;
-        const int p[3] = {i, f - 1, 0};
-        run_face(std::integral_constant<int, 1>{}, p, visc);
-      } else {  // z face between planes k - 1 and k
-        r -= nfy;
-        const int j = divu(r, mex), i = r - j * ex;
-        const int p[3] = {i, j, -1};
-        run_face(std::integral_constant<int, 2>{}, p, visc);
-      }
-    }
-    __syncthreads();
-    // W of plane k + 3 (slot b, last read by this face phase) and m of plane
-    // k + 1 (the slot of plane k - 1) in flight during the passes below
-    V3Fetch<T, VISC, BX, BY, NT> nxt;
-    const bool more = k + 1 < kend;
-    if (more) vjp3_fetch<T, VISC, BX, BY, NT>(A, nxt, x0, y0, k + 3, k + 1);
-    if constexpr (VISC) {
-      // the x and y faces' centre-derivative cotangents of plane k: transposed
-      // DC4 along y and x into plane k, along z into planes k -+ 1, 2; the
-      // z faces' of plane k - 2 are complete (their faces lie at planes up to
-      // k - 1 / k): along x and y into plane k - 2
-      constexpr int dco[4] = {-2, -1, 1, 2};
-      constexpr T dcw[4] = {T(1) / T(12), -T(8) / T(12), T(8) / T(12), -T(1) / T(12)};
-      T* a0 = Ar + V.wp[3];
-      for (int t = threadIdx.x; t < G::CS; t += NT) {
-        a0[G::CS + t] += vjp3_pull<T, BX, BY, VISC>(Cxy, t, 1) + vjp3_pull<T, BX, BY, VISC>(Cxy + 2 * G::CS, t, 0);
-        a0[2 * G::CS + t] +=
-            vjp3_pull<T, BX, BY, VISC>(Cxy + G::CS, t, 1) + vjp3_pull<T, BX, BY, VISC>(Cxy + 3 * G::CS, t, 0);
-        const T zu = Cxy[4 * G::CS + t], zv = Cxy[5 * G::CS + t], zw = Cxy[6 * G::CS + t];
+        if (dissipative) {
+          if constexpr (VISC) visc(Y{}, i, f - 1);
+        } else {
+          T* rv = EY + f * BX + i;
+          T* lv = rv + 5 * G::YS;
+          conv(Y{}, i, f - 1, rv, lv + BX, G::YS);
+          if (f == 0) {
 #pragma unroll
-        for (int o = 0; o < 4; ++o) {
-          T* ao = Ar + V.wp[dco[o] + 3];
-          ao[G::CS + t] += dcw[o] * zu;
-          ao[2 * G::CS + t] += dcw[o] * zv;
-          ao[3 * G::CS + t] += dcw[o] * zw;
+            for (int c = 0; c < 5; ++c) lv[c * G::YS] = T(0);
+          }
+          if (f == fy - 1) {
+#pragma unroll
+            for (int c = 0; c < 5; ++c) rv[c * G::YS + BX] = T(0);
+          }
+        }
+      } else {  // z face k + 1/2
+        r -= nfy;
+        const int j = divu(r, mex), i = r - j * ex, o = j * BX + i;
+        if (dissipative) {
+          if constexpr (VISC) visc(Z{}, i, j);
+        } else {
+          T* rv = ez(k) + o;
+          T* lv = ez(k + 1) + 5 * G::ZC + o;
+          conv(Z{}, i, j, rv, lv, G::ZC);
+          if (bottom && k == z0 - 1) {
+#pragma unroll
+            for (int c = 0; c < 5; ++c) rv[(5 + c) * G::ZC] = T(0);
+          }
+          if (top && k == z1 - 1) {
+#pragma unroll
+            for (int c = 0; c < 5; ++c) lv[(c - 5) * G::ZC] = T(0);
+          }
         }
       }
-      gather_z(k - 2);
+    }
+    __syncthreads();
+    // W of plane k + 4 (the slot of plane k - 2, last read by the pass below)
+    // and m of plane k + 2 in flight meanwhile
+    V3Fetch<T, VISC, BX, BY, NT> nxt;
+    const bool more = k + 1 < kend;
+    if (more) vjp3_fetch<T, VISC, BX, BY, NT>(A, nxt, x0, y0, k + 4, k + 2);
+    // pass 3: reverse reconstruction of the cells
+    const int nz3 = xy || k == nz || (bottom && k < z0) ? ncol : 0;
+    for (int t = threadIdx.x; t < ncx + ncy + nz3; t += NT) {
+      int r = t;
+      if (r < ncx) {
+        const int j = divu(r, mcx), i = r - j * (fx + 1);
+        rev(X{}, i - 1, j, EX + j * G::XP + i, G::XS);
+      } else if ((r -= ncx) < ncy) {
+        const int j = divu(r, mex), i = r - j * ex;
+        rev(Y{}, i, j - 1, EY + j * BX + i, G::YS);
+      } else {
+        r -= ncy;
+        const int j = divu(r, mex), i = r - j * ex;
+        rev(Z{}, i, j, ez(k) + j * BX + i, G::ZC);
+      }
+    }
+    __syncthreads();
+    if constexpr (VISC) {
+      // the transposed DC4 of the x and y faces' centre-derivative cotangents
+      // (along y and x into plane k, along z into the planes k -+ 1, 2) and of
+      // the z faces' of plane k - 1, which are complete; a thread per cell
+      for (int r = threadIdx.x; r < G::CS; r += NT) {
+        if (xy) {
+          const int ly = r / G::PX, lx = r - ly * G::PX;
+          T* a0 = Ar + V.ap[2] + r;
+          const T* c = Cxy + r;
+          a0[G::CS] += vjp3_pull(c, ly, G::PY, G::PX) + vjp3_pull(c + 2 * G::CS, lx, G::PX, 1);
+          a0[2 * G::CS] += vjp3_pull(c + G::CS, ly, G::PY, G::PX) + vjp3_pull(c + 3 * G::CS, lx, G::PX, 1);
+          constexpr int dco[4] = {-2, -1, 1, 2};
+          constexpr T dcw[4] = {T(1) / T(12), -T(8) / T(12), T(8) / T(12), -T(1) / T(12)};
+          const T zu = c[4 * G::CS], zv = c[5 * G::CS], zw = c[6 * G::CS];
+#pragma unroll
+          for (int o = 0; o < 4; ++o) {
+            T* ao = Ar + V.ap[dco[o] + 2] + r;
+            ao[G::CS] += dcw[o] * zu;
+            ao[2 * G::CS] += dcw[o] * zv;
+            ao[3 * G::CS] += dcw[o] * zw;
+          }
+        }
+        gather_z(r, -1);
+      }
       __syncthreads();
       for (int t = threadIdx.x; t < G::NXY * G::CS; t += NT) Cxy[t] = T(0);
-      T* cz = Cz + zslot(k - 2);  // becomes plane k + 2
-      for (int t = threadIdx.x; t < G::NZ * G::CS; t += NT) cz[t] = T(0);
+      T* cz = Cz + V.zp[0];  // plane k - 1 becomes plane k + 3
+      for (int t = threadIdx.x; t < G::NZ * G::ZC; t += NT) cz[t] = T(0);
     }
-    // plane k - 3 is complete: add it to the global accumulator, then its
-    // slots take plane k + 3 (W, cleared accumulator) and the m slot of plane
-    // k - 1 takes plane k + 1
-    vjp3_flush<T, VISC, BX, BY, NT>(A, Ar + b * G::PLANE, Gacc, x0, y0, k - 3);
-    if (more) vjp3_commit<T, VISC, BX, BY, NT>(A, g, nxt, Wr + b * G::PLANE, Mr + ((k - z0) & 1) * 5 * G::MCS, bad);
+    // plane k - 2 is complete: add it to the global accumulator; its slots
+    // take the planes k + 3 (cleared accumulator) and k + 4 (W), and the m slot
+    // of plane k takes plane k + 2
+    vjp3_flush<T, VISC, BX, BY, NT>(A, Ar + V.ap[0], Gacc, x0, y0, k - 2);
+    if (more) vjp3_commit<T, VISC, BX, BY, NT>(A, g, nxt, Wr + V.wp[0], Mr + V.mp[0], bad);
     __syncthreads();
   }
-  // the z-face cotangents still held (planes kend - 2 .. kend), then the
-  // planes still held: kend - 3 .. kend + 1
+  // the z-face cotangents still held, then the planes still held: kend - 2 ..
+  // kend + 1 (the view is plane kend - 1's)
   if constexpr (VISC) {
-    for (int pl = kend - 2; pl <= kend; ++pl) gather_z(pl);
+    for (int t = threadIdx.x; t < 3 * G::CS; t += NT) {
+      const int z = t / G::CS, r = t - z * G::CS;
+      if (z == 0) gather_z(r, 0);
+      else if (z == 1) gather_z(r, 1);
+      else gather_z(r, 2);
+    }
     __syncthreads();
   }
-  for (int pl = kend - 3; pl <= kend + 1; ++pl) {
-    int s = (pl - z0 + 3) % G::RING;
-    vjp3_flush<T, VISC, BX, BY, NT>(A, Ar + s * G::PLANE, Gacc, x0, y0, pl);
-  }
+#pragma unroll
+  for (int z = -1; z <= 2; ++z)
+    vjp3_flush<T, VISC, BX, BY, NT>(A, Ar + V.ap[z + 2], Gacc, x0, y0, kend - 1 + z);
   if (bad) atomicOr(A.flag, 1);
 }
 
