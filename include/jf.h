@@ -337,6 +337,18 @@ jf_status jf_batch_step(jf_handle batch, void* const* U_ptrs, int nsteps, double
 jf_status jf_batch_feed_forward(jf_handle batch, void* const* U0_ptrs, void* const* traj_ptrs, int nsteps,
                                 const double* dt_dev, void* stream);
 
+/* Reverse sweep of jf_batch_feed_forward: from the stored trajectories
+ * (traj_ptrs, as written there) and the cotangents of every slot (grad_ptrs,
+ * the same layout) the cotangent of each initial state, written to
+ * lam0_ptrs[s] (5 * N_s elements, distinct from the other arrays):
+ * lam^n = g^n, lam^t = g^t + (d slot t+1 / d slot t)^T lam^{t+1}.  With the
+ * Rusanov-NN flux and theta_bar != NULL (JF_NN_PARAMS elements) the parameter
+ * gradient of all steps is added to theta_bar.  The schemes of
+ * jf_batch_step_vjp; its launches, without a call per step.  Asynchronous on
+ * `stream`, which must not be in capture. */
+jf_status jf_batch_feed_forward_vjp(jf_handle batch, void* const* traj_ptrs, void* const* grad_ptrs, int nsteps,
+                                    const double* dt_dev, void* const* lam0_ptrs, void* theta_bar, void* stream);
+
 /* Parameters of the Rusanov-NN network of a handle (single grid or batch)
  * whose scheme has flux == JF_FLUX_RUSANOV_NN (Section 7.4).  theta is a
  * caller-owned device array of nparams == JF_NN_PARAMS elements of the

@@ -145,8 +145,10 @@ class _FeedForward(torch.autograd.Function):
     def forward(ctx, batch, nsteps, dt, theta, *U0s):
         if theta is not None and (batch._nn is None or batch._nn.data_ptr() != theta.data_ptr()):
             raise ValueError("theta must be the tensor the batch holds (Batch.set_nn)")
-        trajs = batch.feed_forward([U.detach().contiguous() for U in U0s], nsteps, dt)
+        dt_dev = batch._steps(dt)
+        trajs = batch._feed_forward([U.detach().contiguous() for U in U0s], nsteps, dt_dev)
         ctx.batch, ctx.nsteps, ctx.with_theta = batch, nsteps, theta is not None
+        ctx.dt_dev = dt_dev
         ctx.dts = [float(dt)] * batch.nsim if not hasattr(dt, "__len__") else [float(x) for x in dt]
         ctx.save_for_backward(*trajs)
         return tuple(trajs)
@@ -156,26 +158,16 @@ class _FeedForward(torch.autograd.Function):
         trajs = ctx.saved_tensors
         theta_bar = torch.zeros_like(ctx.batch._nn) if ctx.with_theta else None
 
-        # the C ABI wants 16-byte aligned states, which a trajectory slot of a
-        # state whose size is not a multiple of 16 bytes is not: such slots are
-        # passed as aligned copies
+        # the C ABI wants 16-byte aligned arrays, which a trajectory slot of a
+        # state whose size is not a multiple of 16 bytes (or a view among the
+        # cotangents) is not: such arrays are passed as aligned copies
         def aligned(x):
             return x if x.data_ptr() % 16 == 0 else x.clone()
 
         if ctx.batch.supports_step_vjp():
-            # every simulation of the batch in the same launches, one call per step
-            g = [torch.zeros_like(tr) if gi is None else gi.contiguous() for tr, gi in zip(trajs, grads)]
-            dt = torch.tensor(ctx.dts, dtype=torch.float64, device=trajs[0].device)
-            lam = [gi[ctx.nsteps].clone() for gi in g]
-            nxt = [torch.empty_like(x) for x in lam]
-            if theta_bar is not None:  # one parameter-gradient launch for the whole sweep
-                ctx.batch.param_grad_begin(ctx.nsteps)
-            for t in reversed(range(ctx.nsteps)):
-                ctx.batch.step_vjp([aligned(tr[t]) for tr in trajs], dt, lam, nxt, [aligned(gi[t]) for gi in g],
-                                   theta_bar)
-                lam, nxt = nxt, lam
-            if theta_bar is not None:
-                ctx.batch.param_grad_end(theta_bar)
+            # every simulation of the batch in the same launches, one call for the sweep
+            g = [torch.zeros_like(tr) if gi is None else aligned(gi.contiguous()) for tr, gi in zip(trajs, grads)]
+            lam = ctx.batch.feed_forward_vjp(trajs, g, ctx.nsteps, ctx.dt_dev, theta_bar)
             return (None, None, None, theta_bar, *lam)
         out = []
         for i, (traj, g) in enumerate(zip(trajs, grads)):

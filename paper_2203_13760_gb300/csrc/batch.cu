@@ -315,19 +315,24 @@ jf_status feed_forward_batch(jf_ctx* h, void* const* U0_ptrs, void* const* traj_
       desc[(size_t)t * ns + i] = d;
     }
   }
-  // one allocation for the tables; freed after the stream has used them
+  // one stream-ordered allocation for the tables, freed after the stream has
+  // used them; uploaded from pinned memory, so that the call does not wait for
+  // the stream
+  if (being_captured(s)) { set_error(h, "feed_forward: the stream is being captured"); return JF_ERR_CUDA; }
   const size_t bytes_desc = desc.size() * sizeof(SimDesc<T>), bytes_ptr = rows * ns * sizeof(void*);
   const size_t bytes = bytes_desc + 2 * bytes_ptr + ns * sizeof(long long);
-  std::vector<unsigned char> host(bytes);
-  std::memcpy(host.data(), desc.data(), bytes_desc);
-  std::memcpy(host.data() + bytes_desc, src.data(), bytes_ptr);
-  std::memcpy(host.data() + bytes_desc + bytes_ptr, dst.data(), bytes_ptr);
-  std::memcpy(host.data() + bytes_desc + 2 * bytes_ptr, count.data(), ns * sizeof(long long));
+  cudaError_t e = h->ff_stage.reserve(bytes);
+  if (e != cudaSuccess) return cuda_fail(h, e, "feed_forward: staging");
+  unsigned char* host = static_cast<unsigned char*>(h->ff_stage.host);
+  std::memcpy(host, desc.data(), bytes_desc);
+  std::memcpy(host + bytes_desc, src.data(), bytes_ptr);
+  std::memcpy(host + bytes_desc + bytes_ptr, dst.data(), bytes_ptr);
+  std::memcpy(host + bytes_desc + 2 * bytes_ptr, count.data(), ns * sizeof(long long));
   unsigned char* dev = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&dev), bytes, s);
+  e = cudaMallocAsync(reinterpret_cast<void**>(&dev), bytes, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "feed_forward: tables");
-  e = cudaMemcpyAsync(dev, host.data(), bytes, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // host staging buffer is local
+  e = cudaMemcpyAsync(dev, host, bytes, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = h->ff_stage.uploaded(s);
   if (e != cudaSuccess) { cudaFreeAsync(dev, s); return cuda_fail(h, e, "feed_forward: tables"); }
   const SimDesc<T>* d_desc = reinterpret_cast<const SimDesc<T>*>(dev);
   const T* const* d_src = reinterpret_cast<const T* const*>(dev + bytes_desc);

@@ -23,6 +23,31 @@ unsigned long long* debug_trace_dev() {
 }
 #endif
 
+cudaError_t Staging::reserve(size_t bytes) {
+  cudaError_t e = cudaSuccess;
+  if (!done) e = cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
+  else e = cudaEventSynchronize(done);
+  if (e != cudaSuccess || bytes <= cap) return e;
+  if (host) cudaFreeHost(host);
+  host = nullptr;
+  cap = 0;
+  if ((e = cudaMallocHost(&host, bytes)) == cudaSuccess) cap = bytes;
+  return e;
+}
+
+void Staging::release() {
+  if (done) { cudaEventSynchronize(done); cudaEventDestroy(done); }
+  if (host) cudaFreeHost(host);
+  host = nullptr;
+  done = nullptr;
+  cap = 0;
+}
+
+bool being_captured(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
+}
+
 jf_status alloc_common(jf_ctx* h) {
   cudaError_t e;
 #ifdef JF_DEBUG_BOUNDS
@@ -61,6 +86,13 @@ void release_all(jf_ctx* h) {
   if (h->vjp_desc_done) cudaEventDestroy(h->vjp_desc_done);
   h->vjp_desc_host = h->vjp_desc_dev = nullptr;
   h->vjp_desc_done = nullptr;
+  h->ff_stage.release();
+  h->sweep_stage.release();
+  if (h->sweep_rows) cudaFree(h->sweep_rows);
+  h->sweep_rows = nullptr;
+  h->sweep_rows_cap = 0;
+  if (h->sweep_done) cudaEventDestroy(h->sweep_done);
+  h->sweep_done = nullptr;
   if (h->rec_store) cudaFree(h->rec_store);
   h->rec_store = nullptr;
   h->rec_cap = h->rec_limit = h->rec_used = 0;

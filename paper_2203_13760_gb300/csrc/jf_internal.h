@@ -29,6 +29,18 @@ struct GraphEntry {
   cudaGraphExec_t exec;
 };
 
+// Pinned host buffer of an asynchronous upload.  reserve() waits until the
+// last upload from it has run, so that its bytes may be rewritten; uploaded()
+// marks an upload on s.
+struct Staging {
+  void* host = nullptr;
+  size_t cap = 0;
+  cudaEvent_t done = nullptr;
+  cudaError_t reserve(size_t bytes);
+  cudaError_t uploaded(cudaStream_t s) { return cudaEventRecord(done, s); }
+  void release();
+};
+
 
 }  // namespace jf
 
@@ -76,6 +88,14 @@ struct jf_ctx {
   void* vjp_desc_host = nullptr;
   void* vjp_desc_dev = nullptr;
   cudaEvent_t vjp_desc_done = nullptr;
+  // pinned staging of the tables a call uploads (feed_forward; the reverse
+  // sweep), grown as needed, and the events after which it may be rewritten
+  jf::Staging ff_stage, sweep_stage;
+  // reverse sweep: device rows of descriptors, and the event recorded behind the
+  // last sweep (its workspaces may then be used on another stream)
+  void* sweep_rows = nullptr;
+  size_t sweep_rows_cap = 0;
+  cudaEvent_t sweep_done = nullptr;
   // deferred Rusanov-NN parameter gradient (jf_batch_param_grad_begin / end):
   // face records of the adjoint steps in between, summed in one launch
   void* rec_store = nullptr;
@@ -158,6 +178,11 @@ template <typename T>
 jf_status batch_general_vjp(jf_ctx* h, void* const* Un, const double* dt, void* const* lam_out, void* const* lam_in,
                             void* const* add, void* theta_bar, cudaStream_t s);
 // deferred parameter gradient of a batch (jf_batch_param_grad_begin / end)
+// the whole reverse sweep of a trajectory (jf_batch_feed_forward_vjp)
+template <typename T>
+jf_status batch_sweep(jf_ctx* h, void* const* traj, void* const* grad, int nsteps, const double* dt,
+                      void* const* lam0, void* theta_bar, cudaStream_t s);
+bool being_captured(cudaStream_t s);
 template <typename T>
 jf_status batch_param_grad_begin(jf_ctx* h, int max_steps);
 template <typename T>

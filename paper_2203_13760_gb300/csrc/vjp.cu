@@ -219,6 +219,40 @@ extern "C" jf_status jf_batch_step_vjp(jf_handle h, void* const* Un_ptrs, const 
                                          (cudaStream_t)stream);
 }
 
+extern "C" jf_status jf_batch_feed_forward_vjp(jf_handle h, void* const* traj_ptrs, void* const* grad_ptrs, int nsteps,
+                                               const double* dt_dev, void* const* lam0_ptrs, void* theta_bar,
+                                               void* stream) {
+  if (!h || h->kind != 1) { set_error(h, "jf_batch_feed_forward_vjp: not a batch handle"); return JF_ERR_ARG; }
+  if (!traj_ptrs || !grad_ptrs || !dt_dev || !lam0_ptrs || nsteps < 0) {
+    set_error(h, "jf_batch_feed_forward_vjp: null argument or nsteps < 0");
+    return JF_ERR_ARG;
+  }
+  for (int s = 0; s < h->nsim; ++s)
+    if (!traj_ptrs[s] || !grad_ptrs[s] || !lam0_ptrs[s] || !aligned16(traj_ptrs[s]) || !aligned16(grad_ptrs[s]) ||
+        !aligned16(lam0_ptrs[s]) || lam0_ptrs[s] == traj_ptrs[s] || lam0_ptrs[s] == grad_ptrs[s]) {
+      set_error(h, "jf_batch_feed_forward_vjp: every trajectory, cotangent and result must be a 16-byte aligned "
+                   "device array, the result distinct from the others");
+      return JF_ERR_ARG;
+    }
+  if (theta_bar && (h->scheme.flux != JF_FLUX_RUSANOV_NN || ((uintptr_t)theta_bar % h->esize) != 0)) {
+    set_error(h, "jf_batch_feed_forward_vjp: theta_bar needs the JF_FLUX_RUSANOV_NN flux (and element alignment)");
+    return JF_ERR_ARG;
+  }
+  if (h->rec_defer) {
+    set_error(h, "jf_batch_feed_forward_vjp: a jf_batch_param_grad_begin sweep is open");
+    return JF_ERR_ARG;
+  }
+  std::string why;
+  if (!general_vjp_supported(h, &why)) {
+    set_error(h, "jf_batch_feed_forward_vjp: " + why);
+    return JF_ERR_UNSUPPORTED;
+  }
+  return h->scheme.dtype == JF_F32
+             ? batch_sweep<float>(h, traj_ptrs, grad_ptrs, nsteps, dt_dev, lam0_ptrs, theta_bar, (cudaStream_t)stream)
+             : batch_sweep<double>(h, traj_ptrs, grad_ptrs, nsteps, dt_dev, lam0_ptrs, theta_bar,
+                                   (cudaStream_t)stream);
+}
+
 extern "C" jf_status jf_batch_param_grad_begin(jf_handle h, int max_steps) {
   if (!h || h->kind != 1) { set_error(h, "jf_batch_param_grad_begin: not a batch handle"); return JF_ERR_ARG; }
   if (h->scheme.flux != JF_FLUX_RUSANOV_NN || max_steps < 1) {

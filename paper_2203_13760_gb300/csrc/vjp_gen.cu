@@ -343,6 +343,104 @@ jf_status batch_general_vjp(jf_ctx* h, void* const* Un, const double* dt, void* 
   return JF_OK;
 }
 
+// The reverse sweep of a trajectory of nsteps steps: with lam^n = g^n,
+// lam^t = g^t + J_t^T lam^{t+1} for t = nsteps - 1 .. 0, lam^0 to lam0; the
+// parameter gradient of all steps is summed at the end.  The launches are
+// those of nsteps jf_batch_step_vjp calls; the descriptors of every step's
+// recompute are uploaded at once, so that the host runs ahead of the GPU.
+template <typename T>
+jf_status batch_sweep(jf_ctx* h, void* const* traj, void* const* grad, int nsteps, const double* dt,
+                      void* const* lam0, void* theta_bar, cudaStream_t s) {
+  const int ns = h->nsim, integ = h->scheme.integrator;
+  const char* who = "jf_batch_feed_forward_vjp";
+  if (being_captured(s)) { set_error(h, std::string(who) + ": the stream is being captured"); return JF_ERR_CUDA; }
+  std::vector<GVjpArgs<T>> geo(ns);
+  size_t cells = 0, faces = 0;
+  for (int k = 0; k < ns; ++k) {
+    geo[k] = grid_args<T>(h->grids[k], h->dim);
+    cells += (size_t)geo[k].N;
+    faces += (size_t)faces_of(geo[k]);
+  }
+  cudaError_t e = cudaSuccess;
+  if (!h->sweep_done) e = cudaEventCreateWithFlags(&h->sweep_done, cudaEventDisableTiming);
+  else e = cudaStreamWaitEvent(s, h->sweep_done, 0);  // the workspaces below may be in use on another stream
+  // l1, l2 of every grid, then the face records of a step (as batch_general_vjp); lam of two steps
+  if (e == cudaSuccess && !h->adj[0]) e = cudaMalloc(&h->adj[0], (10 * cells + 5 * faces) * sizeof(T));
+  if (e == cudaSuccess && !h->adj[1]) e = cudaMalloc(&h->adj[1], 10 * cells * sizeof(T));
+  if (e != cudaSuccess) return cuda_fail(h, e, who);
+  jf_status st;
+  if ((st = prepare_param_grad<T>(h, theta_bar)) != JF_OK) return st;
+  Gas<T> g = make_gas<T>(h->gas, h->scheme);
+  if ((st = network<T>(h, g)) != JF_OK) return st;
+  if (theta_bar && (st = batch_param_grad_begin<T>(h, nsteps > 0 ? nsteps : 1)) != JF_OK) return st;
+  h->rec_defer = false;  // the sweep fills the record store itself
+  int count = 0;
+  const StageVariant<T>& sv = stage_variants<T>(&count)[h->table_index];
+  const SimDesc<T>* desc = reinterpret_cast<const SimDesc<T>*>(h->host_desc.data());
+  auto slot = [&](void* const* base, int k, int t) { return static_cast<T*>(base[k]) + (size_t)t * 5 * geo[k].N; };
+  // descriptor rows of the recompute launches (FP32: the persistent kernel)
+  const bool rows = sizeof(T) == 4 && integ != JF_EULER && nsteps > 0;
+  if (rows) {
+    const size_t bytes = (size_t)nsteps * ns * sizeof(SimDesc<T>);
+    if ((e = h->sweep_stage.reserve(bytes)) != cudaSuccess) return cuda_fail(h, e, who);
+    if (bytes > h->sweep_rows_cap) {
+      if (h->sweep_rows) cudaFree(h->sweep_rows);
+      h->sweep_rows = nullptr;
+      h->sweep_rows_cap = 0;
+      if ((e = cudaMalloc(&h->sweep_rows, bytes)) != cudaSuccess) return cuda_fail(h, e, who);
+      h->sweep_rows_cap = bytes;
+    }
+    SimDesc<T>* row = static_cast<SimDesc<T>*>(h->sweep_stage.host);
+    for (int t = 0; t < nsteps; ++t)
+      for (int k = 0; k < ns; ++k) {
+        SimDesc<T>& d = row[(size_t)t * ns + k];
+        d = desc[k];
+        d.U = slot(traj, k, t);
+        d.dt = dt + k;
+      }
+    e = cudaMemcpyAsync(h->sweep_rows, row, bytes, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = h->sweep_stage.uploaded(s);
+    if (e != cudaSuccess) return cuda_fail(h, e, who);
+  }
+  const size_t rec_stage = 5 * faces, rec_step = step_stages(h) * rec_stage;
+  T* lbuf = static_cast<T*>(h->adj[0]);
+  std::vector<StepPtrs<T>> P(ns);
+  for (int t = nsteps - 1; t >= 0; --t) {
+    T* rbuf = theta_bar ? static_cast<T*>(h->rec_store) + (size_t)(nsteps - 1 - t) * rec_step : lbuf + 10 * cells;
+    T* lam = static_cast<T*>(h->adj[1]) + (t & 1 ? 5 * cells : 0);         // lam^t
+    T* next = static_cast<T*>(h->adj[1]) + (t & 1 ? 0 : 5 * cells);        // lam^{t+1}
+    size_t off = 0, roff = 0;
+    for (int k = 0; k < ns; ++k) {
+      const size_t n5 = 5 * (size_t)geo[k].N;
+      P[k] = StepPtrs<T>{slot(traj, k, t), t == nsteps - 1 ? slot(grad, k, nsteps) : next + off,
+                         t == 0 ? static_cast<T*>(lam0[k]) : lam + off, slot(grad, k, t), dt + k, desc[k].U1,
+                         desc[k].U2, lbuf + 2 * off, lbuf + 2 * off + n5, rbuf + roff};
+      off += n5;
+      roff += 5 * (size_t)faces_of(geo[k]);
+    }
+    if (rows) {
+      const SimDesc<T>* dev = static_cast<const SimDesc<T>*>(h->sweep_rows) + (size_t)t * ns;
+      e = sv.launch_batch(dev, static_cast<const WorkItem*>(h->d_work), h->nwork, 1, g, h->flag, h->batch_blocks,
+                          h->batch_rows, s);
+      if (e == cudaSuccess && integ == JF_RK3)
+        e = sv.launch_batch(dev, static_cast<const WorkItem*>(h->d_work), h->nwork, 2, g, h->flag, h->batch_blocks,
+                            h->batch_rows, s);
+      if (e != cudaSuccess) return cuda_fail(h, e, who);
+    } else if ((st = recompute_batch<T>(h, sv, g, P, s)) != JF_OK) {
+      return st;
+    }
+    if ((st = gvjp_chain<T>(h, g, geo, P, nullptr, theta_bar ? rec_stage : 0, s)) != JF_OK) return st;
+    if (theta_bar) h->rec_used += rec_step;
+  }
+  if (nsteps == 0)
+    for (int k = 0; k < ns && e == cudaSuccess; ++k)
+      e = cudaMemcpyAsync(lam0[k], grad[k], 5 * (size_t)geo[k].N * sizeof(T), cudaMemcpyDeviceToDevice, s);
+  if (e != cudaSuccess) return cuda_fail(h, e, who);
+  if (theta_bar && (st = batch_param_grad_end<T>(h, theta_bar, s)) != JF_OK) return st;
+  e = cudaEventRecord(h->sweep_done, s);
+  return e == cudaSuccess ? JF_OK : cuda_fail(h, e, who);
+}
+
 template <typename T>
 jf_status batch_param_grad_begin(jf_ctx* h, int max_steps) {
   size_t faces = 0;
@@ -386,6 +484,10 @@ template jf_status batch_general_vjp<float>(jf_ctx*, void* const*, const double*
                                             void* const*, void*, cudaStream_t);
 template jf_status batch_general_vjp<double>(jf_ctx*, void* const*, const double*, void* const*, void* const*,
                                              void* const*, void*, cudaStream_t);
+template jf_status batch_sweep<float>(jf_ctx*, void* const*, void* const*, int, const double*, void* const*, void*,
+                                      cudaStream_t);
+template jf_status batch_sweep<double>(jf_ctx*, void* const*, void* const*, int, const double*, void* const*, void*,
+                                       cudaStream_t);
 template jf_status batch_param_grad_begin<float>(jf_ctx*, int);
 template jf_status batch_param_grad_begin<double>(jf_ctx*, int);
 template jf_status batch_param_grad_end<float>(jf_ctx*, void*, cudaStream_t);

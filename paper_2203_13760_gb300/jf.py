@@ -73,6 +73,8 @@ SIGNATURES = {
     "jf_rk3_step_vjp_params": (_I, [_VP, _VP, _VP, _VP, _VP, _VP, _VP]),
     "jf_batch_step_vjp": (_I, [_VP, ctypes.POINTER(_VP), _VP, ctypes.POINTER(_VP), ctypes.POINTER(_VP),
                                ctypes.POINTER(_VP), _VP, _VP]),
+    "jf_batch_feed_forward_vjp": (_I, [_VP, ctypes.POINTER(_VP), ctypes.POINTER(_VP), _I, _VP, ctypes.POINTER(_VP),
+                                       _VP, _VP]),
     "jf_batch_param_grad_begin": (_I, [_VP, _I]),
     "jf_batch_param_grad_end": (_I, [_VP, _VP, _VP]),
     "jf_loss_density_l2": (_I, [_VP, _VP, _VP, _VP, _VP, _VP]),
@@ -437,17 +439,48 @@ class Batch:
         """Section 4.5 feed_forward: per simulation the trajectory tensor
         (nsteps + 1, 5, nz, ny, nx), slot 0 = U0, slot t = t steps of the fixed
         step dt (a float, or one value per simulation)."""
+        return self._feed_forward(U0s, nsteps, self._steps(dt))
+
+    def _steps(self, dt):
+        """The fixed steps (a float, or one value per simulation) as a float64
+        CUDA tensor, without waiting for the stream."""
         import torch
-        self._check_fields(U0s)
         dts = [float(dt)] * self.nsim if not hasattr(dt, "__len__") else [float(x) for x in dt]
         if len(dts) != self.nsim:
             raise ValueError("one dt per simulation")
-        dt_dev = torch.tensor(dts, dtype=torch.float64, device="cuda")
+        if all(x == dts[0] for x in dts):
+            return torch.full((self.nsim,), dts[0], dtype=torch.float64, device="cuda")
+        return torch.tensor(dts, dtype=torch.float64, pin_memory=True).to("cuda", non_blocking=True)
+
+    def _feed_forward(self, U0s, nsteps, dt_dev):
+        import torch
+        self._check_fields(U0s)
         trajs = [torch.empty((int(nsteps) + 1,) + tuple(U.shape), dtype=self.dtype, device="cuda") for U in U0s]
         u0 = (ctypes.c_void_p * self.nsim)(*[U.data_ptr() for U in U0s])
         tp = (ctypes.c_void_p * self.nsim)(*[T.data_ptr() for T in trajs])
         _check(lib().jf_batch_feed_forward(self.h, u0, tp, int(nsteps), _ptr(dt_dev), _stream()), self.h)
         return trajs
+
+    def feed_forward_vjp(self, trajs, grads, nsteps, dt, theta_bar=None):
+        """Reverse sweep of feed_forward (jf_batch_feed_forward_vjp): from the
+        trajectories and the cotangents of their slots (the same shapes) the
+        cotangents of the initial states; theta_bar (Rusanov-NN) is added to.
+        dt: a float64 CUDA tensor of one step per simulation."""
+        import torch
+        for ts in (trajs, grads):
+            if len(ts) != self.nsim:
+                raise ValueError("one trajectory per simulation")
+            for i, (t_, g) in enumerate(zip(ts, self.grids)):
+                if (not t_.is_cuda or t_.dtype != self.dtype or not t_.is_contiguous()
+                        or tuple(t_.shape) != (int(nsteps) + 1, 5, g.nz, g.ny, g.nx)):
+                    raise ValueError(f"trajectory {i} has the wrong shape / dtype / device")
+        if dt.dtype != torch.float64 or not dt.is_cuda or dt.numel() != self.nsim:
+            raise ValueError("dt must be a float64 CUDA tensor of one step per simulation")
+        lam0 = [torch.empty(tuple(t_.shape[1:]), dtype=self.dtype, device="cuda") for t_ in trajs]
+        arr = lambda ts: (ctypes.c_void_p * self.nsim)(*[x.data_ptr() for x in ts])  # noqa: E731
+        _check(lib().jf_batch_feed_forward_vjp(self.h, arr(trajs), arr(grads), int(nsteps), _ptr(dt), arr(lam0),
+                                               _ptr(theta_bar) if theta_bar is not None else None, _stream()), self.h)
+        return lam0
 
     def step_vjp(self, Uns, dt, lams, lam_ins=None, adds=None, theta_bar=None):
         """Adjoint of one fixed-dt step of every simulation (jf_batch_step_vjp):
