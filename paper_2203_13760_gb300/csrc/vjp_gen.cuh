@@ -95,9 +95,9 @@ __global__ void __launch_bounds__(256) gvjp_point_kernel(const GVjpBatch<T> B) {
 // Cotangent of W = (rho, u, v, w, p) -> cotangent of U = (rho, rho u, rho v,
 // rho w, E) for an ideal gas, p = (gamma - 1) (E - |m|^2 / (2 rho)).
 template <typename T>
-JF_HD void prim_vjp(const T U[5], const Gas<T>& g, const T Wb[5], T Ub[5]) {
-  const T ir = T(1) / U[0];
-  const T u = U[1] * ir, v = U[2] * ir, w = U[3] * ir;
+JF_HD void prim_vjp(const T W[5], const Gas<T>& g, const T Wb[5], T Ub[5]) {
+  const T ir = trcp(W[0]);
+  const T u = W[1], v = W[2], w = W[3];
   const T k = g.gm1;
   Ub[0] = Wb[0] - (Wb[1] * u + Wb[2] * v + Wb[3] * w) * ir + Wb[4] * k * T(0.5) * (u * u + v * v + w * w);
   Ub[1] = Wb[1] * ir - Wb[4] * k * u;
@@ -131,109 +131,180 @@ JF_HD void side_flux_vjp(const T W[5], const Gas<T>& g, const T Fb[5], const T U
   Wb[4] += pb;
 }
 
-// row[0 .. NN_HIDDEN) -> registers
+// NN_HIDDEN values in registers (a hidden layer's values or cotangents), FP32
+// as pairs for packed operations.
 template <typename T>
-__device__ __forceinline__ void ld_row(const T* row, T v[NN_HIDDEN]) {
+struct HRow {
+  T v[NN_HIDDEN];
+  __device__ __forceinline__ void fill(T x) {
 #pragma unroll
-  for (int j = 0; j < NN_HIDDEN; j += 4) ld4(row + j, v + j);
-}
-// sum_j w[j] v[j] with the weight row w read four at a time
-template <typename T>
-__device__ __forceinline__ T dot_row(const T* w, const T v[NN_HIDDEN], T acc) {
-#pragma unroll
-  for (int j = 0; j < NN_HIDDEN; j += 4) {
-    T q[4];
-    ld4(w + j, q);
-    acc += q[0] * v[j] + q[1] * v[j + 1] + q[2] * v[j + 2] + q[3] * v[j + 3];
+    for (int j = 0; j < NN_HIDDEN; ++j) v[j] = x;
   }
-  return acc;
-}
-// acc[j] += s w[j] over a weight row w
+  __device__ __forceinline__ void load(const T* row) {
+#pragma unroll
+    for (int j = 0; j < NN_HIDDEN; j += 4) ld4(row + j, v + j);
+  }
+  // += s w over a row w (16-byte aligned)
+  __device__ __forceinline__ void axpy(const T* w, T s) {
+#pragma unroll
+    for (int j = 0; j < NN_HIDDEN; j += 4) {
+      T q[4];
+      ld4(w + j, q);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) v[j + m] += s * q[m];
+    }
+  }
+  __device__ __forceinline__ T get(int j) const { return v[j]; }
+  __device__ __forceinline__ void set(int j, T x) { v[j] = x; }
+  __device__ __forceinline__ void store(T* row) const {
+#pragma unroll
+    for (int j = 0; j < NN_HIDDEN; ++j) row[j] = v[j];
+  }
+};
+template <>
+struct HRow<float> {
+  float2 v[NN_HIDDEN / 2];
+  __device__ __forceinline__ void fill(float x) {
+#pragma unroll
+    for (int j = 0; j < NN_HIDDEN / 2; ++j) v[j] = make_float2(x, x);
+  }
+  __device__ __forceinline__ void load(const float* row) {
+#pragma unroll
+    for (int j = 0; j < NN_HIDDEN; j += 4) {
+      const float4 q = *reinterpret_cast<const float4*>(row + j);
+      v[j / 2] = make_float2(q.x, q.y);
+      v[j / 2 + 1] = make_float2(q.z, q.w);
+    }
+  }
+  __device__ __forceinline__ void axpy(const float* w, float s) {
+    const float2 s2 = make_float2(s, s);
+#pragma unroll
+    for (int j = 0; j < NN_HIDDEN; j += 4) {
+      const float4 q = *reinterpret_cast<const float4*>(w + j);
+      v[j / 2] = __ffma2_rn(make_float2(q.x, q.y), s2, v[j / 2]);
+      v[j / 2 + 1] = __ffma2_rn(make_float2(q.z, q.w), s2, v[j / 2 + 1]);
+    }
+  }
+  __device__ __forceinline__ float get(int j) const { return j & 1 ? v[j / 2].y : v[j / 2].x; }
+  __device__ __forceinline__ void set(int j, float x) {
+    if (j & 1) v[j / 2].y = x;
+    else v[j / 2].x = x;
+  }
+  __device__ __forceinline__ void store(float* row) const {
+#pragma unroll
+    for (int j = 0; j < NN_HIDDEN; j += 4)
+      *reinterpret_cast<float4*>(row + j) =
+          make_float4(v[j / 2].x, v[j / 2].y, v[j / 2 + 1].x, v[j / 2 + 1].y);
+  }
+};
+
+// The network's parameters in shared memory for the adjoint kernels: the flat
+// layout (padded to a multiple of 4), then W1, W2 and W3 transposed (inputs by
+// outputs), so that every pass over a layer, forward or reverse, adds whole
+// rows to a row of register accumulators (HRow::axpy: 16-byte loads that all
+// lanes share, FP32 in packed operations).
+constexpr int kNnParamsPad = (NN_PARAMS + 3) / 4 * 4;
+constexpr int kNnW1 = 0, kNnB1 = kNnW1 + 4 * NN_HIDDEN, kNnW2 = kNnB1 + NN_HIDDEN,
+              kNnB2 = kNnW2 + NN_HIDDEN * NN_HIDDEN, kNnW3 = kNnB2 + NN_HIDDEN,
+              kNnB3 = kNnW3 + NN_HIDDEN * NN_HIDDEN, kNnW4 = kNnB3 + NN_HIDDEN, kNnB4 = kNnW4 + NN_HIDDEN;
+constexpr int kNnTRow = NN_HIDDEN + 4;  // row pitch of W2 and W3 transposed (fewer bank conflicts in nn_stage)
+constexpr int kNnT1 = kNnParamsPad, kNnT2 = kNnT1 + 4 * NN_HIDDEN, kNnT3 = kNnT2 + NN_HIDDEN * kNnTRow,
+              kNnShared = kNnT3 + NN_HIDDEN * kNnTRow;
 template <typename T>
-__device__ __forceinline__ void axpy_row(const T* w, T s, T acc[NN_HIDDEN]) {
-#pragma unroll
-  for (int j = 0; j < NN_HIDDEN; j += 4) {
-    T q[4];
-    ld4(w + j, q);
-#pragma unroll
-    for (int m = 0; m < 4; ++m) acc[j + m] += s * q[m];
+__device__ __forceinline__ void nn_stage(const T* __restrict__ theta, T* th) {
+  for (int i = threadIdx.x; i < NN_PARAMS; i += blockDim.x) th[i] = theta[i];
+  for (int i = threadIdx.x; i < 4 * NN_HIDDEN; i += blockDim.x)
+    th[kNnT1 + i % 4 * NN_HIDDEN + i / 4] = theta[kNnW1 + i];
+  for (int i = threadIdx.x; i < NN_HIDDEN * NN_HIDDEN; i += blockDim.x) {
+    const int t = i % NN_HIDDEN * kNnTRow + i / NN_HIDDEN;
+    th[kNnT2 + t] = theta[kNnW2 + i];
+    th[kNnT3 + t] = theta[kNnW3 + i];
   }
 }
 
-// Row pitch of the per-thread hidden rows (a multiple of 4 for the vector
-// loads; 36 puts the 16-byte accesses of 8 consecutive threads on distinct
-// banks).
+// Row pitch of the per-thread hidden rows in shared memory (a multiple of 4
+// for the vector accesses; 36 puts the 16-byte accesses of 8 consecutive
+// threads on distinct banks).
 constexpr int kHRow = NN_HIDDEN + 4;
 
-// alpha = exp(NN(x)) (as nn_alpha) and dx = d alpha / dx.  th: the
-// parameters in shared memory; h1, h2: this thread's two hidden rows (kHRow
-// pitch, shared memory).  Each layer's input is held in registers while its
-// outputs are formed one weight row at a time; the reverse passes run over
-// weight rows too (output cotangent times row added into register
-// accumulators), so every parameter is read as part of a 16-byte row load.
+// acc += sum_j h[j] W[j][:] over the rows of W (pitch PITCH), h (16-byte
+// aligned) read four at a time; a loop, so that the code of a network pass
+// stays small.
+template <int PITCH, typename T>
+__device__ __forceinline__ void nn_rows(const T* W, const T* h, HRow<T>& acc) {
+#pragma unroll 1
+  for (int j = 0; j < NN_HIDDEN; j += 4) {
+    T q[4];
+    ld4(h + j, q);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) acc.axpy(W + (j + m) * PITCH, q[m]);
+  }
+}
+
+// The hidden layers for input x: h1, h2 (this thread's rows, shared memory)
+// and the third layer's values in `h`; returns the network's output o
+// (alpha = exp(o)).
+template <typename T>
+__device__ __forceinline__ T nn_forward(const T* th, const T x[4], T* h1, T* h2, HRow<T>& h) {
+  auto relu = [&]() {
+#pragma unroll
+    for (int j = 0; j < NN_HIDDEN; ++j) h.set(j, tmax(T(0), h.get(j)));
+  };
+  h.load(th + kNnB1);
+#pragma unroll
+  for (int m = 0; m < 4; ++m) h.axpy(th + kNnT1 + m * NN_HIDDEN, x[m]);
+  relu();
+  h.store(h1);
+  h.load(th + kNnB2);
+  nn_rows<kNnTRow>(th + kNnT2, h1, h);
+  relu();
+  h.store(h2);
+  h.load(th + kNnB3);
+  nn_rows<kNnTRow>(th + kNnT3, h2, h);
+  relu();
+  T o = th[kNnB4];
+#pragma unroll
+  for (int j = 0; j < NN_HIDDEN; ++j) o += th[kNnW4 + j] * h.get(j);
+  return o;
+}
+
+// alpha = exp(NN(x)) (as nn_alpha) and dx = d alpha / dx.  h1, h2: this
+// thread's two hidden rows (kHRow pitch, shared memory).
 template <typename T>
 __device__ __forceinline__ T nn_alpha_grad(const T* th, const T x[4], T dx[4], T* h1, T* h2) {
-  const T* W1 = th;
-  const T* b1 = W1 + NN_HIDDEN * 4;
-  const T* W2 = b1 + NN_HIDDEN;
-  const T* b2 = W2 + NN_HIDDEN * NN_HIDDEN;
-  const T* W3 = b2 + NN_HIDDEN;
-  const T* b3 = W3 + NN_HIDDEN * NN_HIDDEN;
-  const T* W4 = b3 + NN_HIDDEN;
-  const T b4 = W4[NN_HIDDEN];
-  unsigned m1 = 0, m2 = 0, m3 = 0;  // ReLU masks (bit i: unit i active)
-  // layer 1 -> h1
-#pragma unroll 4
-  for (int i = 0; i < NN_HIDDEN; ++i) {
-    T w[4];
-    ld4(W1 + 4 * i, w);
-    const T z = b1[i] + w[0] * x[0] + w[1] * x[1] + w[2] * x[2] + w[3] * x[3];
-    h1[i] = tmax(T(0), z);
-    m1 |= (z > T(0) ? 1u : 0u) << i;
-  }
-  T v[NN_HIDDEN];
-  // layer 2 -> h2
-  ld_row(h1, v);
-#pragma unroll 2
-  for (int i = 0; i < NN_HIDDEN; ++i) {
-    const T z = dot_row(W2 + NN_HIDDEN * i, v, b2[i]);
-    h2[i] = tmax(T(0), z);
-    m2 |= (z > T(0) ? 1u : 0u) << i;
-  }
-  // layer 3 and the output
-  ld_row(h2, v);
-  T o = b4;
-#pragma unroll 2
-  for (int i = 0; i < NN_HIDDEN; ++i) {
-    const T z = dot_row(W3 + NN_HIDDEN * i, v, b3[i]);
-    o += W4[i] * tmax(T(0), z);
-    m3 |= (z > T(0) ? 1u : 0u) << i;
-  }
-  const T alpha = texp(o);
-  // reverse, seed d alpha / d o = alpha: cotangent of layer 2's outputs
-  // (v, then masked into h2) = sum over active layer-3 units i of
-  // alpha W4[i] W3[i][:]
+  HRow<T> h;
+  const T alpha = texp(nn_forward(th, x, h1, h2, h));
+  // reverse, seed d alpha / d o = alpha: each layer's cotangents masked by
+  // its activity and stored over the row of the layer above
+  unsigned m1 = 0, m2 = 0;
 #pragma unroll
-  for (int j = 0; j < NN_HIDDEN; ++j) v[j] = T(0);
-#pragma unroll 2
-  for (int i = 0; i < NN_HIDDEN; ++i)
-    if ((m3 >> i) & 1u) axpy_row(W3 + NN_HIDDEN * i, alpha * W4[i], v);
+  for (int j = 0; j < NN_HIDDEN; j += 4) {
+    T a[4], b[4];
+    ld4(h1 + j, a);
+    ld4(h2 + j, b);
 #pragma unroll
-  for (int j = 0; j < NN_HIDDEN; ++j) h2[j] = (m2 >> j) & 1u ? v[j] : T(0);
-  // cotangent of layer 1's outputs = sum_j h2[j] W2[j][:], masked
-#pragma unroll
-  for (int k = 0; k < NN_HIDDEN; ++k) v[k] = T(0);
-#pragma unroll 2
-  for (int j = 0; j < NN_HIDDEN; ++j) {
-    const T s = h2[j];
-    if (s != T(0)) axpy_row(W2 + NN_HIDDEN * j, s, v);
+    for (int m = 0; m < 4; ++m) {
+      m1 |= (a[m] > T(0) ? 1u : 0u) << (j + m);
+      m2 |= (b[m] > T(0) ? 1u : 0u) << (j + m);
+    }
   }
-  dx[0] = dx[1] = dx[2] = dx[3] = T(0);
+#pragma unroll
+  for (int j = 0; j < NN_HIDDEN; ++j) h.set(j, h.get(j) > T(0) ? alpha * th[kNnW4 + j] : T(0));
+  h.store(h2);
+  h.fill(T(0));
+  nn_rows<NN_HIDDEN>(th + kNnW3, h2, h);
+#pragma unroll
+  for (int j = 0; j < NN_HIDDEN; ++j) h.set(j, (m2 >> j) & 1u ? h.get(j) : T(0));
+  h.store(h1);
+  h.fill(T(0));
+  nn_rows<NN_HIDDEN>(th + kNnW2, h1, h);
+#pragma unroll
+  for (int m = 0; m < 4; ++m) dx[m] = T(0);
 #pragma unroll
   for (int k = 0; k < NN_HIDDEN; ++k) {
-    const T s = (m1 >> k) & 1u ? v[k] : T(0);
+    const T s = (m1 >> k) & 1u ? h.get(k) : T(0);
     T w[4];
-    ld4(W1 + 4 * k, w);
+    ld4(th + kNnW1 + 4 * k, w);
 #pragma unroll
     for (int m = 0; m < 4; ++m) dx[m] += w[m] * s;
   }
@@ -247,8 +318,10 @@ __device__ __forceinline__ void rusanov_nn_vjp(const T WL[5], const T WR[5], con
   T EL, ER, irL, irR, cL, cR;
   side_state(WL, g, EL, irL, cL);
   side_state(WR, g, ER, irR, cR);
-  T x[4], dx[4];
-  nn_inputs<T, D>(WL, WR, g, cL, cR, x);
+  // nn_inputs, with the entropy jump's sign kept
+  const T ds = ((tlog(WR[4]) - tlog(WL[4])) - g.gamma * (tlog(WR[0]) - tlog(WL[0]))) * g.inv_gm1;
+  const T x[4] = {fabs(WR[1 + D] - WL[1 + D]), T(0.5) * (WL[1 + D] + WR[1 + D]), T(0.5) * (cL + cR), fabs(ds)};
+  T dx[4];
   const T alpha = nn_alpha_grad(th, x, dx, h1, h2);
   T FL[5], FR[5], UL[5], UR[5];
   side_flux<T, D>(WL, EL, FL, UL);
@@ -276,19 +349,18 @@ __device__ __forceinline__ void rusanov_nn_vjp(const T WL[5], const T WR[5], con
   WRb[1 + D] += s0 * xb[0] + T(0.5) * xb[1];
   // mean sound speed, c = sqrt(gamma p / rho): dc/dp = c / (2 p), dc/drho = -c / (2 rho)
   const T cb = T(0.5) * xb[2];
-  WLb[4] += cb * cL / (T(2) * WL[4]);
-  WLb[0] -= cb * cL / (T(2) * WL[0]);
-  WRb[4] += cb * cR / (T(2) * WR[4]);
-  WRb[0] -= cb * cR / (T(2) * WR[0]);
-  // entropy jump, s = (ln p - gamma ln rho) / (gamma - 1)
-  const T sL = (tlog(WL[4]) - g.gamma * tlog(WL[0])) * g.inv_gm1;
-  const T sR = (tlog(WR[4]) - g.gamma * tlog(WR[0])) * g.inv_gm1;
-  const T s3 = sR - sL < T(0) ? T(-1) : T(1);
-  const T sbR = s3 * xb[3], sbL = -sbR;
-  WLb[4] += sbL * g.inv_gm1 / WL[4];
-  WLb[0] -= sbL * g.gamma * g.inv_gm1 / WL[0];
-  WRb[4] += sbR * g.inv_gm1 / WR[4];
-  WRb[0] -= sbR * g.gamma * g.inv_gm1 / WR[0];
+  const T ipL = trcp(WL[4]), ipR = trcp(WR[4]);
+  WLb[4] += T(0.5) * cb * cL * ipL;
+  WLb[0] -= T(0.5) * cb * cL * irL;
+  WRb[4] += T(0.5) * cb * cR * ipR;
+  WRb[0] -= T(0.5) * cb * cR * irR;
+  // entropy jump, s = (ln p - gamma ln rho) / (gamma - 1), with the sign that
+  // the inputs took it with
+  const T sb = (ds < T(0) ? T(-1) : T(1)) * xb[3] * g.inv_gm1;
+  WLb[4] -= sb * ipL;
+  WLb[0] += sb * g.gamma * irL;
+  WRb[4] += sb * ipR;
+  WRb[0] -= sb * g.gamma * irR;
 }
 
 // WENO3-JS reverse (left-biased value from vm1, v0, vp1): vb[k] += yb dy/dv_k.
@@ -297,9 +369,9 @@ JF_HD void weno3_vjp(T vm1, T v0, T vp1, T eps, T yb, T vb[3]) {
   const T q0 = T(0.5) * (T(3) * v0 - vm1), q1 = T(0.5) * (v0 + vp1);
   const T e0 = v0 - vm1, e1 = vp1 - v0;
   const T t0 = eps + e0 * e0, t1 = eps + e1 * e1;
-  const T r0 = T(1) / t0, r1 = T(1) / t1;
+  const T r0 = trcp(t0), r1 = trcp(t1);
   const T a0 = T(1.0 / 3.0) * r0 * r0, a1 = T(2.0 / 3.0) * r1 * r1;
-  const T inv = T(1) / (a0 + a1);
+  const T inv = trcp(a0 + a1);
   const T y = (a0 * q0 + a1 * q1) * inv;
   const T s = yb * inv;
   const T qb0 = s * a0, qb1 = s * a1;
@@ -313,109 +385,89 @@ JF_HD void weno3_vjp(T vm1, T v0, T vp1, T eps, T yb, T vb[3]) {
 
 // The reverse pass of one face normal to D whose right cell is c (the left
 // cell is c - e_D).  RECON: 0 WENO5-JS, 2 WENO3-JS; FLUX: 0 HLLC (Einfeldt
-// speeds), 4 Rusanov-NN.
-template <typename T, int DIM, int RECON, int FLUX, int D>
-__device__ __forceinline__ void gvjp_face(const GVjpArgs<T>& A, const Gas<T>& g, const int c[3], long long f,
+// speeds), 4 Rusanov-NN.  Worked in the face's frame (the components of a
+// cell in the order rho, normal, the two others, E), so that one copy of the
+// code serves every axis: the pass is executed once per thread, and with a
+// copy per axis the instruction fetch was its largest stall.
+template <typename T, int RECON, int FLUX>
+__device__ __forceinline__ void gvjp_face(const GVjpArgs<T>& A, const Gas<T>& g, int D, const int c[3], long long f,
                                           T* h1, T* h2) {
-  const int n = A.n[D];
+  const int n = D == 0 ? A.n[0] : (D == 1 ? A.n[1] : A.n[2]), cD = D == 0 ? c[0] : (D == 1 ? c[1] : c[2]);
+  const int per = D == 0 ? A.periodic[0] : (D == 1 ? A.periodic[1] : A.periodic[2]);
+  const int wall = D == 0 ? A.wall[0] : (D == 1 ? A.wall[1] : A.wall[2]);
   const long long sD = D == 0 ? 1 : (D == 1 ? (long long)A.n[0] : (long long)A.n[0] * A.n[1]);
-  long long base = 0;  // offset of the face's line (coordinate D = 0)
-  {
-    long long s = 1;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      if (a != D) base += (long long)c[a] * s;
-      s *= A.n[a];
-    }
-  }
+  // offset of the face's line (coordinate D = 0) and of the frame's components
+  const long long base = c[0] + (long long)A.n[0] * (c[1] + (long long)A.n[1] * c[2]) - cD * sD;
+  const long long comp[5] = {0, (1 + D) * A.N, (D == 0 ? 2 : 1) * A.N, (D == 2 ? 2 : 3) * A.N, 4 * A.N};
   // m of the two cells beside the face (a ghost has none)
-  const T scale = T(*A.dt) * A.inv_h[D];
+  const T scale = T(*A.dt) * (D == 0 ? A.inv_h[0] : (D == 1 ? A.inv_h[1] : A.inv_h[2])) * A.s_in;
   T Fb[5];
   {
-    int iL = c[D] - 1, iR = c[D];
-    bool hasL = true, hasR = true;
-    if (A.periodic[D]) {
-      if (iL < 0) iL += n;
-    } else {
-      hasL = iL >= 0;
-      hasR = iR < n;
-    }
+    int iL = cD - 1;
+    const bool hasL = per || iL >= 0, hasR = per || cD < n;
+    if (iL < 0 && per) iL += n;
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-      const T mL = hasL ? A.lam[base + iL * sD + q * A.N] : T(0);
-      const T mR = hasR ? A.lam[base + iR * sD + q * A.N] : T(0);
-      Fb[q] = scale * A.s_in * (mR - mL);
+      const T mL = hasL ? A.lam[base + iL * sD + comp[q]] : T(0);
+      const T mR = hasR ? A.lam[base + cD * sD + comp[q]] : T(0);
+      Fb[q] = scale * (mR - mL);
     }
   }
-  // stencil cells c[D] - 3 .. c[D] + 2 along D, through the boundary map
-  // (loaded twice: for the face states, and again for the reverse pass, so
-  // that the flux's reverse pass runs with few values live)
-  auto stencil = [&](int j, T Uj[5], T Wj[5], long long& at, bool& fl) {
-    fl = false;
-    const int i = map_index_bc(c[D] - 3 + j, n, A.periodic[D], A.wall[D], fl);
-    at = base + i * sD;
+  // primitives of the stencil cells c[D] - 3 .. c[D] + 2 along D, through the
+  // boundary map (slot 2 is the left cell, slot 3 the right one)
+  T W[6][5];
+  long long at[6];
+  bool flip[6];
 #pragma unroll
-    for (int q = 0; q < 5; ++q) Uj[q] = A.Us[at + q * A.N];
-    if (fl) Uj[1 + D] = -Uj[1 + D];
-    const T ir = T(1) / Uj[0];
-    Wj[0] = Uj[0];
-    Wj[1] = Uj[1] * ir;
-    Wj[2] = Uj[2] * ir;
-    Wj[3] = Uj[3] * ir;
-    Wj[4] = g.gm1 * (Uj[4] - T(0.5) * Uj[0] * (Wj[1] * Wj[1] + Wj[2] * Wj[2] + Wj[3] * Wj[3]));
-  };
-  // face states (stencil slot 2 is the left cell, slot 3 the right one)
+  for (int j = 0; j < 6; ++j) {
+    if (RECON == 2 && (j == 0 || j == 5)) continue;
+    at[j] = base + map_index_bc(cD - 3 + j, n, per, wall, flip[j]) * sD;
+    T* w = W[j];
+    const T r = A.Us[at[j]], ir = trcp(r);
+    w[0] = r;
+#pragma unroll
+    for (int q = 1; q < 4; ++q) w[q] = A.Us[at[j] + comp[q]] * ir;
+    if (flip[j]) w[1] = -w[1];
+    w[4] = g.gm1 * (A.Us[at[j] + comp[4]] - T(0.5) * r * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]));
+  }
+  // face states
   T WL[5], WR[5];
   bool fbL = false, fbR = false;  // safe-reconstruction fallback to the cell values
-  {
-    T W[6][5];
 #pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      T Uj[5];
-      long long at;
-      bool fl;
-      stencil(j, Uj, W[j], at, fl);
+  for (int q = 0; q < 5; ++q) {
+    if (RECON == 2) {
+      WL[q] = weno3(W[1][q], W[2][q], W[3][q], g.eps);
+      WR[q] = weno3(W[4][q], W[3][q], W[2][q], g.eps);
+    } else {
+      WL[q] = weno5(W[0][q], W[1][q], W[2][q], W[3][q], W[4][q], g.eps, 0);
+      WR[q] = weno5(W[5][q], W[4][q], W[3][q], W[2][q], W[1][q], g.eps, 0);
     }
+  }
+  if (g.safe) {
+    fbL = !(WL[0] > T(0)) || !(WL[4] > T(0));
+    fbR = !(WR[0] > T(0)) || !(WR[4] > T(0));
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-      if (RECON == 2) {
-        WL[q] = weno3(W[1][q], W[2][q], W[3][q], g.eps);
-        WR[q] = weno3(W[4][q], W[3][q], W[2][q], g.eps);
-      } else {
-        WL[q] = weno5(W[0][q], W[1][q], W[2][q], W[3][q], W[4][q], g.eps, 0);
-        WR[q] = weno5(W[5][q], W[4][q], W[3][q], W[2][q], W[1][q], g.eps, 0);
-      }
-    }
-    if (g.safe) {
-      fbL = !(WL[0] > T(0)) || !(WL[4] > T(0));
-      fbR = !(WR[0] > T(0)) || !(WR[4] > T(0));
-#pragma unroll
-      for (int q = 0; q < 5; ++q) {
-        if (fbL) WL[q] = W[2][q];
-        if (fbR) WR[q] = W[3][q];
-      }
+      if (fbL) WL[q] = W[2][q];
+      if (fbR) WR[q] = W[3][q];
     }
   }
   T WLb[5] = {T(0), T(0), T(0), T(0), T(0)}, WRb[5] = {T(0), T(0), T(0), T(0), T(0)};
   if constexpr (FLUX == 4) {
     T rec[5];
-    rusanov_nn_vjp<T, D>(WL, WR, g, g.nn, Fb, WLb, WRb, rec, h1, h2);
+    rusanov_nn_vjp<T, 0>(WL, WR, g, g.nn, Fb, WLb, WRb, rec, h1, h2);
     if (A.rec)
 #pragma unroll
       for (int m = 0; m < 5; ++m) A.rec[f * 5 + m] = rec[m];
   } else {
-    hllc_vjp<T, D>(WL, WR, g, Fb, WLb, WRb);
+    hllc_vjp<T, 0>(WL, WR, g, Fb, WLb, WRb);
   }
   // reconstruction reverse
-  T W[6][5], U[6][5], Wb[6][5];
-  long long at[6];
-  bool flip[6];
+  T Wb[6][5];
 #pragma unroll
-  for (int j = 0; j < 6; ++j) {
-    stencil(j, U[j], W[j], at[j], flip[j]);
+  for (int j = 0; j < 6; ++j)
 #pragma unroll
     for (int q = 0; q < 5; ++q) Wb[j][q] = T(0);
-  }
 #pragma unroll
   for (int q = 0; q < 5; ++q) {
     if (fbL) {
@@ -448,34 +500,34 @@ __device__ __forceinline__ void gvjp_face(const GVjpArgs<T>& A, const Gas<T>& g,
   for (int j = 0; j < 6; ++j) {
     if (RECON == 2 && (j == 0 || j == 5)) continue;
     T Ub[5];
-    prim_vjp(U[j], g, Wb[j], Ub);
-    if (flip[j]) Ub[1 + D] = -Ub[1 + D];
+    prim_vjp(W[j], g, Wb[j], Ub);
+    if (flip[j]) Ub[1] = -Ub[1];
 #pragma unroll
-    for (int q = 0; q < 5; ++q) atomicAdd(A.out + at[j] + q * A.N, Ub[q]);
+    for (int q = 0; q < 5; ++q) atomicAdd(A.out + at[j] + comp[q], Ub[q]);
   }
 }
 
 // One thread per face of every grid of the launch: within a grid, faces of
 // direction 0 first, then 1, then 2; within a direction x fastest.  A periodic axis has n faces (face 0 is also face n),
 // any other n + 1.  Rusanov-NN: dynamic shared memory of
-// gvjp_face_smem_bytes holds the network parameters (padded to a multiple
-// of 4) and each thread's two hidden-layer rows.
-constexpr int kGvjpThreads = 128;
-constexpr int kNnParamsPad = (NN_PARAMS + 3) / 4 * 4;
+// gvjp_face_smem_bytes holds the network parameters (nn_stage) and each
+// thread's two hidden-layer rows.  Small CTAs spread a training batch's faces
+// (42,240 for 20 grids of 32^2) evenly over the SMs.
+constexpr int kGvjpThreads = 64;
 template <typename T, int FLUX>
 constexpr size_t gvjp_face_smem_bytes() {
-  return FLUX == 4 ? sizeof(T) * ((size_t)kNnParamsPad + (size_t)kGvjpThreads * 2 * kHRow) : 0;
+  return FLUX == 4 ? sizeof(T) * ((size_t)kNnShared + (size_t)kGvjpThreads * 2 * kHRow) : 0;
 }
 
 template <typename T, int DIM, int RECON, int FLUX>
-__global__ void __launch_bounds__(kGvjpThreads) gvjp_face_kernel(const GVjpBatch<T> B, const Gas<T> g) {
+__global__ void __launch_bounds__(kGvjpThreads, sizeof(T) == 4 ? 5 : 1) gvjp_face_kernel(const GVjpBatch<T> B, const Gas<T> g) {
   extern __shared__ __align__(16) unsigned char gvjp_smem[];
   T* th = reinterpret_cast<T*>(gvjp_smem);  // the network parameters (Rusanov-NN)
-  T* h1 = th + kNnParamsPad + threadIdx.x * kHRow;
+  T* h1 = th + kNnShared + threadIdx.x * kHRow;
   T* h2 = h1 + kGvjpThreads * kHRow;
   Gas<T> gs = g;
   if constexpr (FLUX == 4) {
-    for (int i = threadIdx.x; i < NN_PARAMS; i += blockDim.x) th[i] = g.nn[i];
+    nn_stage(g.nn, th);
     __syncthreads();
     gs.nn = th;
   }
@@ -498,9 +550,7 @@ __global__ void __launch_bounds__(kGvjpThreads) gvjp_face_kernel(const GVjpBatch
   r /= ext[0];
   c[1] = (int)(r % ext[1]);
   c[2] = (int)(r / ext[1]);
-  if (d == 0) gvjp_face<T, DIM, RECON, FLUX, 0>(A, gs, c, f, h1, h2);
-  if constexpr (DIM >= 2) if (d == 1) gvjp_face<T, DIM, RECON, FLUX, 1>(A, gs, c, f, h1, h2);
-  if constexpr (DIM == 3) if (d == 2) gvjp_face<T, DIM, RECON, FLUX, 2>(A, gs, c, f, h1, h2);
+  gvjp_face<T, RECON, FLUX>(A, gs, d, c, f, h1, h2);
 }
 
 // Parameter gradient of the Rusanov-NN dissipation: grad += sum over the
@@ -509,53 +559,49 @@ __global__ void __launch_bounds__(kGvjpThreads) gvjp_face_kernel(const GVjpBatch
 // Persistent blocks of kNnWarps warps; the block stages theta in shared
 // memory, and each warp takes chunks of 32 records (one per lane).  Per
 // chunk, each lane evaluates the network of its record and the cotangents of
-// every layer (seed d alpha / d o = alpha, scaled by abar) into shared rows of
-// 33 (conflict-free), reusing rows once they are consumed; then lane L adds
-// row L of every weight gradient summed over the 32 records
-// (dW[L][k] = sum_f G[f][L] H[f][k]) to accumulators kept in registers across
-// chunks.  At the end the block sums its warps' accumulators in shared memory
-// and adds them to grad with one atomic per parameter.
-constexpr int kNnRow = NN_HIDDEN + 1;
-constexpr int kNnWarps = 4;
-constexpr int kNnWarpElems = 4 * 32 * kNnRow + 32 * 5;  // four row sets, inputs, output cotangents
+// every layer (seed d alpha / d o = alpha, scaled by abar) into shared rows,
+// reusing rows once they are consumed; then lane L adds row L of every weight
+// gradient summed over the 32 records (dW[L][k] = sum_f G[f][L] H[f][k]) to
+// accumulators kept in registers across chunks.  At the end the block sums its
+// warps' accumulators in shared memory and adds them to grad with one atomic
+// per parameter.
+//
+// Bound by the FMA pipe and the shared-memory loads (about 6400 FMA per
+// record).  Whole rows in 16-byte loads (pitch 36) and packed FMA: @@
+constexpr int kNnWarps = 6;  // two blocks per SM by shared memory (FP32)
+constexpr int kNnWarpElems = 3 * 32 * kHRow + 32 * 5;  // three row sets, inputs, output cotangents
 template <typename T>
 constexpr size_t nn_grad_smem_bytes() {
-  return sizeof(T) * (size_t)(NN_PARAMS + kNnWarps * kNnWarpElems);
+  return sizeof(T) * (size_t)(kNnShared + kNnWarps * kNnWarpElems);
 }
+static_assert(kNnWarpElems >= NN_PARAMS, "the warps' row sets hold their sums at the end");
 
 template <typename T>
-__global__ void __launch_bounds__(32 * kNnWarps) nn_param_grad_kernel(const T* __restrict__ theta,
+__global__ void __launch_bounds__(32 * kNnWarps, sizeof(T) == 4 ? 2 : 1) nn_param_grad_kernel(const T* __restrict__ theta,
                                                                       const T* __restrict__ rec, long long nrec,
                                                                       T* grad) {
   extern __shared__ __align__(16) unsigned char nn_smem[];
   T* TH = reinterpret_cast<T*>(nn_smem);
-  for (int i = threadIdx.x; i < NN_PARAMS; i += blockDim.x) TH[i] = theta[i];
+  nn_stage(theta, TH);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  T* base = TH + NN_PARAMS + warp * kNnWarpElems;
+  T* base = TH + kNnShared + warp * kNnWarpElems;
   T* R1 = base;                 // H1
-  T* R2 = R1 + 32 * kNnRow;     // H2
-  T* R3 = R2 + 32 * kNnRow;     // H3, then G2
-  T* R4 = R3 + 32 * kNnRow;     // G3, then G1
-  T* X = R4 + 32 * kNnRow;      // [32][4]
+  T* R2 = R1 + 32 * kHRow;      // H2
+  T* R3 = R2 + 32 * kHRow;      // H3, then G2, then G1
+  T* X = R3 + 32 * kHRow;       // [32][4]
   T* OB = X + 32 * 4;           // [32]
-  const T* W1 = TH;
-  const T* b1 = W1 + NN_HIDDEN * 4;
-  const T* W2 = b1 + NN_HIDDEN;
-  const T* b2 = W2 + NN_HIDDEN * NN_HIDDEN;
-  const T* W3 = b2 + NN_HIDDEN;
-  const T* b3 = W3 + NN_HIDDEN * NN_HIDDEN;
-  const T* W4 = b3 + NN_HIDDEN;
   __syncthreads();
   // row `lane` of every gradient, accumulated over this warp's chunks
-  T a3[NN_HIDDEN], a2[NN_HIDDEN], a1[4] = {T(0), T(0), T(0), T(0)};
-#pragma unroll
-  for (int k = 0; k < NN_HIDDEN; ++k) a3[k] = a2[k] = T(0);
+  HRow<T> a3, a2;
+  T a1[4] = {T(0), T(0), T(0), T(0)};
+  a3.fill(T(0));
+  a2.fill(T(0));
   T ab1 = T(0), ab2 = T(0), ab3 = T(0), a4 = T(0), ab4 = T(0);
+  const T w4 = TH[kNnW4 + lane];
   const long long nchunk = (nrec + 31) / 32;
-  T* h1 = R1 + lane * kNnRow;
-  T* h2 = R2 + lane * kNnRow;
-  T* r3 = R3 + lane * kNnRow;
-  T* r4 = R4 + lane * kNnRow;
+  T* h1 = R1 + lane * kHRow;
+  T* h2 = R2 + lane * kHRow;
+  T* r3 = R3 + lane * kHRow;
   for (long long ch = (long long)blockIdx.x * kNnWarps + warp; ch < nchunk; ch += (long long)gridDim.x * kNnWarps) {
     const long long f = ch * 32 + lane;
     T x[4] = {T(0), T(0), T(0), T(0)}, abar = T(0);
@@ -566,104 +612,91 @@ __global__ void __launch_bounds__(32 * kNnWarps) nn_param_grad_kernel(const T* _
     }
 #pragma unroll
     for (int m = 0; m < 4; ++m) X[lane * 4 + m] = x[m];
-    // forward: h1, h2, h3 (r3); each layer's input in registers (v), the
-    // weight rows read four at a time from the shared copy of theta
-    T v[NN_HIDDEN];
-#pragma unroll 4
-    for (int i = 0; i < NN_HIDDEN; ++i) {
-      T w[4];
-      ld4(W1 + 4 * i, w);
-      h1[i] = tmax(T(0), b1[i] + w[0] * x[0] + w[1] * x[1] + w[2] * x[2] + w[3] * x[3]);
-    }
-#pragma unroll
-    for (int j = 0; j < NN_HIDDEN; ++j) v[j] = h1[j];
-#pragma unroll 2
-    for (int i = 0; i < NN_HIDDEN; ++i) h2[i] = tmax(T(0), dot_row(W2 + NN_HIDDEN * i, v, b2[i]));
-#pragma unroll
-    for (int j = 0; j < NN_HIDDEN; ++j) v[j] = h2[j];
-    T o = W4[NN_HIDDEN];
-#pragma unroll 2
-    for (int i = 0; i < NN_HIDDEN; ++i) {
-      const T h3 = tmax(T(0), dot_row(W3 + NN_HIDDEN * i, v, b3[i]));
-      r3[i] = h3;
-      o += W4[i] * h3;
-    }
+    HRow<T> v;
+    const T o = nn_forward(TH, x, h1, h2, v);
     const T ob = f < nrec ? abar * texp(o) : T(0);  // d alpha / d o = alpha
     OB[lane] = ob;
-#pragma unroll 4
-    for (int i = 0; i < NN_HIDDEN; ++i) r4[i] = r3[i] > T(0) ? ob * W4[i] : T(0);  // G3
+    v.store(r3);
     __syncwarp();
-    // layers 4 and 3 (H3 in R3, G3 in R4, H2 in R2)
-#pragma unroll 1
+    // layers 4 and 3 (H3 in R3, H2 in R2): G3 = OB W4 where H3 > 0
+#pragma unroll 2
     for (int r = 0; r < 32; ++r) {
-      const T g3 = R4[r * kNnRow + lane];
+      const T h3 = R3[r * kHRow + lane], b = OB[r];
+      const T g3 = h3 > T(0) ? b * w4 : T(0);
       ab3 += g3;
-      a4 += OB[r] * R3[r * kNnRow + lane];
-      if (lane == 0) ab4 += OB[r];
-#pragma unroll
-      for (int k = 0; k < NN_HIDDEN; ++k) a3[k] += g3 * R2[r * kNnRow + k];
+      a4 += b * h3;
+      ab4 += b;
+      a3.axpy(R2 + r * kHRow, g3);
     }
     __syncwarp();
-    // G2 into R3: g2[j] = [h2_j > 0] sum_i W3[i][j] g3[i] (row updates of v)
+    // G2 into R3: g2[j] = [h2_j > 0] sum_i W3[i][j] g3[i]; g3 over the lane's own H3 row first
 #pragma unroll
-    for (int j = 0; j < NN_HIDDEN; ++j) v[j] = T(0);
-#pragma unroll 2
-    for (int i = 0; i < NN_HIDDEN; ++i) axpy_row(W3 + NN_HIDDEN * i, r4[i], v);
+    for (int j = 0; j < NN_HIDDEN; ++j) v.set(j, v.get(j) > T(0) ? ob * TH[kNnW4 + j] : T(0));
+    v.store(r3);
+    v.fill(T(0));
+    nn_rows<NN_HIDDEN>(TH + kNnW3, r3, v);
 #pragma unroll
-    for (int j = 0; j < NN_HIDDEN; ++j) r3[j] = h2[j] > T(0) ? v[j] : T(0);
+    for (int j = 0; j < NN_HIDDEN; j += 4) {
+      T q[4];
+      ld4(h2 + j, q);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) v.set(j + m, q[m] > T(0) ? v.get(j + m) : T(0));
+    }
+    v.store(r3);
     __syncwarp();
     // layer 2 (G2 in R3, H1 in R1)
-#pragma unroll 1
+#pragma unroll 2
     for (int r = 0; r < 32; ++r) {
-      const T g2 = R3[r * kNnRow + lane];
+      const T g2 = R3[r * kHRow + lane];
       ab2 += g2;
-#pragma unroll
-      for (int k = 0; k < NN_HIDDEN; ++k) a2[k] += g2 * R1[r * kNnRow + k];
+      a2.axpy(R1 + r * kHRow, g2);
     }
     __syncwarp();
-    // G1 into R4: g1[k] = [h1_k > 0] sum_j W2[j][k] g2[j] (row updates of v)
+    // G1 into R3: g1[k] = [h1_k > 0] sum_j W2[j][k] g2[j]
+    v.fill(T(0));
+    nn_rows<NN_HIDDEN>(TH + kNnW2, r3, v);
 #pragma unroll
-    for (int k = 0; k < NN_HIDDEN; ++k) v[k] = T(0);
-#pragma unroll 2
-    for (int j = 0; j < NN_HIDDEN; ++j) axpy_row(W2 + NN_HIDDEN * j, r3[j], v);
+    for (int j = 0; j < NN_HIDDEN; j += 4) {
+      T q[4];
+      ld4(h1 + j, q);
 #pragma unroll
-    for (int k = 0; k < NN_HIDDEN; ++k) r4[k] = h1[k] > T(0) ? v[k] : T(0);
+      for (int m = 0; m < 4; ++m) v.set(j + m, q[m] > T(0) ? v.get(j + m) : T(0));
+    }
     __syncwarp();
-    // layer 1 (G1 in R4, inputs in X)
-#pragma unroll 1
+    v.store(r3);
+    __syncwarp();
+    // layer 1 (G1 in R3, inputs in X)
+#pragma unroll 2
     for (int r = 0; r < 32; ++r) {
-      const T g1 = R4[r * kNnRow + lane];
+      const T g1 = R3[r * kHRow + lane];
       ab1 += g1;
+      T q[4];
+      ld4(X + r * 4, q);
 #pragma unroll
-      for (int m = 0; m < 4; ++m) a1[m] += g1 * X[r * 4 + m];
+      for (int m = 0; m < 4; ++m) a1[m] += g1 * q[m];
     }
     __syncwarp();
   }
   // block sum of the warps' rows (the row sets are free now), then one
   // atomic per parameter
   __syncthreads();
-  T* S = TH + NN_PARAMS;  // [kNnWarps][NN_PARAMS]
-  T* Sw = S + warp * NN_PARAMS;
+  T* S = TH + kNnShared;  // [kNnWarps][kNnWarpElems]
+  T* Sw = S + warp * kNnWarpElems;
   const int L = lane;
 #pragma unroll
-  for (int m = 0; m < 4; ++m) Sw[4 * L + m] = a1[m];
-  Sw[NN_HIDDEN * 4 + L] = ab1;
-  T* sW2 = Sw + NN_HIDDEN * 4 + NN_HIDDEN;
-#pragma unroll
-  for (int k = 0; k < NN_HIDDEN; ++k) sW2[NN_HIDDEN * L + k] = a2[k];
-  sW2[NN_HIDDEN * NN_HIDDEN + L] = ab2;
-  T* sW3 = sW2 + NN_HIDDEN * NN_HIDDEN + NN_HIDDEN;
-#pragma unroll
-  for (int k = 0; k < NN_HIDDEN; ++k) sW3[NN_HIDDEN * L + k] = a3[k];
-  sW3[NN_HIDDEN * NN_HIDDEN + L] = ab3;
-  T* sW4 = sW3 + NN_HIDDEN * NN_HIDDEN + NN_HIDDEN;
-  sW4[L] = a4;
-  if (L == 0) sW4[NN_HIDDEN] = ab4;
+  for (int m = 0; m < 4; ++m) Sw[kNnW1 + 4 * L + m] = a1[m];
+  Sw[kNnB1 + L] = ab1;
+  a2.store(Sw + kNnW2 + NN_HIDDEN * L);
+  Sw[kNnB2 + L] = ab2;
+  a3.store(Sw + kNnW3 + NN_HIDDEN * L);
+  Sw[kNnB3 + L] = ab3;
+  Sw[kNnW4 + L] = a4;
+  if (L == 0) Sw[kNnB4] = ab4;
   __syncthreads();
   for (int i = threadIdx.x; i < NN_PARAMS; i += blockDim.x) {
     T sum = T(0);
 #pragma unroll
-    for (int w = 0; w < kNnWarps; ++w) sum += S[w * NN_PARAMS + i];
+    for (int w = 0; w < kNnWarps; ++w) sum += S[w * kNnWarpElems + i];
     if (sum != T(0)) atomicAdd(grad + i, sum);
   }
 }
