@@ -495,6 +495,11 @@ JF_HD void signal_speeds(const T WL[5], const T WR[5], const Gas<T>& g, int spee
   }
 }
 
+template <typename T>
+JF_HD T total_energy(const T W[5], const Gas<T>& g) {
+  return W[4] * g.inv_gm1 + T(0.5) * W[0] * (W[1] * W[1] + W[2] * W[2] + W[3] * W[3]);
+}
+
 // Total energy, 1/rho and sound speed of one side.
 template <typename T>
 JF_HD void side_state(const T W[5], const Gas<T>& g, T& E, T& ir, T& c) {
@@ -782,6 +787,72 @@ __host__ __device__ __noinline__ T nn_alpha(const T* th, const T x[4]) {
   return texp(out);
 }
 
+#ifdef __CUDACC__
+// nn_alpha of two faces in packed FP32x2 lanes, from the parameters stored
+// twice each (th2[k] = (theta_k, theta_k), 16-byte aligned): per lane the
+// operations of nn_alpha in its order, so the same bits.  A layer runs over its
+// inputs four at a time (from `row`, this thread's NN_PAIR_ROW pairs of shared
+// memory) with all its outputs in registers: independent sums, and a loop whose
+// code stays in the instruction cache (unrolled over both layers the pass was
+// bound by instruction fetch).
+constexpr int NN_PAIR_ROW = NN_HIDDEN + 2;  // 17 x 16 bytes: conflict-free 16-byte accesses
+static __device__ __noinline__ float2 nn_alpha_pair(const float2* th2, const float2 x[4], float2* row) {
+  const float2* b1 = th2 + NN_HIDDEN * 4;
+  const float2* W2 = b1 + NN_HIDDEN;
+  const float2* b2 = W2 + NN_HIDDEN * NN_HIDDEN;
+  const float2* W3 = b2 + NN_HIDDEN;
+  const float2* b3 = W3 + NN_HIDDEN * NN_HIDDEN;
+  const float2* W4 = b3 + NN_HIDDEN;
+  auto ld2 = [](const float2* p, float2& a, float2& b) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    a = make_float2(q.x, q.y);
+    b = make_float2(q.z, q.w);
+  };
+  auto relu = [](float2 z) { return make_float2(tmax(0.0f, z.x), tmax(0.0f, z.y)); };
+  float2 z[NN_HIDDEN];
+  auto keep = [&]() {  // the layer's values to this thread's row
+#pragma unroll
+    for (int i = 0; i < NN_HIDDEN; i += 2) {
+      const float2 a = relu(z[i]), b = relu(z[i + 1]);
+      *reinterpret_cast<float4*>(row + i) = make_float4(a.x, a.y, b.x, b.y);
+    }
+  };
+  auto layer = [&](const float2* W, const float2* b) {
+#pragma unroll
+    for (int i = 0; i < NN_HIDDEN; i += 2) ld2(b + i, z[i], z[i + 1]);
+#pragma unroll 1
+    for (int j = 0; j < NN_HIDDEN; j += 4) {
+      float2 h0, h1, h2, h3;
+      ld2(row + j, h0, h1);
+      ld2(row + j + 2, h2, h3);
+#pragma unroll
+      for (int i = 0; i < NN_HIDDEN; ++i) {
+        float2 w0, w1, w2, w3;
+        ld2(W + NN_HIDDEN * i + j, w0, w1);
+        ld2(W + NN_HIDDEN * i + j + 2, w2, w3);
+        const float2 t = __ffma2_rn(w3, h3, __ffma2_rn(w2, h2, __ffma2_rn(w0, h0, __fmul2_rn(w1, h1))));
+        z[i] = __fadd2_rn(z[i], t);
+      }
+    }
+  };
+#pragma unroll
+  for (int i = 0; i < NN_HIDDEN; ++i) {
+    float2 w0, w1, w2, w3;
+    ld2(th2 + 4 * i, w0, w1);
+    ld2(th2 + 4 * i + 2, w2, w3);
+    z[i] = __ffma2_rn(w3, x[3], __ffma2_rn(w2, x[2], __ffma2_rn(w1, x[1], __ffma2_rn(w0, x[0], b1[i]))));
+  }
+  keep();
+  layer(W2, b2);
+  keep();
+  layer(W3, b3);
+  float2 out = W4[NN_HIDDEN];
+#pragma unroll
+  for (int i = 0; i < NN_HIDDEN; ++i) out = __ffma2_rn(W4[i], relu(z[i]), out);
+  return make_float2(texp(out.x), texp(out.y));
+}
+#endif
+
 // Network inputs of the Rusanov-NN flux at a face along D (Section 7.4):
 // |u_R - u_L|, (u_L + u_R)/2, (c_L + c_R)/2, |s_R - s_L| with u the normal
 // velocity and s = ln(p / rho^gamma) / (gamma - 1).
@@ -798,17 +869,27 @@ JF_HD void nn_inputs(const T WL[5], const T WR[5], const Gas<T>& g, T cL, T cR, 
 // Rusanov-NN (Section 7.4, Eq. (Rusanov)): F = (F_L + F_R)/2 - alpha (U_R - U_L)/2
 // with alpha = exp(NN(x)).
 template <typename T, int D>
-JF_HD void rusanov_nn(const T WL[5], const T WR[5], const Gas<T>& g, T F[5]) {
-  T EL, ER, irL, irR, q, cL, cR;
-  side_states(WL, WR, g, EL, ER, irL, irR, q, cL, cR);
-  T x[4];
-  nn_inputs<T, D>(WL, WR, g, cL, cR, x);
-  const T a = nn_alpha(g.nn, x);
+JF_HD void rusanov_nn(const T WL[5], const T WR[5], const Gas<T>& g, T F[5], T a) {
+  const T EL = total_energy(WL, g), ER = total_energy(WR, g);
   T FL[5], FR[5], UL[5], UR[5];
   side_flux<T, D>(WL, EL, FL, UL);
   side_flux<T, D>(WR, ER, FR, UR);
 #pragma unroll
   for (int q = 0; q < 5; ++q) F[q] = T(0.5) * (FL[q] + FR[q]) - T(0.5) * a * (UR[q] - UL[q]);
+}
+
+// The network's inputs of a face from its states.
+template <typename T, int D>
+JF_HD void nn_face_inputs(const T WL[5], const T WR[5], const Gas<T>& g, T x[4]) {
+  T EL, ER, irL, irR, q, cL, cR;
+  side_states(WL, WR, g, EL, ER, irL, irR, q, cL, cR);
+  nn_inputs<T, D>(WL, WR, g, cL, cR, x);
+}
+template <typename T, int D>
+JF_HD void rusanov_nn(const T WL[5], const T WR[5], const Gas<T>& g, T F[5]) {
+  T x[4];
+  nn_face_inputs<T, D>(WL, WR, g, x);
+  rusanov_nn<T, D>(WL, WR, g, F, nn_alpha(g.nn, x));
 }
 
 // The Riemann solver and signal speeds of the configuration (uniform branch;

@@ -40,6 +40,11 @@
 namespace jf {
 
 constexpr int HALO = 3;
+// Rusanov-NN parameters in shared memory (nn_smem_elems)
+constexpr int kNnPairs = (NN_PARAMS + 3) / 4 * 4, kNnRows = kNnPairs + (2 * NN_PARAMS + 3) / 4 * 4;
+#ifndef __CUDACC__
+constexpr int NN_PAIR_ROW = 0;
+#endif
 
 // Kernel dimensionality (template parameter DIM).  1, 2 and 3 are the grid's
 // active axes: the tile spans x (1D: one row of BX cells; 2D, 3D: BX x BY
@@ -425,12 +430,11 @@ __device__ __forceinline__ void fs_flux(const Val& val, const Gas<T>& g, int rec
   F[4] = H * (Gh[0] + Gh[4]) + un * c * Dw + T(0.5) * q2 * Gh[1] + u[T1] * Gh[2] + u[T2] * Gh[3];
 }
 
-// Convective flux F of a Godunov-type face from its reconstructed states Wm
-// (left) and Wp (right): the safe-reconstruction fallback, then the Riemann
-// solver of the kernel family.
-template <typename T, int D, int BX, int BY, int DIM, bool VISC, int SCH>
-__device__ __forceinline__ void face_riemann(const RingView<T, BX, BY, DIM, VISC>& R, int x0, int y0,
-                                             const Gas<T>& g, T Wm[5], T Wp[5], T F[5]) {
+// Safe reconstruction: a face side with a reconstructed density or pressure
+// <= 0 takes its cell's values.
+template <typename T, int D, int BX, int BY, int DIM, bool VISC>
+__device__ __forceinline__ void face_fallback(const RingView<T, BX, BY, DIM, VISC>& R, int x0, int y0,
+                                              const Gas<T>& g, T Wm[5], T Wp[5]) {
   using Ro = Roles<D>;
   auto val = [&](int c, int n, int t1, int t2) -> T {
     int x, y, e;
@@ -447,6 +451,15 @@ __device__ __forceinline__ void face_riemann(const RingView<T, BX, BY, DIM, VISC
       for (int c = 0; c < 5; ++c) Wp[c] = val(c, 1, 0, 0);
     }
   }
+}
+
+// Convective flux F of a Godunov-type face from its reconstructed states Wm
+// (left) and Wp (right): the safe-reconstruction fallback, then the Riemann
+// solver of the kernel family.
+template <typename T, int D, int BX, int BY, int DIM, bool VISC, int SCH>
+__device__ __forceinline__ void face_riemann(const RingView<T, BX, BY, DIM, VISC>& R, int x0, int y0,
+                                             const Gas<T>& g, T Wm[5], T Wp[5], T F[5]) {
+  face_fallback<T, D, BX, BY, DIM, VISC>(R, x0, y0, g, Wm, Wp);
   if constexpr (sch_general(SCH)) riemann_flux<T, D>(Wm, Wp, g, F);
   else if constexpr (SCH == SCH_NN) rusanov_nn<T, D>(Wm, Wp, g, F);
   else hllc<T, D>(Wm, Wp, g, F, 0);
@@ -649,18 +662,10 @@ __device__ __forceinline__ void face_visc_add(const RingView<T, BX, BY, DIM, VIS
   NF[4] += uf[0] * tau[0] + uf[1] * tau[1] + uf[2] * tau[2] + g.lambda * dTdn;
 }
 
-// Net flux NF = F^d - F through the face between the cell at shared-memory
-// position (x0, y0, plane 0) and its neighbour along D.
-// SCH_DEFAULT: the default scheme (WENO5-JS, HLLC, Einfeldt speeds) compiled
-// alone; SCH_GENERAL(_EXT): the Table 2 Godunov variants chosen at run time
-// from g; SCH_ROE(_EXT): the flux-splitting ROE setup (reconstruction chosen
-// from g); the _EXT forms add WENO3-JS (and walls, in the plane fetch);
-// SCH_NN: the Rusanov-NN flux (Section 7.4; reconstruction chosen from g),
-// a kernel family of its own because the network's hidden layers need far
-// more registers than the other fluxes.
+// WENO left / right states of each primitive component of a face (Section 3.3).
 template <typename T, int D, int BX, int BY, int DIM, bool VISC, int SCH>
-__device__ __forceinline__ void face_flux(const RingView<T, BX, BY, DIM, VISC>& R, int x0, int y0,
-                                          const Gas<T>& g, const T inv_h[3], T NF[5]) {
+__device__ __forceinline__ void face_states(const RingView<T, BX, BY, DIM, VISC>& R, int x0, int y0,
+                                            const Gas<T>& g, T Wm[5], T Wp[5]) {
   using Ro = Roles<D>;
   const int recon = SCH == SCH_DEFAULT ? 0 : g.recon;
   auto val = [&](int c, int n, int t1, int t2) -> T {
@@ -668,12 +673,6 @@ __device__ __forceinline__ void face_flux(const RingView<T, BX, BY, DIM, VISC>& 
     Ro::map(n, t1, t2, x, y, e);
     return R.at(c, x0 + x, y0 + y, e);
   };
-  T F[5];
-  if constexpr (sch_roe(SCH)) {
-    fs_flux<T, D, sch_ext(SCH)>([&](int c, int n) { return val(c, n, 0, 0); }, g, recon, F);
-  } else {
-  // WENO5-JS left / right states of each primitive component (Section 3.3)
-  T Wm[5], Wp[5];
   if (sch_ext(SCH) && recon == 2) {
     // WENO3-JS: cells -1, 0, 1 (left state) and 2, 1, 0 (right state)
 #pragma unroll
@@ -704,7 +703,33 @@ __device__ __forceinline__ void face_flux(const RingView<T, BX, BY, DIM, VISC>& 
     }
   }
   }
-  face_riemann<T, D, BX, BY, DIM, VISC, SCH>(R, x0, y0, g, Wm, Wp, F);
+}
+
+// Net flux NF = F^d - F through the face between the cell at shared-memory
+// position (x0, y0, plane 0) and its neighbour along D.
+// SCH_DEFAULT: the default scheme (WENO5-JS, HLLC, Einfeldt speeds) compiled
+// alone; SCH_GENERAL(_EXT): the Table 2 Godunov variants chosen at run time
+// from g; SCH_ROE(_EXT): the flux-splitting ROE setup (reconstruction chosen
+// from g); the _EXT forms add WENO3-JS (and walls, in the plane fetch);
+// SCH_NN: the Rusanov-NN flux (Section 7.4; reconstruction chosen from g),
+// a kernel family of its own because the network's hidden layers need far
+// more registers than the other fluxes.
+template <typename T, int D, int BX, int BY, int DIM, bool VISC, int SCH>
+__device__ __forceinline__ void face_flux(const RingView<T, BX, BY, DIM, VISC>& R, int x0, int y0,
+                                          const Gas<T>& g, const T inv_h[3], T NF[5]) {
+  using Ro = Roles<D>;
+  T F[5];
+  if constexpr (sch_roe(SCH)) {
+    auto val = [&](int c, int n) -> T {
+      int x, y, e;
+      Ro::map(n, 0, 0, x, y, e);
+      return R.at(c, x0 + x, y0 + y, e);
+    };
+    fs_flux<T, D, sch_ext(SCH)>(val, g, SCH == SCH_DEFAULT ? 0 : g.recon, F);
+  } else {
+    T Wm[5], Wp[5];
+    face_states<T, D, BX, BY, DIM, VISC, SCH>(R, x0, y0, g, Wm, Wp);
+    face_riemann<T, D, BX, BY, DIM, VISC, SCH>(R, x0, y0, g, Wm, Wp, F);
   }
 #pragma unroll
   for (int c = 0; c < 5; ++c) NF[c] = -F[c];
@@ -833,6 +858,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
   // face values of a plane kept in shared memory (x, y; along z only the
   // current cell's value at its upper face, zl, is kept, by its column)
   constexpr bool PC = sch_pc(SCH);
+  constexpr bool NNP = SCH == SCH_NN && sizeof(T) == 4 && plane_dims(DIM) == 2;
   constexpr bool W3 = sch_ext(SCH);
   const int wz = SCH == SCH_DEFAULT ? 0 : g.recon;  // 0 WENO5-JS, 1 WENO5-Z, 2 WENO3-JS (W3)
   constexpr int SX = BY * (BX + 2), SY = plane_dims(DIM) == 2 ? (BY + 2) * BX : 0;
@@ -1090,6 +1116,48 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
         for (int c = 0; c < 5; ++c)
           if (JF_CHECK(t >= 0 && t < G::NFY, "JFDBG Fy t=%d\n", t)) Fy[c * G::NFY + t] = NF[c];
       }
+    } else if constexpr (NNP) {
+      // the x and the y face of a thread through the network together (threads
+      // without an x face evaluate their y face's inputs twice)
+      T Xm[5], Xp[5], Ym[5], Yp[5], x[4], y[4], F[5];
+      const int px = HALO + xf_x - 1, py = G::HY + xf_y, qx = HALO + yf_x, qy = G::HY + yf_y - 1;
+      face_states<T, 1, BX, BY, DIM, VISC, SCH>(R, qx, qy, g, Ym, Yp);
+      face_fallback<T, 1, BX, BY, DIM, VISC>(R, qx, qy, g, Ym, Yp);
+      nn_face_inputs<T, 1>(Ym, Yp, g, y);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) x[m] = y[m];
+      if (xf_x >= 0) {
+        face_states<T, 0, BX, BY, DIM, VISC, SCH>(R, px, py, g, Xm, Xp);
+        face_fallback<T, 0, BX, BY, DIM, VISC>(R, px, py, g, Xm, Xp);
+        nn_face_inputs<T, 0>(Xm, Xp, g, x);
+      }
+      float2 in[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) in[m] = make_float2(x[m], y[m]);
+      const float2* th2 = reinterpret_cast<const float2*>(g.nn + kNnPairs);
+      float2* rows = reinterpret_cast<float2*>(const_cast<float*>(g.nn) + kNnRows);
+      const float2 alpha = nn_alpha_pair(th2, in, rows + threadIdx.x * NN_PAIR_ROW);
+      if (xf_x >= 0) {
+        rusanov_nn<T, 0>(Xm, Xp, g, F, alpha.x);
+        T NF[5];
+#pragma unroll
+        for (int c = 0; c < 5; ++c) NF[c] = -F[c];
+        if constexpr (VISC) face_visc_add<T, 0, BX, BY, DIM, VISC>(R, px, py, g, inv_h, NF);
+        const int t = xf_y * (BX + 1) + xf_x;
+#pragma unroll
+        for (int c = 0; c < 5; ++c) Fx[c * G::NFX + t] = NF[c];
+      }
+      rusanov_nn<T, 1>(Ym, Yp, g, F, alpha.y);
+      T NF[5];
+#pragma unroll
+      for (int c = 0; c < 5; ++c) NF[c] = -F[c];
+      if constexpr (VISC) face_visc_add<T, 1, BX, BY, DIM, VISC>(R, qx, qy, g, inv_h, NF);
+      const int t = yf_y * BX + yf_x;
+#pragma unroll
+      for (int c = 0; c < 5; ++c) Fy[c * G::NFY + t] = NF[c];
+      if constexpr (marches(DIM)) {
+        if (cell_thread) face_flux<T, 2, BX, BY, DIM, VISC, SCH>(R, HALO + tx, G::HY + ty, g, inv_h, NFz_hi);
+      }
     } else {
     if (xf_x >= 0) {
       T NF[5];
@@ -1279,6 +1347,14 @@ constexpr size_t nn_smem_offset() {
   return (stage_smem_elems<T, DIM, VISC, BX, BY>() + q - 1) / q * q;
 }
 
+// Elements of the parameters there: the network's, and in the FP32 kernels of
+// tiles spanning y a copy with every value twice and the threads' hidden rows
+// (nn_alpha_pair), from the elements kNnPairs and kNnRows.
+template <typename T, int DIM, int NT>
+constexpr size_t nn_smem_elems() {
+  return sizeof(T) == 4 && plane_dims(DIM) == 2 ? kNnRows + (size_t)2 * NN_PAIR_ROW * NT : NN_PARAMS;
+}
+
 // The stage kernel.  blockDim.x == Geo::NT.
 //  * Single grid (work == null): one CTA per tile, the tile from blockIdx;
 //    grid = (ceil(nx/BX), ceil(ny/BY), ceil(nz/zchunk)) (3D), (.., .., 1) otherwise.
@@ -1300,7 +1376,7 @@ __global__ void __launch_bounds__(Geo<BX, BY, DIM, VISC>::NT, MINB)
   {
     unsigned dyn;
     asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
-    const size_t need = sizeof(T) * (SCH == SCH_NN ? nn_smem_offset<T, DIM, VISC, BX, BY>() + NN_PARAMS
+    const size_t need = sizeof(T) * (SCH == SCH_NN ? nn_smem_offset<T, DIM, VISC, BX, BY>() + nn_smem_elems<T, DIM, Geo<BX, BY, DIM, VISC>::NT>()
                                                    : stage_smem_elems<T, DIM, VISC, BX, BY>() +
                                                          (sch_pc(SCH) ? recon_smem_elems<DIM, BX, BY, T>() : 0));
     if (!JF_CHECK(dyn >= need, "JFDBG smem %u < %llu\n", dyn, (unsigned long long)need)) return;
@@ -1320,8 +1396,13 @@ __global__ void __launch_bounds__(Geo<BX, BY, DIM, VISC>::NT, MINB)
   if constexpr (SCH == SCH_NN) {
     // the Rusanov-NN parameters, after the stage buffers at a 16-byte
     // aligned offset (the launch adds them to the dynamic shared memory)
+    // (and, FP32 tiles spanning y, once more with every value twice)
     T* th = reinterpret_cast<T*>(smem_raw) + nn_smem_offset<T, DIM, VISC, BX, BY>();
-    for (int i = threadIdx.x; i < NN_PARAMS; i += blockDim.x) th[i] = __ldg(g.nn + i);
+    for (int i = threadIdx.x; i < NN_PARAMS; i += blockDim.x) {
+      const T v = __ldg(g.nn + i);
+      th[i] = v;
+      if constexpr (nn_smem_elems<T, DIM, 0>() > NN_PARAMS) th[kNnPairs + 2 * i] = th[kNnPairs + 2 * i + 1] = v;
+    }
     __syncthreads();
     gk.nn = th;
   }

@@ -9,7 +9,7 @@ namespace jf {
 // per-cell WENO5 face values in the default-scheme kernels.
 template <typename T, int DIM, bool VISC, int BX, int BY, int SCH>
 constexpr size_t launch_smem() {
-  return SCH == SCH_NN ? sizeof(T) * (nn_smem_offset<T, DIM, VISC, BX, BY>() + NN_PARAMS)
+  return SCH == SCH_NN ? sizeof(T) * (nn_smem_offset<T, DIM, VISC, BX, BY>() + nn_smem_elems<T, DIM, Geo<BX, BY, DIM, VISC>::NT>())
                        : stage_smem_bytes<T, DIM, VISC, BX, BY>() +
                              (sch_pc(SCH) ? sizeof(T) * recon_smem_elems<DIM, BX, BY, T>() : 0);
 }
