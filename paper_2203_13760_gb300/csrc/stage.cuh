@@ -858,6 +858,11 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
   // face values of a plane kept in shared memory (x, y; along z only the
   // current cell's value at its upper face, zl, is kept, by its column)
   constexpr bool PC = sch_pc(SCH);
+  // Overlapped loads in the prologue of a march: inviscid default kernels and
+  // FP64, where they cost nothing else (64 uneven 2D grids: 248 -> 241 us per
+  // stage; the viscous FP32 and ROE kernels, at their 128 registers, schedule
+  // their marches worse with them: 256^3 viscous step 4.20 -> 4.45 ms)
+  constexpr bool EARLY = PC && !WALLS && marches(DIM) && (sizeof(T) == 8 || (!VISC && SCH == SCH_DEFAULT));
   constexpr bool NNP = SCH == SCH_NN && sizeof(T) == 4 && plane_dims(DIM) == 2;
   constexpr bool W3 = sch_ext(SCH);
   const int wz = SCH == SCH_DEFAULT ? 0 : g.recon;  // 0 WENO5-JS, 1 WENO5-Z, 2 WENO3-JS (W3)
@@ -887,8 +892,21 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
   PlaneMap<T, BX, BY, DIM, VISC> pmap;    // per-cell families (no walls): the in-plane offsets of its cells
   if constexpr (PC && !WALLS && marches(DIM)) plane_map<T, BX, BY, DIM, VISC>(A, pmap, gx0, gy0);
   if (marches(DIM)) {
+    if constexpr (EARLY) {
+      // three planes at a time, and plane z0 + 3 during the face below
+      PlaneRegs<T, BX, BY, DIM, VISC> first[3];
 #pragma unroll 1
-    for (int q = 0; q < 6; ++q) load_plane<T, BX, BY, DIM, VISC, WALLS>(A, g, ring + q * G::PLANE, gx0, gy0, z0 - 3 + q);
+      for (int q = 0; q < 6; q += 3) {
+#pragma unroll
+        for (int p = 0; p < 3; ++p) fetch_plane_mapped<T, BX, BY, DIM, VISC>(A, first[p], pmap, z0 - 3 + q + p);
+#pragma unroll
+        for (int p = 0; p < 3; ++p) commit_plane<T, BX, BY, DIM, VISC>(A, g, first[p], ring + (q + p) * G::PLANE);
+      }
+      fetch_plane_mapped<T, BX, BY, DIM, VISC>(A, next, pmap, z0 + 3);
+    } else {
+#pragma unroll 1
+      for (int q = 0; q < 6; ++q) load_plane<T, BX, BY, DIM, VISC, WALLS>(A, g, ring + q * G::PLANE, gx0, gy0, z0 - 3 + q);
+    }
     __syncthreads();
     // lower face of plane z0 = upper face of plane z0 - 1 (slot 2); plane
     // offset -3 is never read
@@ -920,7 +938,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
       if constexpr (plane_dims(DIM) == 2) face_carry_init<T, 1>(R, HALO + yf_x, G::HY + yf_y - 1, -1, ycar);
     }
     __syncthreads();  // slot 0 (plane z0 - 3) is overwritten next
-    load_plane<T, BX, BY, DIM, VISC, WALLS>(A, g, ring, gx0, gy0, z0 + 3);
+    if constexpr (EARLY) commit_plane<T, BX, BY, DIM, VISC>(A, g, next, ring);
+    else load_plane<T, BX, BY, DIM, VISC, WALLS>(A, g, ring, gx0, gy0, z0 + 3);
     // (per-cell families: each plane fetches plane k + 4 after its reconstruction phase)
     if (!PC && z0 + 1 < z1) fetch_plane<T, BX, BY, DIM, VISC, WALLS>(A, next, gx0, gy0, z0 + 4);
   } else {
