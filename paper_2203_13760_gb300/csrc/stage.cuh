@@ -957,10 +957,15 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
     const long long qc = ((long long)(marches(DIM) ? k : 0) * A.ny + gy) * A.nx + gx;
     T us[5], un[5];
     auto load_cell = [&]() {
-      if (own && !A.rhs_only) {
+      if constexpr (SPLIT) {
+        if (own && !A.rhs_only) {
+          const bool ok = JF_CHECK(qc >= 0 && qc < A.N, "JFDBG cell qc=%lld N=%lld\n", qc, A.N);
+          us[0] = ok ? __ldg(A.Us + qc + warp * A.N) : T(1);
+          un[0] = A.Un && ok ? A.Un[qc + warp * A.N] : T(0);
+        }
+      } else if (own && !A.rhs_only) {
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
-          if (SPLIT && c != warp) continue;
           const bool ok = JF_CHECK(qc >= 0 && qc < A.N, "JFDBG cell qc=%lld N=%lld\n", qc, A.N);
           us[c] = ok ? __ldg(A.Us + qc + gcomp(DIM, c) * A.N) : T(1);
           un[c] = A.Un && ok ? A.Un[qc + gcomp(DIM, c) * A.N] : T(0);
@@ -1235,9 +1240,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
         comb(4, false);
       }
     } else if (own) {
-#pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        if (SPLIT && c != warp) continue;
+      auto update = [&](int c, T u, T n) {
         const int fx = ty * (BX + 1) + tx;
         T rhs = (Fx[c * G::NFX + fx + 1] - Fx[c * G::NFX + fx]) * inv_h[0];
         if (plane_dims(DIM) == 2) {
@@ -1250,10 +1253,16 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
         if (A.rhs_only) {
           o = rhs;
         } else {
-          o = A.b * (us[c] + dt * rhs);
-          if (A.Un) o += A.a * un[c];
+          o = A.b * (u + dt * rhs);
+          if (A.Un) o += A.a * n;
         }
         if (JF_CHECK(qc >= 0 && qc < A.N, "JFDBG store qc=%lld N=%lld\n", qc, A.N)) A.out[qc + gcomp(DIM, c) * A.N] = o;
+      };
+      if constexpr (SPLIT) {
+        update(warp, us[0], un[0]);
+      } else {
+#pragma unroll
+        for (int c = 0; c < 5; ++c) update(c, us[c], un[c]);
       }
     }
     if (marches(DIM)) {
