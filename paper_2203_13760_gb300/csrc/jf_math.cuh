@@ -851,6 +851,14 @@ static __device__ __noinline__ float2 nn_alpha_pair(const float2* th2, const flo
   for (int i = 0; i < NN_HIDDEN; ++i) out = __ffma2_rn(W4[i], relu(z[i]), out);
   return make_float2(texp(out.x), texp(out.y));
 }
+#else
+constexpr int NN_PAIR_ROW = 0;  // host: lane by lane, no hidden rows
+inline float2 nn_alpha_pair(const float2* th2, const float2 x[4], float2*) {
+  float th[NN_PARAMS], a[4], b[4];
+  for (int k = 0; k < NN_PARAMS; ++k) th[k] = th2[k].x;
+  for (int m = 0; m < 4; ++m) { a[m] = x[m].x; b[m] = x[m].y; }
+  return make_float2(nn_alpha(th, a), nn_alpha(th, b));
+}
 #endif
 
 // Network inputs of the Rusanov-NN flux at a face along D (Section 7.4):

@@ -42,9 +42,6 @@ namespace jf {
 constexpr int HALO = 3;
 // Rusanov-NN parameters in shared memory (nn_smem_elems)
 constexpr int kNnPairs = (NN_PARAMS + 3) / 4 * 4, kNnRows = kNnPairs + (2 * NN_PARAMS + 3) / 4 * 4;
-#ifndef __CUDACC__
-constexpr int NN_PAIR_ROW = 0;
-#endif
 
 // Kernel dimensionality (template parameter DIM).  1, 2 and 3 are the grid's
 // active axes: the tile spans x (1D: one row of BX cells; 2D, 3D: BX x BY
