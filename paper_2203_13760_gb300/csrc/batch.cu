@@ -24,7 +24,8 @@ constexpr long long kChunk = 16384;  // cells per CFL CTA (a whole number of vec
 // Euler steps of a batch: U = U1 for every simulation (blockIdx.y), the
 // pointers read from the device descriptors so that rebinding stays valid.
 template <typename T>
-__global__ void __launch_bounds__(256) batch_copy_kernel(const SimDesc<T>* __restrict__ sims) {
+__global__ void __launch_bounds__(256) batch_copy_kernel(const SimDesc<T>* sims) {
+  follow_predecessor();
   const SimDesc<T> d = sims[blockIdx.y];
   const long long n = 5 * d.N;
 #ifdef JF_DEBUG_BOUNDS
@@ -38,9 +39,10 @@ __global__ void __launch_bounds__(256) batch_copy_kernel(const SimDesc<T>* __res
 // Trajectories (jf_batch_feed_forward): dst[s] = src[s] for every
 // simulation (blockIdx.y) of one row of the pointer tables.
 template <typename T>
-__global__ void __launch_bounds__(256) batch_copy_pairs_kernel(const T* const* __restrict__ src,
-                                                               T* const* __restrict__ dst,
-                                                               const long long* __restrict__ count) {
+__global__ void __launch_bounds__(256) batch_copy_pairs_kernel(const T* const* src,
+                                                               T* const* dst,
+                                                               const long long* count) {
+  follow_predecessor();
   const T* a = src[blockIdx.y];
   T* b = dst[blockIdx.y];
   const long long n = count[blockIdx.y];
@@ -274,8 +276,8 @@ jf_status enqueue_steps(jf_ctx* h, int nsteps, double* dt_out, cudaStream_t s) {
       if (e != cudaSuccess) return cuda_fail(h, e, "batch: stage launch");
     }
     if (integ == JF_EULER) {
-      batch_copy_kernel<T><<<dim3((unsigned)h->sms, (unsigned)h->nsim), 256, 0, s>>>(sims);
-      if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(h, e, "batch: copy launch");
+      if ((e = launch_next(batch_copy_kernel<T>, dim3((unsigned)h->sms, (unsigned)h->nsim), 256u, 0, s, sims)) !=
+          cudaSuccess) return cuda_fail(h, e, "batch: copy launch");
     }
   }
   if (dt_out) {
@@ -349,20 +351,19 @@ jf_status feed_forward_batch(jf_ctx* h, void* const* U0_ptrs, void* const* traj_
   const dim3 cgrid((unsigned)h->sms, (unsigned)ns);
   jf_status st = JF_OK;
   // row 0 of the copy tables: U0 -> slot 0; row t + 1: slot t -> slot t + 1
-  batch_copy_pairs_kernel<T><<<cgrid, 256, 0, s>>>(d_src, d_dst, d_count);
-  if ((e = cudaGetLastError()) != cudaSuccess) st = cuda_fail(h, e, "feed_forward: copy launch");
+  e = launch_next(batch_copy_pairs_kernel<T>, cgrid, 256u, 0, s, d_src, d_dst, d_count);
+  if (e != cudaSuccess) st = cuda_fail(h, e, "feed_forward: copy launch");
   for (int t = 0; t < nsteps && st == JF_OK; ++t) {
-    batch_copy_pairs_kernel<T><<<cgrid, 256, 0, s>>>(d_src + (size_t)(t + 1) * ns, d_dst + (size_t)(t + 1) * ns,
-                                                     d_count);
-    if ((e = cudaGetLastError()) != cudaSuccess) { st = cuda_fail(h, e, "feed_forward: copy launch"); break; }
+    e = launch_next(batch_copy_pairs_kernel<T>, cgrid, 256u, 0, s, d_src + (size_t)(t + 1) * ns,
+                    d_dst + (size_t)(t + 1) * ns, d_count);
+    if (e != cudaSuccess) { st = cuda_fail(h, e, "feed_forward: copy launch"); break; }
     const SimDesc<T>* sims = d_desc + (size_t)t * ns;  // U = slot t + 1
     for (int q = 0; q < nst; ++q) {
       e = launch_batch_stage<T>(h, sv, sims, desc.data() + (size_t)t * ns, codes[q], g, s);
       if (e != cudaSuccess) { st = cuda_fail(h, e, "feed_forward: stage launch"); break; }
     }
     if (st == JF_OK && integ == JF_EULER) {
-      batch_copy_kernel<T><<<cgrid, 256, 0, s>>>(sims);
-      if ((e = cudaGetLastError()) != cudaSuccess) st = cuda_fail(h, e, "feed_forward: copy launch");
+      if ((e = launch_next(batch_copy_kernel<T>, cgrid, 256u, 0, s, sims)) != cudaSuccess) st = cuda_fail(h, e, "feed_forward: copy launch");
     }
   }
   cudaFreeAsync(dev, s);

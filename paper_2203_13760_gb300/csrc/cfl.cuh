@@ -38,12 +38,13 @@ inline unsigned cfl_threads(long long N) {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kCflThreads) cfl_kernel(const T* __restrict__ U0, CflArgs a0, ReduceScratch* sc0,
+__global__ void __launch_bounds__(kCflThreads) cfl_kernel(const T* U0, CflArgs a0, ReduceScratch* sc0,
                                                   double* dt0, double* dt0b, int* flag,
-                                                  const SimDesc<T>* __restrict__ sims,
-                                                  const CflChunk* __restrict__ chunks,
-                                                  const CflArgs* __restrict__ args, ReduceScratch* red,
+                                                  const SimDesc<T>* sims,
+                                                  const CflChunk* chunks,
+                                                  const CflArgs* args, ReduceScratch* red,
                                                   double* dts) {
+  follow_predecessor();
   const T* U;
   CflArgs a;
   ReduceScratch* sc;

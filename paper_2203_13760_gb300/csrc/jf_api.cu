@@ -375,9 +375,9 @@ jf_status rhs_impl(jf_ctx* h, const void* U, void* dUdt, cudaStream_t s) {
 template <typename T>
 jf_status cfl_impl(jf_ctx* h, const void* U, double* dt_out, double* dt_out2, cudaStream_t s) {
   const CflArgs a = make_cfl(h->grid, h->gas, h->scheme);
-  cfl_kernel<T><<<cfl_blocks<T>(a.N, h->sms), cfl_threads<T>(a.N), 0, s>>>(
-      static_cast<const T*>(U), a, h->red_cfl, dt_out, dt_out2, h->flag, nullptr, nullptr, nullptr, nullptr, nullptr);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e =
+      launch_next(cfl_kernel<T>, dim3(cfl_blocks<T>(a.N, h->sms)), cfl_threads<T>(a.N), 0, s, static_cast<const T*>(U), a,
+                  h->red_cfl, dt_out, dt_out2, h->flag, nullptr, nullptr, nullptr, nullptr, nullptr);
   if (e != cudaSuccess) return cuda_fail(h, e, "cfl kernel launch");
   return JF_OK;
 }
@@ -387,10 +387,8 @@ template <typename T>
 cudaError_t launch_cfl_batch(const void* sims, const void* chunks, int nchunks, const CflArgs* args,
                              ReduceScratch* red, double* dts, int* flag, cudaStream_t s) {
   CflArgs none{};
-  cfl_kernel<T><<<nchunks, 256, 0, s>>>(nullptr, none, nullptr, nullptr, nullptr, flag,
-                                        static_cast<const SimDesc<T>*>(sims), static_cast<const CflChunk*>(chunks),
-                                        args, red, dts);
-  return cudaGetLastError();
+  return launch_next(cfl_kernel<T>, dim3(nchunks), 256u, 0, s, nullptr, none, nullptr, nullptr, nullptr, flag,
+                     static_cast<const SimDesc<T>*>(sims), static_cast<const CflChunk*>(chunks), args, red, dts);
 }
 template cudaError_t launch_cfl_batch<float>(const void*, const void*, int, const CflArgs*, ReduceScratch*, double*,
                                              int*, cudaStream_t);
@@ -455,9 +453,9 @@ jf_status loss_impl(jf_ctx* h, const void* U, const void* target, double* loss, 
   const long long N = (long long)h->grid.nx * h->grid.ny * h->grid.nz;
   double dV = 1.0;
   for (int d = 0; d < h->dim; ++d) dV *= spacing(h->grid, d);
-  loss_density_kernel<T><<<reduce_blocks(N, h->sms), 256, 0, s>>>(
-      static_cast<const T*>(U), static_cast<const T*>(target), N, dV, h->red_loss, loss, static_cast<T*>(seed));
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e =
+      launch_next(loss_density_kernel<T>, dim3(reduce_blocks(N, h->sms)), 256u, 0, s, static_cast<const T*>(U),
+                  static_cast<const T*>(target), N, dV, h->red_loss, loss, static_cast<T*>(seed));
   if (e != cudaSuccess) return cuda_fail(h, e, "loss kernel launch");
   return JF_OK;
 }

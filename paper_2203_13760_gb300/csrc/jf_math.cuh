@@ -23,6 +23,68 @@
 
 namespace jf {
 
+// Programmatic dependent launch of the kernels that follow one another on a
+// stream (stages, CFL passes, adjoints): a launch may be made ready while its
+// predecessor still runs, and its CTAs take the SMs that the predecessor's
+// leave.  Every kernel launched this way starts with follow_predecessor(),
+// which waits until the predecessor has finished and its writes are visible,
+// and only then lets its own successor start, so that at most one kernel waits
+// ahead.  These kernels read what their predecessor may have written with plain
+// loads: no __ldg and no const __restrict__ pointers, whose loads are taken for
+// read-only during the whole kernel and may move above the wait.  A launch after a
+// copy, a memset or another library's kernel waits for that as usual.
+//
+// Before and after: FP64 step of a 200-cell tube 39.5 -> 31 us (four dependent
+// launches of a few us each), 97 x 61 x 43 step 139 -> 132 us, gradient of eight
+// 256^2 steps 2.90 -> 2.4 ms, a training step on a 32^2 batch 2.63 -> 2.49 ms;
+// steps of a millisecond and more within 1 %.
+
+__device__ __forceinline__ void follow_predecessor() {
+#ifdef __CUDA_ARCH__
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#endif
+}
+
+// A load of the stage input, which the kernel does not write: free to move past
+// its stores like a read-only load, but (volatile) not above the wait.  A plain
+// load costs the 128-register kernels a percent (256^3 step 4.21 -> 4.23 ms).
+__device__ __forceinline__ float ld_state(const float* p) {
+#ifdef __CUDA_ARCH__
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+#else
+  return *p;
+#endif
+}
+__device__ __forceinline__ double ld_state(const double* p) {
+#ifdef __CUDA_ARCH__
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+#else
+  return *p;
+#endif
+}
+
+#ifdef __CUDACC__
+template <typename... P, typename... A>
+cudaError_t launch_next(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#endif
+
 template <typename T>
 struct Gas {
   T gamma;     // ratio of specific heats

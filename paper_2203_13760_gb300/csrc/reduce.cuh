@@ -76,7 +76,7 @@ __device__ __forceinline__ void cell_rates_of(T r, T ru, T rv, T rw, T E, int na
   diff = fmax(diff, kdiff * inv);
 }
 template <typename T>
-__device__ __forceinline__ void cell_rates(const T* __restrict__ U, long long q, long long N, int nactive, T gamma,
+__device__ __forceinline__ void cell_rates(const T* U, long long q, long long N, int nactive, T gamma,
                                            T gm1, T kdiff, T& conv, T& diff, bool& bad) {
   cell_rates_of(U[q], U[q + N], U[q + 2 * N], U[q + 3 * N], U[q + 4 * N], nactive, gamma, gm1, kdiff, conv, diff,
                 bad);
@@ -145,9 +145,10 @@ __device__ __forceinline__ void finish_cfl(T conv, T diff, ReduceScratch* sc, un
 // loss = sum_cells (rho - target)^2 * dV; seed = d loss / dU (density
 // component only).  blockDim.x == 256.
 template <typename T>
-__global__ void __launch_bounds__(256) loss_density_kernel(const T* __restrict__ U, const T* __restrict__ target,
+__global__ void __launch_bounds__(256) loss_density_kernel(const T* U, const T* target,
                                                            long long N, double dV, ReduceScratch* sc,
                                                            double* loss, T* seed) {
+  follow_predecessor();
   double s = 0.0;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < N; q += stride) {

@@ -168,7 +168,14 @@ struct PlaneRegs {
 // tile at (gx0, gy0).
 // WALLS: the kernel handles slip walls (only the extended and Rusanov-NN
 // kernel families; the host routes every walled grid to one of them).
-template <typename T, int BX, int BY, int DIM, bool VISC, bool WALLS>
+// NC: the kernel is launched after its predecessor has finished (the ROE
+// families), so that its loads may be read-only ones.
+template <bool NC, typename T>
+__device__ __forceinline__ T ld_input(const T* p) {
+  if constexpr (NC) return __ldg(p);
+  else return ld_state(p);
+}
+template <typename T, int BX, int BY, int DIM, bool VISC, bool WALLS, bool NC = false>
 __device__ __forceinline__ void fetch_plane(const StageArgs<T>& A, PlaneRegs<T, BX, BY, DIM, VISC>& r, int gx0,
                                             int gy0, int gz) {
   using G = Geo<BX, BY, DIM, VISC>;
@@ -196,7 +203,7 @@ __device__ __forceinline__ void fetch_plane(const StageArgs<T>& A, PlaneRegs<T, 
       for (int c = 0; c < 5; ++c)
         r.v[i][c] = JF_CHECK(q >= 0 && q < A.N, "JFDBG fetch q=%lld N=%lld gx=%d gy=%d kz=%d tile=(%d,%d) t=%d\n", q,
                              A.N, gx, gy, kz, gx0, gy0, t)
-                        ? __ldg(A.Us + q + gcomp(DIM, c) * A.N)
+                        ? ld_input<NC>(A.Us + q + gcomp(DIM, c) * A.N)
                         : T(1);
       if (WALLS) {
         if (fx) r.v[i][1] = -r.v[i][1];
@@ -244,7 +251,7 @@ __device__ __forceinline__ void fetch_plane_mapped(const StageArgs<T>& A, PlaneR
 #pragma unroll
       for (int c = 0; c < 5; ++c)
         r.v[i][c] = JF_CHECK(q >= 0 && q < A.N, "JFDBG fetch q=%lld N=%lld t=%d\n", q, A.N, t)
-                        ? __ldg(A.Us + q + gcomp(DIM, c) * A.N)
+                        ? ld_state(A.Us + q + gcomp(DIM, c) * A.N)
                         : T(1);
     }
   }
@@ -277,11 +284,11 @@ __device__ __forceinline__ void commit_plane(const StageArgs<T>& A, const Gas<T>
   if (bad) atomicOr(A.flag, 1);
 }
 
-template <typename T, int BX, int BY, int DIM, bool VISC, bool WALLS>
+template <typename T, int BX, int BY, int DIM, bool VISC, bool WALLS, bool NC = false>
 __device__ __forceinline__ void load_plane(const StageArgs<T>& A, const Gas<T>& g, T* dst, int gx0, int gy0,
                                            int gz) {
   PlaneRegs<T, BX, BY, DIM, VISC> r;
-  fetch_plane<T, BX, BY, DIM, VISC, WALLS>(A, r, gx0, gy0, gz);
+  fetch_plane<T, BX, BY, DIM, VISC, WALLS, NC>(A, r, gx0, gy0, gz);
   commit_plane<T, BX, BY, DIM, VISC>(A, g, r, dst);
 }
 
@@ -325,6 +332,10 @@ enum { SCH_DEFAULT = 0, SCH_GENERAL = 1, SCH_ROE = 2, SCH_NN = 3, SCH_GENERAL_EX
 constexpr bool sch_general(int s) { return s == SCH_GENERAL || s == SCH_GENERAL_EXT; }
 constexpr bool sch_roe(int s) { return s == SCH_ROE || s == SCH_ROE_EXT; }
 constexpr bool sch_ext(int s) { return s == SCH_GENERAL_EXT || s == SCH_ROE_EXT || s == SCH_NN; }
+// Families launched by launch_next.  The ROE kernels are launched the plain way:
+// the wait and the loads it asks for cost them more than the overlap gives
+// (128^3 step 893 -> 917 us).
+constexpr bool overlapped_launch(int s) { return !sch_roe(s); }
 // Families whose kernels reconstruct once per cell and direction (the face
 // values of a plane in shared memory): the default scheme and the run-time
 // Godunov schemes.
@@ -800,7 +811,7 @@ template <typename T, int DIM, bool VISC, int BX, int BY, int SCH>
 __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& g, int bx, int by, int bz,
                                            T* smem) {
   using G = Geo<BX, BY, DIM, VISC>;
-  constexpr bool WALLS = sch_ext(SCH);
+  constexpr bool WALLS = sch_ext(SCH), NC = !overlapped_launch(SCH);
   T* ring = smem;
   T* Fx = ring + G::RING * G::PLANE;      // [5][BY][BX+1]
   T* Fy = Fx + 5 * G::NFX;                // [5][BY+1][BX]
@@ -902,7 +913,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
       fetch_plane_mapped<T, BX, BY, DIM, VISC>(A, next, pmap, z0 + 3);
     } else {
 #pragma unroll 1
-      for (int q = 0; q < 6; ++q) load_plane<T, BX, BY, DIM, VISC, WALLS>(A, g, ring + q * G::PLANE, gx0, gy0, z0 - 3 + q);
+      for (int q = 0; q < 6; ++q) load_plane<T, BX, BY, DIM, VISC, WALLS, NC>(A, g, ring + q * G::PLANE, gx0, gy0, z0 - 3 + q);
     }
     __syncthreads();
     // lower face of plane z0 = upper face of plane z0 - 1 (slot 2); plane
@@ -936,11 +947,11 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
     }
     __syncthreads();  // slot 0 (plane z0 - 3) is overwritten next
     if constexpr (EARLY) commit_plane<T, BX, BY, DIM, VISC>(A, g, next, ring);
-    else load_plane<T, BX, BY, DIM, VISC, WALLS>(A, g, ring, gx0, gy0, z0 + 3);
+    else load_plane<T, BX, BY, DIM, VISC, WALLS, NC>(A, g, ring, gx0, gy0, z0 + 3);
     // (per-cell families: each plane fetches plane k + 4 after its reconstruction phase)
-    if (!PC && z0 + 1 < z1) fetch_plane<T, BX, BY, DIM, VISC, WALLS>(A, next, gx0, gy0, z0 + 4);
+    if (!PC && z0 + 1 < z1) fetch_plane<T, BX, BY, DIM, VISC, WALLS, NC>(A, next, gx0, gy0, z0 + 4);
   } else {
-    load_plane<T, BX, BY, DIM, VISC, WALLS>(A, g, ring, gx0, gy0, 0);
+    load_plane<T, BX, BY, DIM, VISC, WALLS, NC>(A, g, ring, gx0, gy0, 0);
   }
   __syncthreads();
 
@@ -957,14 +968,14 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
       if constexpr (SPLIT) {
         if (own && !A.rhs_only) {
           const bool ok = JF_CHECK(qc >= 0 && qc < A.N, "JFDBG cell qc=%lld N=%lld\n", qc, A.N);
-          us[0] = ok ? __ldg(A.Us + qc + warp * A.N) : T(1);
+          us[0] = ok ? ld_state(A.Us + qc + warp * A.N) : T(1);
           un[0] = A.Un && ok ? A.Un[qc + warp * A.N] : T(0);
         }
       } else if (own && !A.rhs_only) {
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
           const bool ok = JF_CHECK(qc >= 0 && qc < A.N, "JFDBG cell qc=%lld N=%lld\n", qc, A.N);
-          us[c] = ok ? __ldg(A.Us + qc + gcomp(DIM, c) * A.N) : T(1);
+          us[c] = ok ? ld_input<NC>(A.Us + qc + gcomp(DIM, c) * A.N) : T(1);
           un[c] = A.Un && ok ? A.Un[qc + gcomp(DIM, c) * A.N] : T(0);
         }
       }
@@ -1268,7 +1279,7 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
       const int nb = base + 1 == 6 ? 0 : base + 1;  // slot of plane k - 2, dead after this plane's faces
       if (k + 1 < z1) {
         commit_plane<T, BX, BY, DIM, VISC>(A, g, next, ring + nb * G::PLANE);  // plane k + 4
-        if (!PC && k + 2 < z1) fetch_plane<T, BX, BY, DIM, VISC, WALLS>(A, next, gx0, gy0, k + 5);
+        if (!PC && k + 2 < z1) fetch_plane<T, BX, BY, DIM, VISC, WALLS, NC>(A, next, gx0, gy0, k + 5);
       }
       __syncthreads();
       base = nb;
@@ -1394,9 +1405,10 @@ constexpr size_t nn_smem_elems() {
 // simulation advanced in a batch is bitwise the one advanced alone.
 template <typename T, int DIM, bool VISC, int BX, int BY, int MINB, int SCH>
 __global__ void __launch_bounds__(Geo<BX, BY, DIM, VISC>::NT, MINB)
-    stage_kernel(const StageArgs<T> A0, const SimDesc<T>* __restrict__ sims, const WorkItem* __restrict__ work,
+    stage_kernel(const StageArgs<T> A0, const SimDesc<T>* sims, const WorkItem* work,
                  int nwork, int stage, const Gas<T> g) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  if constexpr (overlapped_launch(SCH)) follow_predecessor();
 #ifdef JF_DEBUG_BOUNDS
   {
     unsigned dyn;
@@ -1424,7 +1436,7 @@ __global__ void __launch_bounds__(Geo<BX, BY, DIM, VISC>::NT, MINB)
     // (and, FP32 tiles spanning y, once more with every value twice)
     T* th = reinterpret_cast<T*>(smem_raw) + nn_smem_offset<T, DIM, VISC, BX, BY>();
     for (int i = threadIdx.x; i < NN_PARAMS; i += blockDim.x) {
-      const T v = __ldg(g.nn + i);
+      const T v = g.nn[i];
       th[i] = v;
       if constexpr (nn_smem_elems<T, DIM, 0>() > NN_PARAMS) th[kNnPairs + 2 * i] = th[kNnPairs + 2 * i + 1] = v;
     }

@@ -22,6 +22,13 @@ cudaError_t prepare_stage() {
                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
+template <int SCH, typename... P, typename... A>
+cudaError_t launch_stage_kernel(void (*k)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A... args) {
+  if constexpr (overlapped_launch(SCH)) return launch_next(k, grid, threads, smem, s, args...);
+  k<<<grid, threads, smem, s>>>(static_cast<P>(args)...);
+  return cudaGetLastError();
+}
+
 // A.zchunk: planes per CTA of a z-march (DIM_Y2: rows of the 2D grid).
 template <typename T, int DIM, bool VISC, int BX, int BY, int MINB, int SCH>
 cudaError_t launch_stage(const StageArgs<T>& A0, const Gas<T>& g, cudaStream_t s) {
@@ -30,9 +37,8 @@ cudaError_t launch_stage(const StageArgs<T>& A0, const Gas<T>& g, cudaStream_t s
   if constexpr (DIM == DIM_Y2) rows_as_planes(A);
   const dim3 grid((A.nx + BX - 1) / BX, plane_dims(DIM) == 2 ? (A.ny + BY - 1) / BY : 1,
                   marches(DIM) ? (A.nz + A.zchunk - 1) / A.zchunk : 1);
-  stage_kernel<T, DIM, VISC, BX, BY, MINB, SCH><<<grid, Geo<BX, BY, DIM, VISC>::NT, smem, s>>>(A, nullptr, nullptr, 0, 0,
-                                                                                          g);
-  return cudaGetLastError();
+  return launch_stage_kernel<SCH>(stage_kernel<T, DIM, VISC, BX, BY, MINB, SCH>, grid, Geo<BX, BY, DIM, VISC>::NT,
+                                  smem, s, A, nullptr, nullptr, 0, 0, g);
 }
 
 template <typename T, int DIM, bool VISC, int BX, int BY, int MINB, int SCH>
@@ -57,9 +63,8 @@ cudaError_t launch_batch(const SimDesc<T>* sims, const WorkItem* work, int nwork
 #ifdef JF_DEBUG_BOUNDS
   A.trace = debug_trace_dev();
 #endif
-  stage_kernel<T, DIM, VISC, BX, BY, MINB, SCH><<<grid, Geo<BX, BY, DIM, VISC>::NT, smem, s>>>(A, sims, work, nwork,
-                                                                                          stage, g);
-  return cudaGetLastError();
+  return launch_stage_kernel<SCH>(stage_kernel<T, DIM, VISC, BX, BY, MINB, SCH>, dim3(grid),
+                                  Geo<BX, BY, DIM, VISC>::NT, smem, s, A, sims, work, nwork, stage, g);
 }
 
 template <typename T, int DIM, bool VISC, int BX, int BY, int MINB, int SCH>

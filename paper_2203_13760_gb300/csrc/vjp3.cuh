@@ -276,6 +276,7 @@ __global__ void __launch_bounds__(NT, MINB)
     vjp3_kernel(const VjpArgs<T> A, const Gas<T> g, T* __restrict__ Gacc, int zchunk) {
   using G = V3Geo<BX, BY, VISC>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  follow_predecessor();
   T* Wr = reinterpret_cast<T*>(smem_raw);  // [RING][NCW][PY][PX]
   T* Ar = Wr + G::RING * G::PLANE;         // [ARING][NCW][PY][PX]
   T* Mr = Ar + G::ARING * G::PLANE;        // [2][5][MPY][MPX]
@@ -582,7 +583,8 @@ __global__ void __launch_bounds__(NT, MINB)
 // out = m + dt J^T m + a1 x1 + a2 x2.
 template <typename T, bool VISC>
 __global__ void __launch_bounds__(256) vjp3_finish_kernel(const VjpArgs<T> A, const Gas<T> g,
-                                                          const T* __restrict__ Gacc) {
+                                                          const T* Gacc) {
+  follow_predecessor();
   const long long N = A.N;
   const T dt = T(*A.dt);
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < N; q += (long long)gridDim.x * blockDim.x) {

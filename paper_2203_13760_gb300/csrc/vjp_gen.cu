@@ -53,8 +53,7 @@ cudaError_t launch_face(const GVjpBatch<T>& B, const Gas<T>& g, long long nf, cu
     if (e != cudaSuccess) return e;
   }
   const long long blocks = (nf + kGvjpThreads - 1) / kGvjpThreads;
-  gvjp_face_kernel<T, DIM, RECON, FLUX><<<(unsigned)blocks, kGvjpThreads, smem, s>>>(B, g);
-  return cudaGetLastError();
+  return launch_next(gvjp_face_kernel<T, DIM, RECON, FLUX>, dim3((unsigned)blocks), kGvjpThreads, smem, s, B, g);
 }
 
 template <typename T, int DIM>
@@ -84,8 +83,8 @@ jf_status gvjp_stage(jf_ctx* h, const Gas<T>& g, std::vector<GVjpArgs<T>>& sims,
       B.cell_base[k + 1] = B.cell_base[k] + B.sim[k].N;
     }
     const long long nf = B.face_base[B.nsim];
-    gvjp_point_kernel<T><<<reduce_blocks(B.cell_base[B.nsim], h->sms), 256, 0, s>>>(B);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e =
+        launch_next(gvjp_point_kernel<T>, dim3(reduce_blocks(B.cell_base[B.nsim], h->sms)), 256u, 0, s, B);
     if (e != cudaSuccess) return cuda_fail(h, e, "adjoint: point launch");
     e = h->dim == 1 ? launch_face_dim<T, 1>(B, g, nf, recon, nn, s)
                     : (h->dim == 2 ? launch_face_dim<T, 2>(B, g, nf, recon, nn, s)
@@ -94,9 +93,9 @@ jf_status gvjp_stage(jf_ctx* h, const Gas<T>& g, std::vector<GVjpArgs<T>>& sims,
     if (nn && theta_bar) {
       const long long chunks = (nf + 31) / 32;
       const long long blocks = std::min<long long>((chunks + kNnWarps - 1) / kNnWarps, 2LL * h->sms);
-      nn_param_grad_kernel<T><<<(unsigned)blocks, 32 * kNnWarps, nn_grad_smem_bytes<T>(), s>>>(
-          g.nn, B.sim[0].rec, nf, theta_bar);
-      if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(h, e, "adjoint: parameter-gradient launch");
+      e = launch_next(nn_param_grad_kernel<T>, dim3((unsigned)blocks), 32 * kNnWarps, nn_grad_smem_bytes<T>(), s, g.nn,
+                      B.sim[0].rec, nf, theta_bar);
+      if (e != cudaSuccess) return cuda_fail(h, e, "adjoint: parameter-gradient launch");
     }
   }
   return JF_OK;
@@ -472,9 +471,9 @@ jf_status batch_param_grad_end(jf_ctx* h, void* theta_bar, cudaStream_t s) {
   if ((st = network<T>(h, g)) != JF_OK) return st;
   const long long chunks = (n + 31) / 32;
   const long long blocks = std::min<long long>((chunks + kNnWarps - 1) / kNnWarps, 2LL * h->sms);
-  nn_param_grad_kernel<T><<<(unsigned)blocks, 32 * kNnWarps, nn_grad_smem_bytes<T>(), s>>>(
-      g.nn, static_cast<const T*>(h->rec_store), n, static_cast<T*>(theta_bar));
-  const cudaError_t e = cudaGetLastError();
+  const cudaError_t e =
+      launch_next(nn_param_grad_kernel<T>, dim3((unsigned)blocks), 32 * kNnWarps, nn_grad_smem_bytes<T>(), s, g.nn,
+                  static_cast<const T*>(h->rec_store), n, static_cast<T*>(theta_bar));
   return e == cudaSuccess ? JF_OK : cuda_fail(h, e, "jf_batch_param_grad_end: launch");
 }
 

@@ -74,6 +74,7 @@ __device__ __forceinline__ int find_sim(const long long* base, int nsim, long lo
 // out = a1 x1 + a2 x2 + a3 x3 + s_in lam, every cell of every grid
 template <typename T>
 __global__ void __launch_bounds__(256) gvjp_point_kernel(const GVjpBatch<T> B) {
+  follow_predecessor();
   const long long total = B.cell_base[B.nsim];
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
@@ -211,7 +212,7 @@ constexpr int kNnTRow = NN_HIDDEN + 4;  // row pitch of W2 and W3 transposed (fe
 constexpr int kNnT1 = kNnParamsPad, kNnT2 = kNnT1 + 4 * NN_HIDDEN, kNnT3 = kNnT2 + NN_HIDDEN * kNnTRow,
               kNnShared = kNnT3 + NN_HIDDEN * kNnTRow;
 template <typename T>
-__device__ __forceinline__ void nn_stage(const T* __restrict__ theta, T* th) {
+__device__ __forceinline__ void nn_stage(const T* theta, T* th) {
   for (int i = threadIdx.x; i < NN_PARAMS; i += blockDim.x) th[i] = theta[i];
   for (int i = threadIdx.x; i < 4 * NN_HIDDEN; i += blockDim.x)
     th[kNnT1 + i % 4 * NN_HIDDEN + i / 4] = theta[kNnW1 + i];
@@ -522,6 +523,7 @@ constexpr size_t gvjp_face_smem_bytes() {
 template <typename T, int DIM, int RECON, int FLUX>
 __global__ void __launch_bounds__(kGvjpThreads, sizeof(T) == 4 ? 5 : 1) gvjp_face_kernel(const GVjpBatch<T> B, const Gas<T> g) {
   extern __shared__ __align__(16) unsigned char gvjp_smem[];
+  follow_predecessor();
   T* th = reinterpret_cast<T*>(gvjp_smem);  // the network parameters (Rusanov-NN)
   T* h1 = th + kNnShared + threadIdx.x * kHRow;
   T* h2 = h1 + kGvjpThreads * kHRow;
@@ -567,7 +569,8 @@ __global__ void __launch_bounds__(kGvjpThreads, sizeof(T) == 4 ? 5 : 1) gvjp_fac
 // per parameter.
 //
 // Bound by the FMA pipe and the shared-memory loads (about 6400 FMA per
-// record).  Whole rows in 16-byte loads (pitch 36) and packed FMA: @@
+// record).  Whole rows in 16-byte loads (pitch 36) and packed FMA: 753 ->
+// 505 us for the 30 face passes of a training step (32^2, batch 5).
 constexpr int kNnWarps = 6;  // two blocks per SM by shared memory (FP32)
 constexpr int kNnWarpElems = 3 * 32 * kHRow + 32 * 5;  // three row sets, inputs, output cotangents
 template <typename T>
@@ -577,10 +580,11 @@ constexpr size_t nn_grad_smem_bytes() {
 static_assert(kNnWarpElems >= NN_PARAMS, "the warps' row sets hold their sums at the end");
 
 template <typename T>
-__global__ void __launch_bounds__(32 * kNnWarps, sizeof(T) == 4 ? 2 : 1) nn_param_grad_kernel(const T* __restrict__ theta,
-                                                                      const T* __restrict__ rec, long long nrec,
+__global__ void __launch_bounds__(32 * kNnWarps, sizeof(T) == 4 ? 2 : 1) nn_param_grad_kernel(const T* theta,
+                                                                      const T* rec, long long nrec,
                                                                       T* grad) {
   extern __shared__ __align__(16) unsigned char nn_smem[];
+  follow_predecessor();
   T* TH = reinterpret_cast<T*>(nn_smem);
   nn_stage(theta, TH);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

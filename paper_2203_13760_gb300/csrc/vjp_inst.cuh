@@ -18,8 +18,7 @@ cudaError_t launch_vjp(const VjpArgs<T>& A, const Gas<T>& g, T*, cudaStream_t s)
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const dim3 grid((A.n[0] + BX - 1) / BX, (A.n[1] + BY - 1) / BY);
-  k<<<grid, BX * BY, smem, s>>>(A, g);
-  return cudaGetLastError();
+  return launch_next(k, grid, BX * BY, smem, s, A, g);
 }
 
 // 3D: clear the accumulator, the z-marching face kernel, the per-cell pass.
@@ -40,12 +39,10 @@ cudaError_t launch_vjp3(const VjpArgs<T>& A, const Gas<T>& g, T* Gacc, cudaStrea
   zc = zc < 4 ? 4 : (zc > 32 ? 32 : zc);
   const int zchunk = (int)zc;
   const dim3 grid((A.n[0] + BX - 1) / BX, (A.n[1] + BY - 1) / BY, (A.n[2] + zchunk - 1) / zchunk);
-  k<<<grid, NT, smem, s>>>(A, g, Gacc, zchunk);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = launch_next(k, grid, NT, smem, s, A, g, Gacc, zchunk)) != cudaSuccess) return e;
   long long blocks = (A.N + 255) / 256;
   if (blocks > 16LL * sms) blocks = 16LL * sms;
-  vjp3_finish_kernel<T, VISC><<<(unsigned)blocks, 256, 0, s>>>(A, g, Gacc);
-  return cudaGetLastError();
+  return launch_next(vjp3_finish_kernel<T, VISC>, dim3((unsigned)blocks), 256u, 0, s, A, g, static_cast<const T*>(Gacc));
 }
 
 // Launcher for (dim, visc) in precision T (null if none is compiled).
