@@ -33,10 +33,12 @@
 // separable steps (cell-centre derivative cotangents, then a gather pass) and
 // the tasks are ordered for conflict-free banks.
 //
-// Bound by instruction issue (45 % of the slots at 16 warps per SM).
-// Measured, 256^2 FP32 viscous (256 boxes, one wave): 23.1 us per launch; with
-// atomics in the place of the stepped additions 26.8; face by face (every face
-// reconstructed and reversed on its own, 30 atomics each) 31.5.
+// Bound by the latency of dependent arithmetic and shared memory (45 % of the
+// issue slots at 16 warps per SM) and the barriers between the steps.
+// Measured, 256^2 FP32 viscous (256 boxes, one wave, 256 threads): 23.1 us per
+// launch; with atomics in the place of the stepped additions 26.8; face by face
+// (every face reconstructed and reversed on its own, 30 atomics each) 31.5.
+// With 384 threads a step's three launches take 67.2 us, with 256 70.2.
 #pragma once
 #include "stage.cuh"
 #include <type_traits>
@@ -68,7 +70,6 @@ struct VGeo {
   static constexpr int NCW = VISC ? 6 : 5;
   static constexpr int MX = 3, MY = DIM >= 2 ? 3 : 0;  // m halo
   static constexpr int MPX = BX + 2 * MX, MPY = BY + 2 * MY, MCS = MPX * MPY;
-  static constexpr int NT = BX * BY;
   // cotangents accumulate over the box and a 5-cell halo (every cell a
   // stencil reaches), with no ownership test per addition; boxes near a
   // non-periodic boundary fold ghost cells onto the cells they copy afterwards
@@ -156,9 +157,9 @@ struct VTile {
   }
 };
 
-// The stage VJP kernel.  blockDim.x == BX * BY, grid = (ceil(nx/BX), ceil(ny/BY)).
-template <typename T, int DIM, bool VISC, int BX, int BY, int MINB>
-__global__ void __launch_bounds__(BX * BY, MINB) vjp_stage_kernel(const VjpArgs<T> A, const Gas<T> g) {
+// The stage VJP kernel.  blockDim.x == NT >= BX * BY, grid = (ceil(nx/BX), ceil(ny/BY)).
+template <typename T, int DIM, bool VISC, int BX, int BY, int MINB, int NT>
+__global__ void __launch_bounds__(NT, MINB) vjp_stage_kernel(const VjpArgs<T> A, const Gas<T> g) {
   using G = VGeo<BX, BY, DIM, VISC>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   follow_predecessor();
@@ -173,7 +174,7 @@ __global__ void __launch_bounds__(BX * BY, MINB) vjp_stage_kernel(const VjpArgs<
 
   // stage W (halo 5) and m = s_in lam (halo 3; zero on zero-gradient ghosts)
   bool bad = false;
-  for (int t = tid; t < G::CS; t += G::NT) {
+  for (int t = tid; t < G::CS; t += NT) {
     const int lx = t % G::PX, ly = t / G::PX;
     const int gx = map_index(g0[0] + lx - G::HX, A.n[0], A.periodic[0]);
     const int gy = DIM >= 2 ? map_index(g0[1] + ly - G::HY, A.n[1], A.periodic[1]) : 0;
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(BX * BY, MINB) vjp_stage_kernel(const VjpArgs<
     if (VISC) Wb[5 * G::CS + t] = p * inv * g.inv_R;
   }
   if (bad) atomicOr(A.flag, 1);
-  for (int t = tid; t < G::MCS; t += G::NT) {
+  for (int t = tid; t < G::MCS; t += NT) {
     const int lx = t % G::MPX, ly = t / G::MPX;
     const int r[2] = {g0[0] + lx - G::MX, DIM >= 2 ? g0[1] + ly - G::MY : 0};
     bool ghost = false;
@@ -203,7 +204,7 @@ __global__ void __launch_bounds__(BX * BY, MINB) vjp_stage_kernel(const VjpArgs<
 #pragma unroll
     for (int c = 0; c < 5; ++c) Mb[c * G::MCS + t] = ghost ? T(0) : A.s_in * A.lam[q + c * A.N];
   }
-  for (int t = tid; t < (6 * DIM + G::NCB) * G::ACS; t += G::NT) acc[t] = T(0);
+  for (int t = tid; t < (6 * DIM + G::NCB) * G::ACS; t += NT) acc[t] = T(0);
   __syncthreads();
 
   VTile<T, DIM, VISC, BX, BY> V;
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(BX * BY, MINB) vjp_stage_kernel(const VjpArgs<
     cell_fwd<T, d>(V, position(dtag, s - 3, o), g.eps, e, e + 5 * cs, cs);
   };
   constexpr int f0 = (BX + 6) * CX, f1 = DIM >= 2 ? (BY + 6) * BX : 0;
-  for (int f = tid; f < f0 + f1; f += G::NT) {
+  for (int f = tid; f < f0 + f1; f += NT) {
     if (f < f0) fwd(X{}, std::integral_constant<int, BX + 6>{}, std::integral_constant<int, CX>{}, f);
     else if constexpr (DIM >= 2) fwd(Y{}, std::integral_constant<int, BY + 6>{}, std::integral_constant<int, BX>{}, f - f0);
   }
@@ -285,7 +286,7 @@ __global__ void __launch_bounds__(BX * BY, MINB) vjp_stage_kernel(const VjpArgs<
     }
   };
   constexpr int c0 = (BX + 5) * CX, c1 = DIM >= 2 ? (BY + 5) * BX : 0;
-  for (int f = tid; f < c0 + c1; f += G::NT) {
+  for (int f = tid; f < c0 + c1; f += NT) {
     if (f < c0) conv(X{}, std::integral_constant<int, BX + 5>{}, std::integral_constant<int, CX>{}, f);
     else if constexpr (DIM >= 2) conv(Y{}, std::integral_constant<int, BY + 5>{}, std::integral_constant<int, BX>{}, f - c0);
   }
@@ -299,7 +300,7 @@ __global__ void __launch_bounds__(BX * BY, MINB) vjp_stage_kernel(const VjpArgs<
   // pass 3: the cells -2 .. B + 1 from the cotangents of their two values
   constexpr int r0 = (BX + 4) * CX, r1 = DIM >= 2 ? (BY + 4) * BX : 0;
 #pragma unroll 1
-  for (int f0 = 0; f0 < r0 + r1; f0 += G::NT) {
+  for (int f0 = 0; f0 < r0 + r1; f0 += NT) {
     const int f = f0 + tid;
     T vb[5][5];
     int s = 0, o = 0;
@@ -340,7 +341,7 @@ __global__ void __launch_bounds__(BX * BY, MINB) vjp_stage_kernel(const VjpArgs<
       return true;
     };
 #pragma unroll 1
-    for (int f0 = 0; f0 < v0 + v1; f0 += G::NT) {
+    for (int f0 = 0; f0 < v0 + v1; f0 += NT) {
       const int f = f0 + tid;
       ViscCot<T> out;
       int s = 0, o = 0;
@@ -370,7 +371,7 @@ __global__ void __launch_bounds__(BX * BY, MINB) vjp_stage_kernel(const VjpArgs<
     }
   }
   if constexpr (DIM >= 2) {  // one accumulator from here on
-    for (int t = tid; t < 6 * G::ACS; t += G::NT) acc[t] += acc[6 * G::ACS + t];
+    for (int t = tid; t < 6 * G::ACS; t += NT) acc[t] += acc[6 * G::ACS + t];
     __syncthreads();
   }
 
@@ -379,7 +380,7 @@ __global__ void __launch_bounds__(BX * BY, MINB) vjp_stage_kernel(const VjpArgs<
     // sum_o dcw[o] cb(Y - dco[o] e) (dco = -2, -1, 1, 2; dcw = (1, -8, 8, -1) / 12).
     // Slots: x faces (tangent y) 0: du/dy -> u, 1: dv/dy -> v;
     // y faces (tangent x) 2: dv/dx -> v, 3: du/dx -> u.
-    for (int t = tid; t < G::ACS; t += G::NT) {
+    for (int t = tid; t < G::ACS; t += NT) {
       const int lx = t % G::APX, ly = t / G::APX;
       // (cells beyond the accumulation region hold no cotangent)
       auto spread = [&](int slot, int step, int pos, int len) {
@@ -412,7 +413,7 @@ __global__ void __launch_bounds__(BX * BY, MINB) vjp_stage_kernel(const VjpArgs<
       fold |= !A.periodic[a] && (g0[a] - h < 0 || g0[a] + B + h > A.n[a]);
     }
     if (fold) {
-      for (int t = tid; t < G::ACS; t += G::NT) {
+      for (int t = tid; t < G::ACS; t += NT) {
         const int lx = t % G::APX - G::AX, ly = t / G::APX - G::AY;
         const int ox = V.owner(lx, g0[0], A.n[0], A.periodic[0], BX);
         const int oy = DIM >= 2 ? V.owner(ly, g0[1], A.n[1], A.periodic[1], BY) : 0;
@@ -429,7 +430,7 @@ __global__ void __launch_bounds__(BX * BY, MINB) vjp_stage_kernel(const VjpArgs<
   // cells: cotangent of W (+T) -> cotangent of U, then the stage combination
   const int tx = tid % BX, ty = tid / BX;
   const int gx = g0[0] + tx, gy = g0[1] + ty;
-  if (gx < A.n[0] && gy < A.n[1]) {
+  if (tid < BX * BY && gx < A.n[0] && gy < A.n[1]) {
     const T r = V.w(0, tx, ty, 0), u = V.w(1, tx, ty, 0), v = V.w(2, tx, ty, 0), w = V.w(3, tx, ty, 0);
     const T p = V.w(4, tx, ty, 0);
     const int cell = (ty + G::AY) * G::APX + tx + G::AX;

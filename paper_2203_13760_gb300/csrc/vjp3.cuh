@@ -30,12 +30,16 @@
 //    W(U) and T = p / (rho R) to G and forms the stage combination.
 //
 // Summation order of the atomics, and so the last bits, may vary between
-// runs, as in the box kernel.
+// runs.
 //
-// Bound by instruction issue at 16 warps per SM (one CTA of 512 threads fills
-// the shared memory).  32 x 8 cells give 768 convective and 768 dissipative
-// faces per plane, three tasks per thread.  Measured, 128^3 FP32 viscous: 933 us
-// per launch (932 face by face); its error against 64 bits is half of that.
+// Bound by latency at 18 warps per SM (one CTA fills the shared memory): a
+// scheduler issues in 44 % of its cycles, the rest are waits for barriers,
+// shared memory and dependent arithmetic.  A warp takes a row of a full tile
+// (no bank conflicts along x), and the threads of a CTA (vjp_f32.cu) fill the
+// rounds of the passes.  Measured, 128^3 FP32 viscous, a step and its
+// adjoint: 3901 us with 512 threads and rows of BX + 1 tasks, 3788 with the
+// warps on rows, 3583 with 576 threads (adjoint alone 3214 -> 3004 us).  Its error against 64 bits is half of that of a
+// face-by-face pass.
 #pragma once
 #include "vjp.cuh"
 
@@ -294,12 +298,12 @@ __global__ void __launch_bounds__(NT, MINB)
   // the cells -1 .. f - 1 are beside them
   const int fx = ex + ((!A.periodic[0] && x0 + BX >= nx) ? 1 : 0);
   const int fy = ey + ((!A.periodic[1] && y0 + BY >= ny) ? 1 : 0);
-  // task decoding divides by fx, fx + 1 and ex (1 .. BX + 2): for d >= 2,
+  // task decoding divides by fx and ex (1 .. BX + 1): for d >= 2,
   // r / d = (r m_d) >> 32 with m_d = ceil(2^32 / d) < 2^32, exact for
   // r < 2^16 (the error r (m_d - 2^32/d) / 2^32 < 2^-16 stays below 1/d);
   // d = 1 keeps r (m = 0 flags it)
   auto recip = [](int d) { return d > 1 ? 0xffffffffu / (unsigned)d + 1u : 0u; };
-  const unsigned mfx = recip(fx), mcx = recip(fx + 1), mex = recip(ex);
+  const unsigned mfx = recip(fx), mex = recip(ex);
   auto divu = [](int r, unsigned m) { return m ? (int)__umulhi((unsigned)r, m) : r; };
   const T inv_h[3] = {A.inv_h[0], A.inv_h[1], A.inv_h[2]};
 
@@ -402,6 +406,22 @@ __global__ void __launch_bounds__(NT, MINB)
   using Y = std::integral_constant<int, 1>;
   using Z = std::integral_constant<int, 2>;
   const int ncol = ex * ey;
+  // task r of a pass over the cells: first the tile's own cells along x, so
+  // that a warp holds one row of a full tile, then `others`, then the rim
+  // cells along x (-1, and ex on a boundary)
+  auto x_task = [&](int r, int ncx, int others, int& j, int& i) -> bool {
+    if (ncx == 0) return false;
+    if (r < ncol) {
+      j = divu(r, mex);
+      i = r - j * ex;
+      return true;
+    }
+    r -= ncol + others;
+    if (r < 0) return false;
+    i = r < ey ? -1 : ex;
+    j = r < ey ? r : r - ey;
+    return true;
+  };
 
   // the upper values of the cells of plane z0 - 1
   set_view(z0 - 1);
@@ -422,12 +442,11 @@ __global__ void __launch_bounds__(NT, MINB)
     const int ncx = xy ? ey * (fx + 1) : 0, ncy = xy ? (fy + 1) * ex : 0, nzf = k < z1 ? ncol : 0;
     // pass 1: face values of the cells along x and y (plane k), z (plane k + 1)
     for (int t = threadIdx.x; t < ncx + ncy + nzf; t += NT) {
-      int r = t;
-      if (r < ncx) {
-        const int j = divu(r, mcx), i = r - j * (fx + 1);  // cell i - 1
-        T* e = EX + j * G::XP + i;
-        cell_fwd<T, 0>(V, Along<0>{{i - 1, j, 0}}, g.eps, e, e + 5 * G::XS, G::XS);
-      } else if ((r -= ncx) < ncy) {
+      int r = t, j, i;
+      if (x_task(r, ncx, ncy + nzf, j, i)) {
+        T* e = EX + j * G::XP + i + 1;
+        cell_fwd<T, 0>(V, Along<0>{{i, j, 0}}, g.eps, e, e + 5 * G::XS, G::XS);
+      } else if ((r -= ncx ? ex * ey : 0) < ncy) {
         const int j = divu(r, mex), i = r - j * ex;  // cell row j - 1
         T* e = EY + j * BX + i;
         cell_fwd<T, 1>(V, Along<1>{{i, j - 1, 0}}, g.eps, e, e + 5 * G::YS, G::YS);
@@ -511,11 +530,10 @@ __global__ void __launch_bounds__(NT, MINB)
     // pass 3: reverse reconstruction of the cells
     const int nz3 = xy || k == nz || (bottom && k < z0) ? ncol : 0;
     for (int t = threadIdx.x; t < ncx + ncy + nz3; t += NT) {
-      int r = t;
-      if (r < ncx) {
-        const int j = divu(r, mcx), i = r - j * (fx + 1);
-        rev(X{}, i - 1, j, EX + j * G::XP + i, G::XS);
-      } else if ((r -= ncx) < ncy) {
+      int r = t, j, i;
+      if (x_task(r, ncx, ncy + nz3, j, i)) {
+        rev(X{}, i, j, EX + j * G::XP + i + 1, G::XS);
+      } else if ((r -= ncx ? ex * ey : 0) < ncy) {
         const int j = divu(r, mex), i = r - j * ex;
         rev(Y{}, i, j - 1, EY + j * BX + i, G::YS);
       } else {

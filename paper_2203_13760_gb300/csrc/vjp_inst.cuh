@@ -11,14 +11,14 @@ namespace jf {
 template <typename T>
 using VjpLaunch = cudaError_t (*)(const VjpArgs<T>& A, const Gas<T>& g, T* scratch, cudaStream_t s);
 
-template <typename T, int DIM, bool VISC, int BX, int BY, int MINB>
+template <typename T, int DIM, bool VISC, int BX, int BY, int MINB, int NT>
 cudaError_t launch_vjp(const VjpArgs<T>& A, const Gas<T>& g, T*, cudaStream_t s) {
   constexpr size_t smem = vjp_smem_bytes<T, DIM, VISC, BX, BY>();
-  auto k = vjp_stage_kernel<T, DIM, VISC, BX, BY, MINB>;
+  auto k = vjp_stage_kernel<T, DIM, VISC, BX, BY, MINB, NT>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const dim3 grid((A.n[0] + BX - 1) / BX, (A.n[1] + BY - 1) / BY);
-  return launch_next(k, grid, BX * BY, smem, s, A, g);
+  return launch_next(k, grid, NT, smem, s, A, g);
 }
 
 // 3D: clear the accumulator, the z-marching face kernel, the per-cell pass.

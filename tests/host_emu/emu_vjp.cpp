@@ -55,13 +55,13 @@ static void launch(dim3 grid, int threads, size_t smem, F body) {
       }
 }
 
-template <typename T, int DIM, bool VISC, int BX, int BY>
+template <typename T, int DIM, bool VISC, int BX, int BY, int NT>
 static void box(const VjpArgs<T>& A, const Gas<T>& g) {
   dim3 grid;
   grid.x = (A.n[0] + BX - 1) / BX;
   grid.y = (A.n[1] + BY - 1) / BY;
-  launch(grid, BX * BY, vjp_smem_bytes<T, DIM, VISC, BX, BY>(),
-         [&] { vjp_stage_kernel<T, DIM, VISC, BX, BY, 1>(A, g); });
+  launch(grid, NT, vjp_smem_bytes<T, DIM, VISC, BX, BY>(),
+         [&] { vjp_stage_kernel<T, DIM, VISC, BX, BY, 1, NT>(A, g); });
 }
 
 template <typename T, bool VISC, int BX, int BY, int NT>
@@ -118,12 +118,12 @@ static int run(std::ifstream& in, const char* path) {
   constexpr bool f32 = sizeof(T) == 4;
   const bool visc = h[7];
   if (h[2] > 1) {
-    if (visc) march<T, true, f32 ? 32 : 16, f32 ? 8 : 4, f32 ? 512 : 128>(A, g, h[6]);
-    else march<T, false, f32 ? 32 : 16, 8, f32 ? 512 : 256>(A, g, h[6]);
+    if (visc) march<T, true, f32 ? 32 : 16, f32 ? 8 : 4, f32 ? 576 : 224>(A, g, h[6]);
+    else march<T, false, f32 ? 32 : 16, 8, f32 ? 576 : 320>(A, g, h[6]);
   } else if (h[1] > 1) {
-    if (visc) box<T, 2, true, 16, 16>(A, g); else box<T, 2, false, 16, 16>(A, g);
+    if (visc) box<T, 2, true, 16, 16, 384>(A, g); else box<T, 2, false, 16, 16, 384>(A, g);
   } else {
-    if (visc) box<T, 1, true, 128, 1>(A, g); else box<T, 1, false, 128, 1>(A, g);
+    if (visc) box<T, 1, true, 128, 1, 160>(A, g); else box<T, 1, false, 128, 1, 160>(A, g);
   }
   std::ofstream(path, std::ios::binary).write((char*)out.get(), sizeof(T) * 5 * N);
   return flag;
