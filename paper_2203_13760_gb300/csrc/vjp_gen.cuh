@@ -155,6 +155,17 @@ struct HRow {
       for (int m = 0; m < 4; ++m) v[j + m] += s * q[m];
     }
   }
+  // as a 4 x 8 block: += the products of g[0 .. 3] and h[0 .. 7] (16-byte aligned)
+  __device__ __forceinline__ void outer(const T* g, const T* h) {
+    T a[4], b[8];
+    ld4(g, a);
+    ld4(h, b);
+    ld4(h + 4, b + 4);
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+      for (int c = 0; c < 8; ++c) v[8 * m + c] += a[m] * b[c];
+  }
   __device__ __forceinline__ T get(int j) const { return v[j]; }
   __device__ __forceinline__ void set(int j, T x) { v[j] = x; }
   __device__ __forceinline__ void store(T* row) const {
@@ -185,6 +196,16 @@ struct HRow<float> {
       v[j / 2] = __ffma2_rn(make_float2(q.x, q.y), s2, v[j / 2]);
       v[j / 2 + 1] = __ffma2_rn(make_float2(q.z, q.w), s2, v[j / 2 + 1]);
     }
+  }
+  __device__ __forceinline__ void outer(const float* g, const float* h) {
+    const float4 a = *reinterpret_cast<const float4*>(g);
+    const float4 p = *reinterpret_cast<const float4*>(h), q = *reinterpret_cast<const float4*>(h + 4);
+    const float am[4] = {a.x, a.y, a.z, a.w};
+    const float2 b[4] = {make_float2(p.x, p.y), make_float2(p.z, p.w), make_float2(q.x, q.y), make_float2(q.z, q.w)};
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[4 * m + c] = __ffma2_rn(make_float2(am[m], am[m]), b[c], v[4 * m + c]);
   }
   __device__ __forceinline__ float get(int j) const { return j & 1 ? v[j / 2].y : v[j / 2].x; }
   __device__ __forceinline__ void set(int j, float x) {
@@ -562,15 +583,17 @@ __global__ void __launch_bounds__(kGvjpThreads, sizeof(T) == 4 ? 5 : 1) gvjp_fac
 // memory, and each warp takes chunks of 32 records (one per lane).  Per
 // chunk, each lane evaluates the network of its record and the cotangents of
 // every layer (seed d alpha / d o = alpha, scaled by abar) into shared rows,
-// reusing rows once they are consumed; then lane L adds row L of every weight
-// gradient summed over the 32 records (dW[L][k] = sum_f G[f][L] H[f][k]) to
-// accumulators kept in registers across chunks.  At the end the block sums its
+// reusing rows once they are consumed; then the lanes add the weight gradients
+// summed over the 32 records (dW[i][k] = sum_f G[f][i] H[f][k]) to accumulators
+// kept in registers across chunks, each lane 4 x 8 entries of a 32 x 32 layer.  At the end the block sums its
 // warps' accumulators in shared memory and adds them to grad with one atomic
 // per parameter.
 //
 // Bound by the FMA pipe and the shared-memory loads (about 6400 FMA per
 // record).  Whole rows in 16-byte loads (pitch 36) and packed FMA: 753 ->
-// 505 us for the 30 face passes of a training step (32^2, batch 5).
+// 505 us for the 1.27 million records of a training step (20 boxes of 32^2, 15
+// RK2 steps); 4 x 8 blocks in the place of a row per lane, three loads for 16
+// packed multiply-adds and not ten: 464 us.
 constexpr int kNnWarps = 6;  // two blocks per SM by shared memory (FP32)
 constexpr int kNnWarpElems = 3 * 32 * kHRow + 32 * 5;  // three row sets, inputs, output cotangents
 template <typename T>
@@ -595,7 +618,9 @@ __global__ void __launch_bounds__(32 * kNnWarps, sizeof(T) == 4 ? 2 : 1) nn_para
   T* X = R3 + 32 * kHRow;       // [32][4]
   T* OB = X + 32 * 4;           // [32]
   __syncthreads();
-  // row `lane` of every gradient, accumulated over this warp's chunks
+  // this lane's 4 x 8 block of the gradients of W3 and W2 and entry `lane` of
+  // the others, accumulated over this warp's chunks
+  const int br = 4 * (lane >> 2), bc = 8 * (lane & 3);
   HRow<T> a3, a2;
   T a1[4] = {T(0), T(0), T(0), T(0)};
   a3.fill(T(0));
@@ -622,7 +647,7 @@ __global__ void __launch_bounds__(32 * kNnWarps, sizeof(T) == 4 ? 2 : 1) nn_para
     OB[lane] = ob;
     v.store(r3);
     __syncwarp();
-    // layers 4 and 3 (H3 in R3, H2 in R2): G3 = OB W4 where H3 > 0
+    // layer 4 (H3 in R3) and b3: G3 = OB W4 where H3 > 0
 #pragma unroll 2
     for (int r = 0; r < 32; ++r) {
       const T h3 = R3[r * kHRow + lane], b = OB[r];
@@ -630,13 +655,16 @@ __global__ void __launch_bounds__(32 * kNnWarps, sizeof(T) == 4 ? 2 : 1) nn_para
       ab3 += g3;
       a4 += b * h3;
       ab4 += b;
-      a3.axpy(R2 + r * kHRow, g3);
     }
     __syncwarp();
-    // G2 into R3: g2[j] = [h2_j > 0] sum_i W3[i][j] g3[i]; g3 over the lane's own H3 row first
+    // layer 3: G3 into R3 (H2 in R2)
 #pragma unroll
     for (int j = 0; j < NN_HIDDEN; ++j) v.set(j, v.get(j) > T(0) ? ob * TH[kNnW4 + j] : T(0));
     v.store(r3);
+    __syncwarp();
+#pragma unroll 2
+    for (int r = 0; r < 32; ++r) a3.outer(R3 + r * kHRow + br, R2 + r * kHRow + bc);
+    // G2 into R3: g2[j] = [h2_j > 0] sum_i W3[i][j] g3[i]
     v.fill(T(0));
     nn_rows<NN_HIDDEN>(TH + kNnW3, r3, v);
 #pragma unroll
@@ -646,14 +674,14 @@ __global__ void __launch_bounds__(32 * kNnWarps, sizeof(T) == 4 ? 2 : 1) nn_para
 #pragma unroll
       for (int m = 0; m < 4; ++m) v.set(j + m, q[m] > T(0) ? v.get(j + m) : T(0));
     }
+    __syncwarp();
     v.store(r3);
     __syncwarp();
     // layer 2 (G2 in R3, H1 in R1)
 #pragma unroll 2
     for (int r = 0; r < 32; ++r) {
-      const T g2 = R3[r * kHRow + lane];
-      ab2 += g2;
-      a2.axpy(R1 + r * kHRow, g2);
+      ab2 += R3[r * kHRow + lane];
+      a2.outer(R3 + r * kHRow + br, R1 + r * kHRow + bc);
     }
     __syncwarp();
     // G1 into R3: g1[k] = [h1_k > 0] sum_j W2[j][k] g2[j]
@@ -690,9 +718,14 @@ __global__ void __launch_bounds__(32 * kNnWarps, sizeof(T) == 4 ? 2 : 1) nn_para
 #pragma unroll
   for (int m = 0; m < 4; ++m) Sw[kNnW1 + 4 * L + m] = a1[m];
   Sw[kNnB1 + L] = ab1;
-  a2.store(Sw + kNnW2 + NN_HIDDEN * L);
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      Sw[kNnW2 + NN_HIDDEN * (br + m) + bc + c] = a2.get(8 * m + c);
+      Sw[kNnW3 + NN_HIDDEN * (br + m) + bc + c] = a3.get(8 * m + c);
+    }
   Sw[kNnB2 + L] = ab2;
-  a3.store(Sw + kNnW3 + NN_HIDDEN * L);
   Sw[kNnB3 + L] = ab3;
   Sw[kNnW4 + L] = a4;
   if (L == 0) Sw[kNnB4] = ab4;
