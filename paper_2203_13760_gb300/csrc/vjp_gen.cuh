@@ -234,13 +234,13 @@ constexpr int kNnT1 = kNnParamsPad, kNnT2 = kNnT1 + 4 * NN_HIDDEN, kNnT3 = kNnT2
               kNnShared = kNnT3 + NN_HIDDEN * kNnTRow;
 template <typename T>
 __device__ __forceinline__ void nn_stage(const T* theta, T* th) {
-  for (int i = threadIdx.x; i < NN_PARAMS; i += blockDim.x) th[i] = theta[i];
-  for (int i = threadIdx.x; i < 4 * NN_HIDDEN; i += blockDim.x)
-    th[kNnT1 + i % 4 * NN_HIDDEN + i / 4] = theta[kNnW1 + i];
+  block_copy(theta, NN_PARAMS, [&](int i, T v) { th[i] = v; });
+  __syncthreads();
+  for (int i = threadIdx.x; i < 4 * NN_HIDDEN; i += blockDim.x) th[kNnT1 + i % 4 * NN_HIDDEN + i / 4] = th[kNnW1 + i];
   for (int i = threadIdx.x; i < NN_HIDDEN * NN_HIDDEN; i += blockDim.x) {
     const int t = i % NN_HIDDEN * kNnTRow + i / NN_HIDDEN;
-    th[kNnT2 + t] = theta[kNnW2 + i];
-    th[kNnT3 + t] = theta[kNnW3 + i];
+    th[kNnT2 + t] = th[kNnW2 + i];
+    th[kNnT3 + t] = th[kNnW3 + i];
   }
 }
 
