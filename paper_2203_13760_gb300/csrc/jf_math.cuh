@@ -849,75 +849,113 @@ __host__ __device__ __noinline__ T nn_alpha(const T* th, const T x[4]) {
   return texp(out);
 }
 
+// The transposed weights for nn_alpha_pair: W1 [4][NN_HIDDEN], then W2 and W3
+// [NN_HIDDEN][NN_TPITCH], a row per input.
+constexpr int NN_TPITCH = NN_HIDDEN + 4, NN_T2 = 4 * NN_HIDDEN, NN_T3 = NN_T2 + NN_HIDDEN * NN_TPITCH,
+              NN_TELEMS = NN_T3 + NN_HIDDEN * NN_TPITCH;
+// Where parameter i goes in them (-1: a bias or W4, not there).
+JF_HD int nn_transposed(int i) {
+  constexpr int W2 = 5 * NN_HIDDEN, W3 = W2 + (NN_HIDDEN + 1) * NN_HIDDEN;
+  if (i < 4 * NN_HIDDEN) return i % 4 * NN_HIDDEN + i / 4;
+  if (i >= W2 && i < W2 + NN_HIDDEN * NN_HIDDEN) return NN_T2 + (i - W2) % NN_HIDDEN * NN_TPITCH + (i - W2) / NN_HIDDEN;
+  if (i >= W3 && i < W3 + NN_HIDDEN * NN_HIDDEN) return NN_T3 + (i - W3) % NN_HIDDEN * NN_TPITCH + (i - W3) / NN_HIDDEN;
+  return -1;
+}
+
 #ifdef __CUDACC__
-// nn_alpha of two faces in packed FP32x2 lanes, from the parameters stored
-// twice each (th2[k] = (theta_k, theta_k), 16-byte aligned): per lane the
-// operations of nn_alpha in its order, so the same bits.  A layer runs over its
-// inputs four at a time (from `row`, this thread's NN_PAIR_ROW pairs of shared
-// memory) with all its outputs in registers: independent sums, and a loop whose
-// code stays in the instruction cache (unrolled over both layers the pass was
-// bound by instruction fetch).
-constexpr int NN_PAIR_ROW = NN_HIDDEN + 2;  // 17 x 16 bytes: conflict-free 16-byte accesses
-static __device__ __noinline__ float2 nn_alpha_pair(const float2* th2, const float2 x[4], float2* row) {
-  const float2* b1 = th2 + NN_HIDDEN * 4;
-  const float2* W2 = b1 + NN_HIDDEN;
-  const float2* b2 = W2 + NN_HIDDEN * NN_HIDDEN;
-  const float2* W3 = b2 + NN_HIDDEN;
-  const float2* b3 = W3 + NN_HIDDEN * NN_HIDDEN;
-  const float2* W4 = b3 + NN_HIDDEN;
-  auto ld2 = [](const float2* p, float2& a, float2& b) {
+// nn_alpha of two faces (the lanes of x), from the parameters th and the
+// transposed weights tt (16-byte aligned): per face the operations of nn_alpha
+// in its order, so the same bits.  Two outputs of a layer share a packed FP32x2
+// operation, so that four weights of one load serve both faces: with every
+// weight stored twice and the faces in the lanes a pass took twice the loads, and
+// the stage of 20 boxes of 32^2 18.6 us in the place of 16.4.
+// A layer runs over its inputs four at a time (from `row`, this thread's
+// NN_PAIR_ROW values of shared memory) with all its outputs in registers:
+// independent sums, and a loop whose code stays in the instruction cache.
+constexpr int NN_PAIR_ROW = 2 * NN_HIDDEN + 4;  // 17 x 16 bytes: conflict-free 16-byte accesses
+static __device__ __noinline__ float2 nn_alpha_pair(const float* th, const float* tt, const float2 x[4], float* row) {
+  const float* b1 = th + NN_HIDDEN * 4;
+  const float* b2 = b1 + NN_HIDDEN + NN_HIDDEN * NN_HIDDEN;
+  const float* b3 = b2 + NN_HIDDEN + NN_HIDDEN * NN_HIDDEN;
+  const float* W4 = b3 + NN_HIDDEN;
+  auto ld2 = [](const float* p, float2& a, float2& b) {
     const float4 q = *reinterpret_cast<const float4*>(p);
     a = make_float2(q.x, q.y);
     b = make_float2(q.z, q.w);
   };
-  auto relu = [](float2 z) { return make_float2(tmax(0.0f, z.x), tmax(0.0f, z.y)); };
-  float2 z[NN_HIDDEN];
-  auto keep = [&]() {  // the layer's values to this thread's row
+  auto splat = [](float v) { return make_float2(v, v); };
+  float2 zx[NN_HIDDEN / 2], zy[NN_HIDDEN / 2];
+  auto bias = [&](const float* b) {
 #pragma unroll
-    for (int i = 0; i < NN_HIDDEN; i += 2) {
-      const float2 a = relu(z[i]), b = relu(z[i + 1]);
-      *reinterpret_cast<float4*>(row + i) = make_float4(a.x, a.y, b.x, b.y);
+    for (int i = 0; i < NN_HIDDEN / 2; i += 2) {
+      ld2(b + 2 * i, zx[i], zx[i + 1]);
+      zy[i] = zx[i];
+      zy[i + 1] = zx[i + 1];
     }
   };
-  auto layer = [&](const float2* W, const float2* b) {
+  auto keep = [&]() {  // the layer's values to this thread's row
 #pragma unroll
-    for (int i = 0; i < NN_HIDDEN; i += 2) ld2(b + i, z[i], z[i + 1]);
+    for (int i = 0; i < NN_HIDDEN / 2; i += 2) {
+      *reinterpret_cast<float4*>(row + 2 * i) = make_float4(tmax(0.0f, zx[i].x), tmax(0.0f, zx[i].y),
+                                                            tmax(0.0f, zx[i + 1].x), tmax(0.0f, zx[i + 1].y));
+      *reinterpret_cast<float4*>(row + NN_HIDDEN + 2 * i) = make_float4(tmax(0.0f, zy[i].x), tmax(0.0f, zy[i].y),
+                                                                        tmax(0.0f, zy[i + 1].x), tmax(0.0f, zy[i + 1].y));
+    }
+  };
+  auto layer = [&](const float* W, const float* b) {
+    bias(b);
 #pragma unroll 1
     for (int j = 0; j < NN_HIDDEN; j += 4) {
-      float2 h0, h1, h2, h3;
-      ld2(row + j, h0, h1);
-      ld2(row + j + 2, h2, h3);
+      float hx[4], hy[4];
+      ld4(row + j, hx);
+      ld4(row + NN_HIDDEN + j, hy);
 #pragma unroll
-      for (int i = 0; i < NN_HIDDEN; ++i) {
-        float2 w0, w1, w2, w3;
-        ld2(W + NN_HIDDEN * i + j, w0, w1);
-        ld2(W + NN_HIDDEN * i + j + 2, w2, w3);
-        const float2 t = __ffma2_rn(w3, h3, __ffma2_rn(w2, h2, __ffma2_rn(w0, h0, __fmul2_rn(w1, h1))));
-        z[i] = __fadd2_rn(z[i], t);
+      for (int i = 0; i < NN_HIDDEN / 2; i += 2) {
+        float2 w[4][2];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) ld2(W + (j + m) * NN_TPITCH + 2 * i, w[m][0], w[m][1]);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          auto sum = [&](const float h[4]) {
+            return __ffma2_rn(w[3][q], splat(h[3]), __ffma2_rn(w[2][q], splat(h[2]),
+                                                               __ffma2_rn(w[0][q], splat(h[0]), __fmul2_rn(w[1][q], splat(h[1])))));
+          };
+          zx[i + q] = __fadd2_rn(zx[i + q], sum(hx));
+          zy[i + q] = __fadd2_rn(zy[i + q], sum(hy));
+        }
       }
     }
   };
+  bias(b1);
+#pragma unroll
+  for (int i = 0; i < NN_HIDDEN / 2; i += 2)
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      float2 w[2];
+      ld2(tt + NN_HIDDEN * m + 2 * i, w[0], w[1]);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        zx[i + q] = __ffma2_rn(w[q], splat(x[m].x), zx[i + q]);
+        zy[i + q] = __ffma2_rn(w[q], splat(x[m].y), zy[i + q]);
+      }
+    }
+  keep();
+  layer(tt + NN_T2, b2);
+  keep();
+  layer(tt + NN_T3, b3);
+  float ox = W4[NN_HIDDEN], oy = ox;
 #pragma unroll
   for (int i = 0; i < NN_HIDDEN; ++i) {
-    float2 w0, w1, w2, w3;
-    ld2(th2 + 4 * i, w0, w1);
-    ld2(th2 + 4 * i + 2, w2, w3);
-    z[i] = __ffma2_rn(w3, x[3], __ffma2_rn(w2, x[2], __ffma2_rn(w1, x[1], __ffma2_rn(w0, x[0], b1[i]))));
+    const float w = W4[i];
+    ox = fmaf(w, tmax(0.0f, i & 1 ? zx[i / 2].y : zx[i / 2].x), ox);
+    oy = fmaf(w, tmax(0.0f, i & 1 ? zy[i / 2].y : zy[i / 2].x), oy);
   }
-  keep();
-  layer(W2, b2);
-  keep();
-  layer(W3, b3);
-  float2 out = W4[NN_HIDDEN];
-#pragma unroll
-  for (int i = 0; i < NN_HIDDEN; ++i) out = __ffma2_rn(W4[i], relu(z[i]), out);
-  return make_float2(texp(out.x), texp(out.y));
+  return make_float2(texp(ox), texp(oy));
 }
 #else
-constexpr int NN_PAIR_ROW = 0;  // host: lane by lane, no hidden rows
-inline float2 nn_alpha_pair(const float2* th2, const float2 x[4], float2*) {
-  float th[NN_PARAMS], a[4], b[4];
-  for (int k = 0; k < NN_PARAMS; ++k) th[k] = th2[k].x;
+constexpr int NN_PAIR_ROW = 0;  // host: face by face, no hidden rows
+inline float2 nn_alpha_pair(const float* th, const float*, const float2 x[4], float*) {
+  float a[4], b[4];
   for (int m = 0; m < 4; ++m) { a[m] = x[m].x; b[m] = x[m].y; }
   return make_float2(nn_alpha(th, a), nn_alpha(th, b));
 }

@@ -41,7 +41,7 @@ namespace jf {
 
 constexpr int HALO = 3;
 // Rusanov-NN parameters in shared memory (nn_smem_elems)
-constexpr int kNnPairs = (NN_PARAMS + 3) / 4 * 4, kNnRows = kNnPairs + (2 * NN_PARAMS + 3) / 4 * 4;
+constexpr int kNnTrans = (NN_PARAMS + 3) / 4 * 4, kNnRows = kNnTrans + NN_TELEMS;
 
 // Kernel dimensionality (template parameter DIM).  1, 2 and 3 are the grid's
 // active axes: the tile spans x (1D: one row of BX cells; 2D, 3D: BX x BY
@@ -1166,9 +1166,8 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
       float2 in[4];
 #pragma unroll
       for (int m = 0; m < 4; ++m) in[m] = make_float2(x[m], y[m]);
-      const float2* th2 = reinterpret_cast<const float2*>(g.nn + kNnPairs);
-      float2* rows = reinterpret_cast<float2*>(const_cast<float*>(g.nn) + kNnRows);
-      const float2 alpha = nn_alpha_pair(th2, in, rows + threadIdx.x * NN_PAIR_ROW);
+      float* row = const_cast<float*>(g.nn) + kNnRows + threadIdx.x * NN_PAIR_ROW;
+      const float2 alpha = nn_alpha_pair(g.nn, g.nn + kNnTrans, in, row);
       if (xf_x >= 0) {
         rusanov_nn<T, 0>(Xm, Xp, g, F, alpha.x);
         T NF[5];
@@ -1407,11 +1406,11 @@ constexpr size_t nn_smem_offset() {
 }
 
 // Elements of the parameters there: the network's, and in the FP32 kernels of
-// tiles spanning y a copy with every value twice and the threads' hidden rows
-// (nn_alpha_pair), from the elements kNnPairs and kNnRows.
+// tiles spanning y the transposed weights and the threads' hidden rows
+// (nn_alpha_pair), from the elements kNnTrans and kNnRows.
 template <typename T, int DIM, int NT>
 constexpr size_t nn_smem_elems() {
-  return sizeof(T) == 4 && plane_dims(DIM) == 2 ? kNnRows + (size_t)2 * NN_PAIR_ROW * NT : NN_PARAMS;
+  return sizeof(T) == 4 && plane_dims(DIM) == 2 ? kNnRows + (size_t)NN_PAIR_ROW * NT : NN_PARAMS;
 }
 
 // The stage kernel.  blockDim.x == Geo::NT.
@@ -1460,7 +1459,10 @@ __global__ void __launch_bounds__(Geo<BX, BY, DIM, VISC>::NT, MINB)
     T* th = reinterpret_cast<T*>(smem_raw) + nn_smem_offset<T, DIM, VISC, BX, BY>();
     block_copy(g.nn, NN_PARAMS, [&](int i, T v) {
       th[i] = v;
-      if constexpr (nn_smem_elems<T, DIM, 0>() > NN_PARAMS) th[kNnPairs + 2 * i] = th[kNnPairs + 2 * i + 1] = v;
+      if constexpr (nn_smem_elems<T, DIM, 0>() > NN_PARAMS) {
+        const int t = nn_transposed(i);
+        if (t >= 0) th[kNnTrans + t] = v;
+      }
     });
     __syncthreads();
     gk.nn = th;
