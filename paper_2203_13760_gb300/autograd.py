@@ -17,10 +17,10 @@ a fixed step).
 ``feed_forward(batch, U0s, n, dt, theta=None)``
                               Section 4.5: the trajectories of a batch of
                               (uneven) simulations, differentiable w.r.t. the
-                              initial states (reverse sweep on the stored
-                              trajectory with jf_rk3_step_vjp) and, for the
-                              Rusanov-NN flux of Section 7.4, w.r.t. the
-                              network parameters theta (jf_rk3_step_vjp_params).
+                              initial states and, for the Rusanov-NN flux of
+                              Section 7.4, w.r.t. the network parameters theta
+                              (jf_batch_feed_forward_vjp: the reverse sweep on
+                              the stored trajectories in one call).
 ``trajectory_mse(trajs, refs)``
                               Section 7.2: 1/N_T sum_i MSE(U^i, U^i_ref).
 ``primitive_mse(owner, U, Uref, ncomp=4)``

@@ -2,7 +2,7 @@
 // extended forms: slip walls (mirrored ghost cells) and WENO3-JS on top of
 // the Table 2 choices.  The host picks them only for grids with a wall side or
 // the WENO3-JS reconstruction, so the plain forms keep their register budget.
-// One tile shape per dimensionality and physics.
+// 2D: 32 x 7 (default) and 32 x 4 (jf_set_variant).
 // Compiled with the same approximate division and square root as stage_f32.cu.
 #include "stage_inst.cuh"
 

@@ -1,4 +1,5 @@
-// Instantiations of the stage kernel in FP64 (IEEE division and square root).
+// Instantiations of the stage kernel in FP64 (divisions and square roots:
+// approximation and Newton steps, trcp / tsqrt).
 #include <vector>
 
 #include "stage_inst.cuh"
@@ -12,10 +13,10 @@ template <>
 const StageVariant<double>* stage_variants<double>(int* count) {
   static const std::vector<StageVariant<double>> table = [] {
     std::vector<StageVariant<double>> v = {
-      // 3D (the first entry per configuration is the default): 32 x 6, one
-      // CTA of 7 warps per SM (208 KB of shared memory), measured at TGV 256^3
-      // 82.2 M cell-updates/s against 68.8 M for 32 x 4 (5 warps) and 49.1 M
-      // for 32 x 2 at two CTAs per SM
+      // 3D (the first entry per configuration is the default): 32 x 7, one
+      // CTA of 8 warps per SM, the z state of a column in registers (with
+      // it, the carried viscous stencils and the tile 32 x 6 -> 32 x 7 the
+      // 128^3 step went from 22.7 to 20.3 ms)
       make_variant<double, 3, true, 32, 7, 1, SCH_DEFAULT>(),
       make_variant<double, 3, true, 32, 4, 1, SCH_DEFAULT>(),
       make_variant<double, 3, true, 32, 2, 2, SCH_DEFAULT>(),

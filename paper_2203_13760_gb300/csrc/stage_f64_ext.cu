@@ -1,7 +1,7 @@
 // FP64 stage kernels of the run-time-scheme and ROE families in their
 // extended forms: slip walls (mirrored ghost cells) and WENO3-JS on top of
 // the Table 2 choices.  The host picks them only for grids with a wall side or
-// the WENO3-JS reconstruction.  One tile shape per dimensionality and physics.
+// the WENO3-JS reconstruction.  2D: the tile shapes of stage_f64.cu.
 #include "stage_inst.cuh"
 
 namespace jf {

@@ -1,7 +1,6 @@
 // FP64 stage kernels with the scheme chosen at run time (Table 2 variants:
-// HLL / Rusanov fluxes, Davis / Toro signal speeds, WENO5-Z), one tile shape
-// per dimensionality and physics; in 3D also 32 x 4 beside the default 32 x 6
-// (HLL at TGV 128^3: 78.3 against 66.4 M cell-updates/s).
+// HLL / Rusanov fluxes, Davis / Toro signal speeds, WENO5-Z), in the tile
+// shapes of stage_f64.cu.
 #include "stage_inst.cuh"
 
 namespace jf {
