@@ -34,12 +34,12 @@
 //
 // Bound by latency at 18 warps per SM (one CTA fills the shared memory): a
 // scheduler issues in 50 % of its cycles (44 % with 512 threads), the rest are
-// waits for barriers, shared memory and dependent arithmetic.  A warp takes a row of a full tile
-// (no bank conflicts along x), and the threads of a CTA (vjp_f32.cu) fill the
-// rounds of the passes.  Measured, 128^3 FP32 viscous, a step and its
-// adjoint: 3901 us with 512 threads and rows of BX + 1 tasks, 3788 with the
-// warps on rows, 3583 with 576 threads (adjoint alone 3214 -> 3004 us).  Its error against 64 bits is half of that of a
-// face-by-face pass.
+// waits for barriers, shared memory and dependent arithmetic.  A warp takes a
+// row of a full tile (no bank conflicts along x), and the threads of a CTA
+// (vjp_f32.cu) fill the rounds of the passes.  Measured, 128^3 FP32 viscous, a
+// step and its adjoint: 3901 us with 512 threads and rows of BX + 1 tasks, 3788
+// with the warps on rows, 3583 with 576 threads (adjoint alone 3214 -> 3004 us).
+// Its error against 64 bits is half of that of a face-by-face pass.
 #pragma once
 #include "vjp.cuh"
 
