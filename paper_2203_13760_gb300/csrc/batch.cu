@@ -88,6 +88,9 @@ jf_status setup_variant(jf_ctx* h, int v) {
         const StageVariant<T>& t0 = tab[list[0].first];
         if (rows_preferred(h->grids.data(), h->nsim, r.bx, r.minb, t0.bx, t0.by, h->sms)) v = i;
         break;
+      } else if (sizeof(T) == 4 && h->dim == 2 && scheme_kind(h) == SCH_GENERAL_EXT && tab[list[i].first].by == 8) {
+        const StageVariant<T>& t0 = tab[list[0].first];
+        if (tall_tiles_preferred(h->grids.data(), h->nsim, t0.bx, t0.by, 8, 2 * h->sms)) v = i;
       }
   }
   if (v >= (int)list.size()) { set_error(h, "batch: variant index out of range"); return JF_ERR_ARG; }

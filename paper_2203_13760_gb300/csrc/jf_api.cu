@@ -251,6 +251,24 @@ bool rows_preferred(const jf_grid* grids, int n, int rows_bx, int rows_ctas_per_
   return rows <= 1.08 * tiles && row_tiles >= 12.0 * sms * (rows_ctas_per_sm > 0 ? rows_ctas_per_sm : 1);
 }
 
+// 2D FP32 grids of the extended run-time schemes (walls, WENO3-JS): tiles of
+// `tall` rows (more useful cells per halo row, but their extra warp halves the
+// registers' slack) in the place of `by`.  Over many waves of `slots` resident
+// CTAs the taller tile is faster, and wherever it saves a wave; up to two equal
+// waves the lower one is.  Measured, walled WENO3 stage, 32 x 7 and 32 x 8: 256^2
+// 4.87 and 5.38 us, 300^2 7.68 and 7.95, 384^2 10.76 (three waves) and 9.22 (two),
+// 512^2 15.4 and 15.1, 1024^2 54.1 and 51.2.
+bool tall_tiles_preferred(const jf_grid* grids, int n, int bx, int by, int tall, int slots) {
+  long long t = 0, q = 0;
+  for (int i = 0; i < n; ++i) {
+    const long long c = (grids[i].nx + bx - 1) / bx;
+    t += c * ((grids[i].ny + by - 1) / by);
+    q += c * ((grids[i].ny + tall - 1) / tall);
+  }
+  const long long s = slots > 0 ? slots : 1, wt = (t + s - 1) / s, wq = (q + s - 1) / s;
+  return wq < wt || wt > 2;
+}
+
 // 2D FP64 grids: the FP64 pipe is shared by an SM's warps, so a launch takes
 // the busiest SM's tiles times the warp tasks of a tile (2 BY + 3
 // reconstructions and 2 BY + 2 faces).  The tile shape with the fewest: small
@@ -287,6 +305,9 @@ jf_status select_variant(jf_ctx* h, int v, bool prepare) {
         const StageVariant<T>& t0 = tab[list[0].first];
         if (rows_preferred(&h->grid, 1, r.bx, r.minb, t0.bx, t0.by, h->sms)) v = i;
         break;
+      } else if (sizeof(T) == 4 && h->dim == 2 && scheme_kind(h) == SCH_GENERAL_EXT && tab[list[i].first].by == 8) {
+        const StageVariant<T>& t0 = tab[list[0].first];
+        if (tall_tiles_preferred(&h->grid, 1, t0.bx, t0.by, 8, 2 * h->sms)) v = i;
       }
   }
   if (v >= (int)list.size()) { set_error(h, "variant index out of range"); return JF_ERR_ARG; }

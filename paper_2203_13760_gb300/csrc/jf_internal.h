@@ -141,6 +141,7 @@ bool dissipative(const jf_gas& gas, const jf_scheme& s);
 // or WENO3-JS; a walled grid with the default scheme runs SCH_GENERAL_EXT),
 // or SCH_NN (Rusanov-NN)
 bool has_walls(const jf_grid& g);
+bool tall_tiles_preferred(const jf_grid* grids, int n, int bx, int by, int tall, int slots);
 int scheme_kind(const jf_scheme& s, bool walls);
 int scheme_kind(const jf_ctx* h);
 CflArgs make_cfl(const jf_grid& g, const jf_gas& gas, const jf_scheme& s);
