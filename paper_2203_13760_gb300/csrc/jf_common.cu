@@ -45,7 +45,11 @@ void Staging::release() {
 
 bool being_captured(cudaStream_t s) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();  // answered here: not left for the next caller's check
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
 }
 
 jf_status alloc_common(jf_ctx* h) {

@@ -81,7 +81,9 @@ cudaError_t launch_next(void (*kernel)(P...), dim3 grid, unsigned threads, size_
   cfg.stream = s;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+  if (e != cudaSuccess) cudaGetLastError();  // returned here: not left for the next caller's check
+  return e;
 }
 #endif
 
