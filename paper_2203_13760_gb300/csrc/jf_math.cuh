@@ -118,8 +118,9 @@ constexpr int NN_PARAMS = 32 * 4 + 32 + 2 * (32 * 32 + 32) + 32 + 1;
 // Chebyshev's y + y (e + e^2) with e = 1 - x y and Halley's
 // s + s e (1/2 + 3/8 e) with e = 1 - x y^2: 3 and 5 FP64 operations, where an
 // IEEE division or square root takes about ten and the FP64 pipe (2 FMA per
-// clock and SM) is what bounds the FP64 kernels.  The results are within 1
-// ulp (measured over exponents -1000..1000).  FP32: against __fdividef, whose
+// clock and SM) is what bounds the FP64 kernels.  Zero, infinity and NaN give
+// what IEEE division and square root give; arguments and results below 2^-1022
+// count as zero.  FP32: against __fdividef, whose
 // multiplication it saves, the same bits, and the ROE step at 128^3 takes 903
 // instead of 941 us, the default one at 256^3 4.205 instead of 4.264 ms.
 template <typename T> JF_HD T trcp(T x);
@@ -136,8 +137,10 @@ template <> JF_HD double trcp<double>(double x) {
 #ifdef __CUDA_ARCH__
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
+  const double e = fma(-x, y, 1.0), r = fma(y, fma(e, e, e), y);
+  // 1/0, 1/inf, 1/NaN: the approximation is the result, and e would be NaN
+  // (its exponent field is 0 or 0x7ff; 32-bit operations)
+  return ((__double2hiint(y) + 0x00100000) & 0x7fe00000) == 0 ? y : r;
 #else
   return 1.0 / x;
 #endif
@@ -163,7 +166,9 @@ template <> JF_HD double tsqrt<double>(double x) {
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double r = x * y, e = fma(-r, y, 1.0);
   const double s = fma(r * e, fma(0.375, e, 0.5), r);
-  return __double2hiint(x) == 0 ? 0.0 : s;  // sqrt(0) (a 32-bit compare)
+  // sqrt(+-0) and sqrt(inf) are x itself (32-bit operations)
+  const int hi = __double2hiint(x);
+  return (hi & 0x7ff00000) == 0 || hi == 0x7ff00000 ? x : s;
 #else
   return sqrt(x);
 #endif

@@ -1,0 +1,44 @@
+"""The FP64 reciprocal and square root of the point-wise numerics as the device
+evaluates them (a PTX approximation and refinement steps; host code divides, so
+only a GPU sees them), against IEEE arithmetic."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+RCP, SQRT = 0, 1
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    so = tmp_path_factory.mktemp("point_math") / "point_math.so"
+    subprocess.run([nvcc, "-gencode", "arch=compute_103a,code=sm_103a", "-std=c++17", "-O3", "--expt-relaxed-constexpr",
+                    "-shared", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "paper_2203_13760_gb300", "csrc"),
+                    os.path.join(ROOT, "tests", "gpu_checks", "point_math.cu"), "-o", str(so)], check=True)
+    return ctypes.CDLL(str(so))
+
+
+def _unary(lib, f, x):
+    dx = torch.tensor(x, dtype=torch.float64, device="cuda")
+    dy = torch.empty_like(dx)
+    torch.cuda.synchronize()
+    assert lib.pm_unary(f, ctypes.c_void_p(dx.data_ptr()), ctypes.c_void_p(dy.data_ptr()), dx.numel()) == 0
+    return dy.cpu().numpy()
+
+
+def test_special_values(lib):
+    """Zeros, infinities, NaN and negative arguments as in IEEE arithmetic."""
+    inf, nan = np.inf, np.nan
+    x = np.array([0.0, -0.0, inf, -inf, nan, 1.0, -2.0, 2.0**-1022, 2.0**1000])
+    with np.errstate(all="ignore"):
+        for f, want in ((RCP, 1.0 / x), (SQRT, np.sqrt(x))):
+            got = _unary(lib, f, x)
+            assert np.array_equal(got, want, equal_nan=True), (f, got, want)
+            assert np.array_equal(np.signbit(got[want == 0]), np.signbit(want[want == 0]))
