@@ -114,11 +114,14 @@ constexpr int NN_PARAMS = 32 * 4 + 32 + 2 * (32 * 32 + 32) + 32 + 1;
 // takes the hardware approximations (rcp.approx.ftz: one MUFU operation,
 // within 1 ulp for |x| < 2^126; host code divides exactly).  FP64 device code
 // starts from the PTX approximations rcp / rsqrt.approx.ftz.f64 (about 20
-// bits, not on the FP64 pipe) and refines them with one third-order step,
-// Chebyshev's y + y (e + e^2) with e = 1 - x y and Halley's
-// s + s e (1/2 + 3/8 e) with e = 1 - x y^2: 3 and 5 FP64 operations, where an
-// IEEE division or square root takes about ten and the FP64 pipe (2 FMA per
-// clock and SM) is what bounds the FP64 kernels.  Zero, infinity and NaN give
+// bits, not on the FP64 pipe) and refines them: the reciprocal with one
+// third-order step (Chebyshev), y + y (e + e^2) with e = 1 - x y; the root
+// r = x y with two Newton steps r + (x - r^2) y / 2, whose residuals a fused
+// multiply-add forms exactly.  3 and 5 FP64 operations, where an IEEE division
+// or square root takes about ten and the FP64 pipe (2 FMA per clock and SM) is
+// what bounds the FP64 kernels.  The last operation rounds a correction of some
+// 2^-20 (2^-40) of the result, so the error stays within 0.51 ulp; a form that
+// rounds x y and takes one third-order step from it reaches 0.75.  Zero, infinity and NaN give
 // what IEEE division and square root give; arguments and results below 2^-1022
 // count as zero.  FP32: against __fdividef, whose
 // multiplication it saves, the same bits, and the ROE step at 128^3 takes 903
@@ -146,26 +149,14 @@ template <> JF_HD double trcp<double>(double x) {
 #endif
 }
 
-// 1 / sqrt(x) in FP64 (x > 0).
-JF_HD double trsqrt(double x) {
-#ifdef __CUDA_ARCH__
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x * y, y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-#else
-  return 1.0 / sqrt(x);
-#endif
-}
-
 template <typename T> JF_HD T tsqrt(T x);
 template <> JF_HD float tsqrt<float>(float x) { return sqrtf(x); }
 template <> JF_HD double tsqrt<double>(double x) {
 #ifdef __CUDA_ARCH__
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double r = x * y, e = fma(-r, y, 1.0);
-  const double s = fma(r * e, fma(0.375, e, 0.5), r);
+  const double h = __hiloint2double(__double2hiint(y) - 0x00100000, __double2loint(y));  // y / 2
+  const double r = x * y, r1 = fma(fma(-r, r, x), h, r), s = fma(fma(-r1, r1, x), h, r1);
   // sqrt(+-0) and sqrt(inf) are x itself (32-bit operations)
   const int hi = __double2hiint(x);
   return (hi & 0x7ff00000) == 0 || hi == 0x7ff00000 ? x : s;
@@ -577,17 +568,15 @@ JF_HD void side_state(const T W[5], const Gas<T>& g, T& E, T& ir, T& c) {
   c = tsqrt(g.gamma * W[4] * ir);
 }
 
-// Both sides' E, 1/rho and c, and q = sqrt(rho_R / rho_L); FP64 forms the
-// reciprocals and q from one inverse square root y = (rho_L rho_R)^(-1/2):
-// q = rho_R y, 1/rho_L = q y, 1/rho_R = rho_L y^2.
+// Both sides' E, 1/rho and c, and q = sqrt(rho_R / rho_L); FP64 forms the two
+// reciprocals from one, 1/rho_L = rho_R / (rho_L rho_R) and the converse.
 template <typename T>
 JF_HD void side_states(const T WL[5], const T WR[5], const Gas<T>& g, T& EL, T& ER, T& irL, T& irR, T& q, T& cL,
                        T& cR) {
   if constexpr (sizeof(T) == 8) {
-    const T y = trsqrt(WL[0] * WR[0]);
-    q = WR[0] * y;
-    irL = q * y;
-    irR = WL[0] * y * y;
+    const T inv = trcp(WL[0] * WR[0]);
+    irL = WR[0] * inv;
+    irR = WL[0] * inv;
     EL = WL[4] * g.inv_gm1 + T(0.5) * WL[0] * (WL[1] * WL[1] + WL[2] * WL[2] + WL[3] * WL[3]);
     ER = WR[4] * g.inv_gm1 + T(0.5) * WR[0] * (WR[1] * WR[1] + WR[2] * WR[2] + WR[3] * WR[3]);
     cL = tsqrt(g.gamma * WL[4] * irL);
@@ -595,8 +584,8 @@ JF_HD void side_states(const T WL[5], const T WR[5], const Gas<T>& g, T& EL, T& 
   } else {
     side_state(WL, g, EL, irL, cL);
     side_state(WR, g, ER, irR, cR);
-    q = tsqrt(WR[0] * irL);
   }
+  q = tsqrt(WR[0] * irL);
 }
 
 // Physical flux along D and conservative state of one side.
@@ -631,7 +620,7 @@ JF_HD bool not_negative(double x) {
 template <int D>
 JF_HD void hllc_einfeldt(const double WL[5], const double WR[5], const Gas<double>& g, double F[5]) {
   const double rL = WL[0], rR = WR[0], pL = WL[4], pR = WR[4], unL = WL[1 + D], unR = WR[1 + D];
-  const double y = trsqrt(rL * rR), q = rR * y, irL = q * y, irR = rL * y * y;
+  const double inv = trcp(rL * rR), irL = rR * inv, irR = rL * inv, q = tsqrt(rR * irL);
   const double aL = g.gamma * pL * irL, aR = g.gamma * pR * irR;  // c_K^2
   const double wL = trcp(1.0 + q), wR = q * wL;
   const double du = WR[1] - WL[1], dv = WR[2] - WL[2], dw = WR[3] - WL[3];

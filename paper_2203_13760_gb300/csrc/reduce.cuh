@@ -55,20 +55,20 @@ __device__ __forceinline__ double warp_sum(double v) {
 
 // Per-cell rates of the CFL criterion, folded into running maxima: the wave
 // rate max_d |u_d| + c over the active axes and the diffusion rate kdiff / rho.
-// Computed in the field's precision (FP64 units are scarce on this part); the
+// Computed in the field's precision with IEEE division and root (the step is a
+// reported number); the
 // maxima are later formed in FP64, and a rate converted to FP64 is exact, so
 // the result is the exact maximum of the per-cell values.
 template <typename T>
 __device__ __forceinline__ void cell_rates_of(T r, T ru, T rv, T rw, T E, int nactive, T gamma, T gm1, T kdiff,
                                               T& conv, T& diff, bool& bad) {
-  T inv;
-  if constexpr (sizeof(T) == 8) inv = trcp(r); else inv = T(1) / r;
+  const T inv = T(1) / r;
   const T u = ru * inv;
   const T v = rv * inv;
   const T w = rw * inv;
   const T p = gm1 * (E - T(0.5) * r * (u * u + v * v + w * w));
   bad |= !(r > T(0)) || !(p > T(0));
-  const T c = tsqrt(gamma * p * inv);
+  const T c = sqrt(gamma * p * inv);
   T m = fabs(u);
   if (nactive > 1) m = fmax(m, fabs(v));
   if (nactive > 2) m = fmax(m, fabs(w));

@@ -42,3 +42,18 @@ def test_special_values(lib):
             got = _unary(lib, f, x)
             assert np.array_equal(got, want, equal_nan=True), (f, got, want)
             assert np.array_equal(np.signbit(got[want == 0]), np.signbit(want[want == 0]))
+
+
+@pytest.mark.parametrize("f,order", [(RCP, 1.0), (SQRT, 1.5)])
+def test_rounding(lib, f, order):
+    """Error against extended precision, over random mantissas and exponents.
+    The approximations keep the upper 20 bits of argument and result, so their
+    relative error is e <= 2^-19; the steps leave `order` e^3 and one rounding."""
+    rng = np.random.default_rng(17)
+    x = np.concatenate([rng.uniform(1, 4, 200000), 1 + rng.integers(0, 1 << 20, 50000) * 2.0**-52,
+                        rng.uniform(1, 2, 200000) * 2.0 ** rng.integers(-1000, 1000, 200000)])
+    got = _unary(lib, f, x)
+    X = x.astype(np.longdouble)
+    want = 1 / X if f == RCP else np.sqrt(X)
+    ulp = float(np.max(np.abs(got.astype(np.longdouble) - want) / np.spacing(got)))
+    assert ulp <= 0.5 + order * 2.0**-57 / 2.0**-53 + 0.01, ulp
