@@ -610,9 +610,12 @@ JF_HD void side_flux(const T W[5], T E, T F[5], T U[5]) {
 //   c~^2 = w_L c_L^2 + w_R c_R^2 + (gamma - 1)/2 w_L w_R |u_R - u_L|^2
 // (the identity behind H~ - |u~|^2/2, without its cancellation), the energy of
 // the chosen side only, and signs read from the high words.
+// x >= 0 by 32-bit compares: +0 to +inf, or -0; false for the NaN of an invalid
+// side, whose face must not pass as the regular flux of the other one.
 JF_HD bool not_negative(double x) {
 #ifdef __CUDA_ARCH__
-  return __double2hiint(x) >= 0;
+  const unsigned hi = (unsigned)__double2hiint(x);
+  return hi <= 0x7ff00000u || hi == 0x80000000u;
 #else
   return x >= 0.0;
 #endif

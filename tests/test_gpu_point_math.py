@@ -1,6 +1,6 @@
-"""The FP64 reciprocal and square root of the point-wise numerics as the device
-evaluates them (a PTX approximation and refinement steps; host code divides, so
-only a GPU sees them), against IEEE arithmetic."""
+"""The FP64 reciprocal, square root and HLLC flux of the point-wise numerics as
+the device evaluates them (PTX approximations, refinement steps and integer
+tests; host code takes other branches, so only a GPU sees them)."""
 import ctypes
 import os
 import shutil
@@ -57,3 +57,31 @@ def test_rounding(lib, f, order):
     want = 1 / X if f == RCP else np.sqrt(X)
     ulp = float(np.max(np.abs(got.astype(np.longdouble) - want) / np.spacing(got)))
     assert ulp <= 0.5 + order * 2.0**-57 / 2.0**-53 + 0.01, ulp
+
+
+def _hllc(lib, W, speeds=0, host=False):
+    """W (2, 5, n): left and right states; the fluxes (5, n), on the device or
+    in the host's branch."""
+    dW = torch.tensor(np.ascontiguousarray(W), dtype=torch.float64, device="cpu" if host else "cuda")
+    F = torch.empty((5, W.shape[2]), dtype=torch.float64, device=dW.device)
+    torch.cuda.synchronize()
+    assert lib.pm_hllc(int(host), ctypes.c_void_p(dW.data_ptr()), ctypes.c_void_p(F.data_ptr()), W.shape[2],
+                       ctypes.c_double(1.4), speeds) == 0
+    return F.cpu().numpy()
+
+
+@pytest.mark.parametrize("speeds", [0, 1, 2])
+@pytest.mark.parametrize("side", [0, 1])
+@pytest.mark.parametrize("comp", [0, 4])
+def test_hllc_of_an_invalid_side(lib, speeds, side, comp):
+    """A face with a negative density or pressure on one side (an overshoot of
+    the reconstruction) has NaN wave speeds.  Its flux is NaN on the device
+    where IEEE comparisons, which are false for NaN, make it so."""
+    rng = np.random.default_rng(5)
+    W = rng.uniform(0.5, 1.5, (2, 5, 256))
+    W[:, 1:4] = rng.uniform(-2.0, 2.0, (2, 3, 256))
+    assert np.isfinite(_hllc(lib, W, speeds)).all()
+    W[side, comp] *= -1
+    F, want = _hllc(lib, W, speeds), _hllc(lib, W, speeds, host=True)
+    assert np.array_equal(np.isnan(F), np.isnan(want))
+    assert np.allclose(F, want, rtol=1e-12, atol=1e-12, equal_nan=True)
