@@ -620,6 +620,20 @@ JF_HD bool not_negative(double x) {
   return x >= 0.0;
 #endif
 }
+// S_K (U*_K - U_K) added to the mass, normal momentum and energy flux of a star
+// side (FP64), from theta = (S* - u_n) / (S - S*): with fac = rho (1 + theta)
+//   fac - rho = rho theta,  fac S* - rho u_n = rho (S* - u_n + theta S*),
+//   fac (E/rho + (S* - u_n)(S* + p/m)) - E = E theta + fac (S* - u_n)(S* + p/m),
+// without the cancellation of the left-hand sides and without 1/rho (a
+// contact at rest keeps its fluxes 0, p, 0 exactly).  1 / (S - S*) and p / m from
+// one reciprocal.
+JF_HD void hllc_star(double r, double p, double un, double E, double mass, double S, double m, double Ss, double& F0,
+                     double& Fn, double& F4) {
+  const double d = S - Ss, x = trcp(m * d), k = Ss - un, theta = k * (m * x), rt = r * theta;
+  F0 = fma(S, rt, mass);
+  Fn = fma(S * r, fma(theta, Ss, k), Fn);
+  F4 = fma(S, fma(E, theta, (r + rt) * k * fma(p * d, x, Ss)), F4);
+}
 template <int D>
 JF_HD void hllc_einfeldt(const double WL[5], const double WR[5], const Gas<double>& g, double F[5]) {
   const double rL = WL[0], rR = WR[0], pL = WL[4], pR = WR[4], unL = WL[1 + D], unR = WR[1 + D];
@@ -635,18 +649,13 @@ JF_HD void hllc_einfeldt(const double WL[5], const double WR[5], const Gas<doubl
   const double Ss = fma(-mR, unR, fma(mL, unL, pR - pL)) * trcp(mL - mR);
   const bool sup = not_negative(SL), left = sup || not_negative(Ss);
   const bool star = left ? !sup : SR > 0.0;
-  const double r = left ? rL : rR, p = left ? pL : pR, un = left ? unL : unR, ir = left ? irL : irR;
+  const double r = left ? rL : rR, p = left ? pL : pR, un = left ? unL : unR;
   const double w0 = left ? WL[1] : WR[1], w1 = left ? WL[2] : WR[2], w2 = left ? WL[3] : WR[3];
   const double S = left ? SL : SR, m = left ? mL : mR;
   const double E = fma(0.5 * r, fma(w2, w2, fma(w1, w1, w0 * w0)), p * g.inv_gm1);
   const double mass = r * un;
   double F0 = mass, Fn = fma(mass, un, p), F4 = un * (E + p);
-  if (star) {  // fac and p / m from one reciprocal, as in hllc
-    const double d = S - Ss, x = trcp(m * d), fac = m * m * x, p_m = p * d * x;
-    F0 = fma(S, fac - r, mass);
-    Fn = fma(S, fma(fac, Ss, -mass), Fn);
-    F4 = fma(S, fma(fac, fma(Ss - un, Ss + p_m, E * ir), -E), F4);
-  }
+  if (star) hllc_star(r, p, un, E, mass, S, m, Ss, F0, Fn, F4);
   F[0] = F0;
   F[1] = F0 * w0;
   F[2] = F0 * w1;
@@ -682,7 +691,6 @@ JF_HD void hllc(const T WL[5], const T WR[5], const Gas<T>& g, T F[5], int speed
   const bool left = (SL >= T(0)) || (Ss >= T(0));
   const bool star = left ? !(SL >= T(0)) : (SR > T(0));
   const T r = left ? rL : rR, p = left ? pL : pR, un = left ? unL : unR, E = left ? EL : ER;
-  const T ir = left ? irL : irR;
   const T w0 = left ? WL[1] : WR[1], w1 = left ? WL[2] : WR[2], w2 = left ? WL[3] : WR[3];
   const T S = left ? SL : SR, m = left ? mL : mR;
   // physical flux F_K of the chosen side, plus S_K (U*_K - U_K) on a star
@@ -693,21 +701,16 @@ JF_HD void hllc(const T WL[5], const T WR[5], const Gas<T>& g, T F[5], int speed
   const T mass = r * un;
   T F0 = mass, Fn = mass * un + p, F4 = un * (E + p);
   if (star) {
-    // fac = m / (S - S*) and p / m; FP64 takes both from one division,
-    // x = 1 / (m (S - S*)) (m and S - S* are non-zero on a star side:
-    // S_L < u_L - c_L, S_L < 0 <= S*, and the mirror image)
-    T fac, p_m;
+    // (m and S - S* are non-zero on a star side: S_L < u_L - c_L, S_L < 0 <= S*,
+    // and the mirror image)
     if constexpr (sizeof(T) == 8) {
-      const T d = S - Ss, x = trcp(m * d);
-      fac = m * m * x;
-      p_m = p * d * x;
+      hllc_star(r, p, un, E, mass, S, m, Ss, F0, Fn, F4);
     } else {
-      fac = m * trcp(S - Ss);
-      p_m = p * trcp(m);
+      const T ir = left ? irL : irR, fac = m * trcp(S - Ss), p_m = p * trcp(m);
+      F0 = mass + S * (fac - r);
+      Fn = Fn + S * (fac * Ss - mass);
+      F4 = F4 + S * (fac * (E * ir + (Ss - un) * (Ss + p_m)) - E);
     }
-    F0 = mass + S * (fac - r);
-    Fn = Fn + S * (fac * Ss - mass);
-    F4 = F4 + S * (fac * (E * ir + (Ss - un) * (Ss + p_m)) - E);
   }
   F[0] = F0;
   F[1] = F0 * w0;

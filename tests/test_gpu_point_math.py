@@ -85,3 +85,16 @@ def test_hllc_of_an_invalid_side(lib, speeds, side, comp):
     F, want = _hllc(lib, W, speeds), _hllc(lib, W, speeds, host=True)
     assert np.array_equal(np.isnan(F), np.isnan(want))
     assert np.allclose(F, want, rtol=1e-12, atol=1e-12, equal_nan=True)
+
+
+@pytest.mark.parametrize("speeds", [0, 1, 2])
+def test_contact_at_rest(lib, speeds):
+    """A contact discontinuity at rest: S* = 0 = u_n exactly, so no mass and no
+    energy cross the face and the momentum flux is the pressure."""
+    rng = np.random.default_rng(6)
+    W = np.zeros((2, 5, 256))
+    W[:, 0] = rng.uniform(0.1, 10.0, (2, 256))
+    W[:, 4] = rng.uniform(0.1, 10.0, 256)
+    F = _hllc(lib, W, speeds)
+    assert np.array_equal(F[1], W[0, 4])
+    assert not F[[0, 2, 3, 4]].any()
