@@ -472,19 +472,28 @@ __device__ __forceinline__ void weno5_cell_pair_lean(float2 vm2, float2 vm1, flo
 // v[i-1], v[i], v[i+1]: q0 = (3 v[i] - v[i-1]) / 2, q1 = (v[i] + v[i+1]) / 2,
 // beta0 = (v[i] - v[i-1])^2, beta1 = (v[i+1] - v[i])^2,
 // alpha_k = d_k / (eps + beta_k)^2, d = (1/3, 2/3), omega_k = alpha_k / sum.
+// FP64: in differences, v0 + (r0 e0 + 2 r1 e1) / (2 (r0 + 2 r1)) with e0, e1 and
+// r_k as below: one reciprocal, and its rounding only scales the correction.
 template <typename T>
 JF_HD T weno3(T vm1, T v0, T vp1, T eps) {
-  const T q0 = T(0.5) * (T(3) * v0 - vm1), q1 = T(0.5) * (v0 + vp1);
-  const T t0 = eps + (v0 - vm1) * (v0 - vm1), t1 = eps + (vp1 - v0) * (vp1 - v0);
-  const T a0 = T(1.0 / 3.0) * trcp(t0 * t0), a1 = T(2.0 / 3.0) * trcp(t1 * t1);
-  return (a0 * q0 + a1 * q1) * trcp(a0 + a1);
+  if constexpr (sizeof(T) == 8) {
+    const T e0 = v0 - vm1, e1 = vp1 - v0, t0 = eps + e0 * e0, t1 = eps + e1 * e1;
+    const T r0 = t1 * t1, r1 = T(2) * (t0 * t0);
+    return v0 + (r0 * e0 + r1 * e1) * trcp(T(2) * (r0 + r1));
+  } else {
+    const T q0 = T(0.5) * (T(3) * v0 - vm1), q1 = T(0.5) * (v0 + vp1);
+    const T t0 = eps + (v0 - vm1) * (v0 - vm1), t1 = eps + (vp1 - v0) * (vp1 - v0);
+    const T a0 = T(1.0 / 3.0) * trcp(t0 * t0), a1 = T(2.0 / 3.0) * trcp(t1 * t1);
+    return (a0 * q0 + a1 * q1) * trcp(a0 + a1);
+  }
 }
 // Both WENO3-JS face values of one cell from v[j-1..j+1] (as weno5_cell):
 // with e0 = v0 - v[-1], e1 = v[1] - v0 and r_k = 1 / (eps + e_k^2)^2,
 //   right = v0 + (r0 e0 + 2 r1 e1) / (2 (r0 + 2 r1)),
 //   left  = v0 - (r1 e1 + 2 r0 e0) / (2 (r1 + 2 r0)).
-// FP64: r0, r1 scaled by (eps + e0^2)^2 (eps + e1^2)^2, and one reciprocal
-// for both values.
+// FP64: r0, r1 scaled by (eps + e0^2)^2 (eps + e1^2)^2.  A reciprocal for each
+// value: one for both, of the product of the sums, takes as many operations
+// and ends the range of eps and of the jumps at the fourth root of FP64's.
 template <typename T>
 JF_HD void weno3_cell(T vm1, T v0, T vp1, T eps, T& right, T& left) {
   const T e0 = v0 - vm1, e1 = vp1 - v0;
@@ -500,14 +509,8 @@ JF_HD void weno3_cell(T vm1, T v0, T vp1, T eps, T& right, T& left) {
   const T Sr = r0 + T(2) * r1, Sl = r1 + T(2) * r0;
   const T p0 = r0 * e0, p1 = r1 * e1;
   const T nr = p0 + T(2) * p1, nl = p1 + T(2) * p0;
-  if constexpr (sizeof(T) == 8) {
-    const T inv = trcp(T(2) * Sr * Sl);
-    right = v0 + nr * (Sl * inv);
-    left = v0 - nl * (Sr * inv);
-  } else {
-    right = v0 + nr * trcp(T(2) * Sr);
-    left = v0 - nl * trcp(T(2) * Sl);
-  }
+  right = v0 + nr * trcp(T(2) * Sr);
+  left = v0 - nl * trcp(T(2) * Sl);
 }
 __device__ __forceinline__ float2 weno3_pair(float2 vm1, float2 v0, float2 vp1, float eps) {
   return make_float2(weno3(vm1.x, v0.x, vp1.x, eps), weno3(vm1.y, v0.y, vp1.y, eps));
