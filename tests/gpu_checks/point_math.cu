@@ -1,8 +1,9 @@
-// The point-wise functions of jf_math.cuh as the device evaluates them, one
+// The point-wise functions of jf_math.cuh and vjp_gen.cuh as the device evaluates them, one
 // argument (or pair of face states) per thread, for tests/test_gpu_point_math.py.
 #include <cuda_runtime.h>
 
 #include "jf_math.cuh"
+#include "vjp_gen.cuh"
 
 using namespace jf;
 
@@ -27,6 +28,16 @@ __global__ void hllc_kernel(const double* W, double* F, int n, Gas<double> g, in
   if (i < n) hllc_at(i, W, F, n, g, speeds);
 }
 
+// the cotangent of the x momentum under a unit cotangent of the x velocity: 1 / rho
+__global__ void prim_vjp_kernel(const float* rho, float* out, int n, Gas<float> g) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const float W[5] = {rho[i], 0.3f, -0.2f, 0.1f, 1.0f}, Wb[5] = {0.0f, 1.0f, 0.0f, 0.0f, 0.0f};
+  float Ub[5];
+  prim_vjp(W, g, Wb, Ub);
+  out[i] = Ub[1];
+}
+
 static int finish() {
   const cudaError_t e = cudaGetLastError();
   return (int)(e == cudaSuccess ? cudaDeviceSynchronize() : e);
@@ -48,5 +59,12 @@ extern "C" int pm_hllc(int host, const double* W, double* F, int n, double gamma
     return 0;
   }
   hllc_kernel<<<(n + 255) / 256, 256>>>(W, F, n, g, speeds);
+  return finish();
+}
+
+extern "C" int pm_prim_vjp(const float* rho, float* out, int n) {
+  Gas<float> g{};
+  g.gm1 = 0.4f;
+  prim_vjp_kernel<<<(n + 255) / 256, 256>>>(rho, out, n, g);
   return finish();
 }

@@ -1,6 +1,7 @@
-"""The FP64 reciprocal, square root and HLLC flux of the point-wise numerics as
-the device evaluates them (PTX approximations, refinement steps and integer
-tests; host code takes other branches, so only a GPU sees them)."""
+"""The FP64 reciprocal, square root and HLLC flux of the point-wise numerics and
+the FP32 division of the per-face adjoint as the device evaluates them (PTX
+approximations, refinement steps and integer tests; host code takes other
+branches, so only a GPU sees them)."""
 import ctypes
 import os
 import shutil
@@ -98,3 +99,14 @@ def test_contact_at_rest(lib, speeds):
     F = _hllc(lib, W, speeds)
     assert np.array_equal(F[1], W[0, 4])
     assert not F[[0, 2, 3, 4]].any()
+
+
+def test_fp32_division_of_the_per_face_adjoint(lib):
+    """1 / rho of the conversion's reverse pass is rounded as IEEE division
+    rounds it (no contraction can touch it: the other terms are zero)."""
+    rho = np.random.default_rng(8).uniform(0.1, 10.0, 20000).astype(np.float32)
+    d = torch.tensor(rho, device="cuda")
+    out = torch.empty_like(d)
+    torch.cuda.synchronize()
+    assert lib.pm_prim_vjp(ctypes.c_void_p(d.data_ptr()), ctypes.c_void_p(out.data_ptr()), d.numel()) == 0
+    assert np.array_equal(out.cpu().numpy(), np.float32(1) / rho)
