@@ -478,8 +478,8 @@ template <typename T>
 JF_HD T weno3(T vm1, T v0, T vp1, T eps) {
   if constexpr (sizeof(T) == 8) {
     const T e0 = v0 - vm1, e1 = vp1 - v0, t0 = eps + e0 * e0, t1 = eps + e1 * e1;
-    const T r0 = t1 * t1, r1 = T(2) * (t0 * t0);
-    return v0 + (r0 * e0 + r1 * e1) * trcp(T(2) * (r0 + r1));
+    const T r0 = t1 * t1, r1 = t0 * t0;
+    return fma(fma(T(0.5), r0 * e0, r1 * e1), trcp(fma(T(2), r1, r0)), v0);
   } else {
     const T q0 = T(0.5) * (T(3) * v0 - vm1), q1 = T(0.5) * (v0 + vp1);
     const T t0 = eps + (v0 - vm1) * (v0 - vm1), t1 = eps + (vp1 - v0) * (vp1 - v0);
@@ -492,8 +492,8 @@ JF_HD T weno3(T vm1, T v0, T vp1, T eps) {
 //   right = v0 + (r0 e0 + 2 r1 e1) / (2 (r0 + 2 r1)),
 //   left  = v0 - (r1 e1 + 2 r0 e0) / (2 (r1 + 2 r0)).
 // FP64: r0, r1 scaled by (eps + e0^2)^2 (eps + e1^2)^2.  A reciprocal for each
-// value: one for both, of the product of the sums, takes as many operations
-// and ends the range of eps and of the jumps at the fourth root of FP64's.
+// value: one for both, of the product of the sums, takes an operation more and
+// ends the range of eps and of the jumps at the fourth root of FP64's.
 template <typename T>
 JF_HD void weno3_cell(T vm1, T v0, T vp1, T eps, T& right, T& left) {
   const T e0 = v0 - vm1, e1 = vp1 - v0;
@@ -508,9 +508,14 @@ JF_HD void weno3_cell(T vm1, T v0, T vp1, T eps, T& right, T& left) {
   }
   const T Sr = r0 + T(2) * r1, Sl = r1 + T(2) * r0;
   const T p0 = r0 * e0, p1 = r1 * e1;
-  const T nr = p0 + T(2) * p1, nl = p1 + T(2) * p0;
-  right = v0 + nr * trcp(T(2) * Sr);
-  left = v0 - nl * trcp(T(2) * Sl);
+  if constexpr (sizeof(T) == 8) {  // halves taken in the numerators
+    right = fma(fma(T(0.5), p0, p1), trcp(Sr), v0);
+    left = fma(-fma(T(0.5), p1, p0), trcp(Sl), v0);
+  } else {
+    const T nr = p0 + T(2) * p1, nl = p1 + T(2) * p0;
+    right = v0 + nr * trcp(T(2) * Sr);
+    left = v0 - nl * trcp(T(2) * Sl);
+  }
 }
 __device__ __forceinline__ float2 weno3_pair(float2 vm1, float2 v0, float2 vp1, float eps) {
   return make_float2(weno3(vm1.x, v0.x, vp1.x, eps), weno3(vm1.y, v0.y, vp1.y, eps));
