@@ -149,6 +149,19 @@ template <> JF_HD double trcp<double>(double x) {
 #endif
 }
 
+// 1 / sqrt(x) in FP64, x > 0, one third-order step (Halley): 0.8 ulp, for the
+// weights of a Roe average, which scale differences only.
+JF_HD double trsqrt(double x) {
+#ifdef __CUDA_ARCH__
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+#else
+  return 1.0 / sqrt(x);
+#endif
+}
+
 template <typename T> JF_HD T tsqrt(T x);
 template <> JF_HD float tsqrt<float>(float x) { return sqrtf(x); }
 template <> JF_HD double tsqrt<double>(double x) {
@@ -645,8 +658,8 @@ JF_HD void hllc_star(double r, double p, double un, double E, double mass, doubl
 template <int D>
 JF_HD void hllc_einfeldt(const double WL[5], const double WR[5], const Gas<double>& g, double F[5]) {
   const double rL = WL[0], rR = WR[0], pL = WL[4], pR = WR[4], unL = WL[1 + D], unR = WR[1 + D];
-  const double inv = trcp(rL * rR), irL = rR * inv, irR = rL * inv, q = tsqrt(rR * irL);
-  const double aL = g.gamma * pL * irL, aR = g.gamma * pR * irR;  // c_K^2
+  const double rr = rL * rR, gi = g.gamma * trcp(rr), q = rR * trsqrt(rr);  // q = sqrt(rho_R / rho_L)
+  const double aL = pL * rR * gi, aR = pR * rL * gi;                       // c_K^2
   const double wL = trcp(1.0 + q), wR = q * wL;
   const double du = WR[1] - WL[1], dv = WR[2] - WL[2], dw = WR[3] - WL[3];
   const double jump = fma(dw, dw, fma(dv, dv, du * du));
