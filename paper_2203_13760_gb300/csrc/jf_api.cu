@@ -152,8 +152,7 @@ static const int kZChunks[] = {0, 32, 16, 64, 8};
 // as the hardware issues them, each costing its planes plus kPrologue planes
 // for its prologue (six plane loads and a face, measured at about half a
 // plane), over `slots` resident CTA slots.
-static double schedule_length(long long tiles, int nz, int z, long long slots) {
-  constexpr double kPrologue = 0.5;
+static double schedule_length(long long tiles, int nz, int z, long long slots, double kPrologue = 0.5) {
   std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
   for (long long i = 0; i < slots; ++i) free_at.push(0.0);
   double end = 0.0;
@@ -269,6 +268,26 @@ bool tall_tiles_preferred(const jf_grid* grids, int n, int bx, int by, int tall,
   return wq < wt || wt > 2;
 }
 
+// The same choice for single 3D grids (32 x 8 in the place of 32 x 7): the shorter
+// schedule of planes, a plane of the taller tile taking 1.13 times one of the
+// lower (inviscid; viscous 1.21, reconstructed per face), and a CTA 1.5 planes
+// for its prologue; and the taller tile wherever only its CTAs fit one per SM.
+// Measured, walled WENO3 stage in us, 32 x 7 and 32 x 8: inviscid 32^3 13.2 and 12.5,
+// 40^3 17.4 and 18.7, 48^3 21.7 and 19.0, 64^3 30.2 and 28.9, 112^3 143 and 122, 128^3 150
+// and 200; viscous 48^3 27.2 and 25.6, 64^3 39.5 and 40.6, 112^3 192 and 181, 128^3 201 and
+// 302.
+bool tall_tiles_preferred_3d(const jf_grid& g, int bx, int by, int tall, bool visc, int ctas_per_sm, int sms) {
+  const long long c = (g.nx + bx - 1) / bx, t = c * ((g.ny + by - 1) / by), q = c * ((g.ny + tall - 1) / tall);
+  const int zt = zchunk_rule(g.nx, g.ny, g.nz, bx, by, ctas_per_sm, sms);
+  const int zq = zchunk_rule(g.nx, g.ny, g.nz, bx, tall, ctas_per_sm, sms);
+  const long long nt = t * ((g.nz + zt - 1) / zt), nq = q * ((g.nz + zq - 1) / zq);
+  if (nq <= sms && nt > sms) return true;
+  const double plane = visc ? 1.21 : 1.13;
+  if (nt > 400000) return plane * q < t;  // many waves (bounds the host's work)
+  const long long slots = (long long)sms * ctas_per_sm;
+  return plane * schedule_length(q, g.nz, zq, slots, 1.5) < schedule_length(t, g.nz, zt, slots, 1.5);
+}
+
 // 2D FP64 grids: the FP64 pipe is shared by an SM's warps, so a launch takes
 // the busiest SM's tiles times the warp tasks of a tile (2 BY + 3
 // reconstructions and 2 BY + 2 faces).  The tile shape with the fewest: small
@@ -305,9 +324,11 @@ jf_status select_variant(jf_ctx* h, int v, bool prepare) {
         const StageVariant<T>& t0 = tab[list[0].first];
         if (rows_preferred(&h->grid, 1, r.bx, r.minb, t0.bx, t0.by, h->sms)) v = i;
         break;
-      } else if (sizeof(T) == 4 && h->dim == 2 && scheme_kind(h) == SCH_GENERAL_EXT && tab[list[i].first].by == 8) {
+      } else if (sizeof(T) == 4 && h->dim >= 2 && scheme_kind(h) == SCH_GENERAL_EXT && tab[list[i].first].by == 8) {
         const StageVariant<T>& t0 = tab[list[0].first];
-        if (tall_tiles_preferred(&h->grid, 1, t0.bx, t0.by, 8, 2 * h->sms)) v = i;
+        if (h->dim == 2 ? tall_tiles_preferred(&h->grid, 1, t0.bx, t0.by, 8, 2 * h->sms)
+                        : tall_tiles_preferred_3d(h->grid, t0.bx, t0.by, 8, visc, t0.minb, h->sms)) v = i;
+        if (h->dim == 3) break;  // its first chunk, the automatic one
       }
   }
   if (v >= (int)list.size()) { set_error(h, "variant index out of range"); return JF_ERR_ARG; }

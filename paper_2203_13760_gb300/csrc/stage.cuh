@@ -340,6 +340,14 @@ constexpr bool overlapped_launch(int s) { return !sch_roe(s); }
 // values of a plane in shared memory): the default scheme and the run-time
 // Godunov schemes.
 constexpr bool sch_pc(int s) { return s == SCH_DEFAULT || sch_general(s); }
+// The viscous FP32 kernels of the extended forms in 32 x 8 tiles (nine warps,
+// 112 registers at two CTAs per SM) reconstruct at every face: with the
+// per-cell state they spill (3D walled WENO3 stage, 112^3: 243 us against 181; 2D,
+// 1024^2: 61.5 against 60.0).
+template <typename T, int DIM, bool VISC, int BY>
+constexpr bool per_cell(int s) {
+  return sch_pc(s) && !(s == SCH_GENERAL_EXT && VISC && sizeof(T) == 4 && plane_dims(DIM) == 2 && BY == 8);
+}
 
 // Flux-splitting face flux of the ROE setup (Section 3.3, Flux-Splitting
 // approach; Section 5): Roe average of the two cells beside the face, the
@@ -862,10 +870,10 @@ __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& 
     }
   };
 
-  // per-cell families (sch_pc): WENO5 runs once per cell and direction (weno5_cell), the
+  // per-cell families (per_cell): WENO5 runs once per cell and direction (weno5_cell), the
   // face values of a plane kept in shared memory (x, y; along z only the
   // current cell's value at its upper face, zl, is kept, by its column)
-  constexpr bool PC = sch_pc(SCH);
+  constexpr bool PC = per_cell<T, DIM, VISC, BY>(SCH);
   // Overlapped loads in the prologue of a march: inviscid default kernels and
   // FP64, where they cost nothing else (64 uneven 2D grids: 248 -> 241 us per
   // stage; the viscous FP32 and ROE kernels, at their 128 registers, schedule
@@ -1437,7 +1445,7 @@ __global__ void __launch_bounds__(Geo<BX, BY, DIM, VISC>::NT, MINB)
     asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
     const size_t need = sizeof(T) * (SCH == SCH_NN ? nn_smem_offset<T, DIM, VISC, BX, BY>() + nn_smem_elems<T, DIM, Geo<BX, BY, DIM, VISC>::NT>()
                                                    : stage_smem_elems<T, DIM, VISC, BX, BY>() +
-                                                         (sch_pc(SCH) ? recon_smem_elems<DIM, BX, BY, T>() : 0));
+                                                         (per_cell<T, DIM, VISC, BY>(SCH) ? recon_smem_elems<DIM, BX, BY, T>() : 0));
     if (!JF_CHECK(dyn >= need, "JFDBG smem %u < %llu\n", dyn, (unsigned long long)need)) return;
     if (work && threadIdx.x == 0)
       for (int i = blockIdx.x; i < nwork; i += gridDim.x) {
