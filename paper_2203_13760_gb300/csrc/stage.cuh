@@ -168,8 +168,8 @@ struct PlaneRegs {
 // tile at (gx0, gy0).
 // WALLS: the kernel handles slip walls (only the extended and Rusanov-NN
 // kernel families; the host routes every walled grid to one of them).
-// NC: the kernel is launched after its predecessor has finished (the ROE
-// families), so that its loads may be read-only ones.
+// NC: the kernel is launched after its predecessor has finished
+// (!overlapped_launch), so that its loads may be read-only ones.
 template <bool NC, typename T>
 __device__ __forceinline__ T ld_input(const T* p) {
   if constexpr (NC) return __ldg(p);
@@ -334,8 +334,9 @@ constexpr bool sch_roe(int s) { return s == SCH_ROE || s == SCH_ROE_EXT; }
 constexpr bool sch_ext(int s) { return s == SCH_GENERAL_EXT || s == SCH_ROE_EXT || s == SCH_NN; }
 // Families launched by launch_next.  The ROE kernels are launched the plain way:
 // the wait and the loads it asks for cost them more than the overlap gives
-// (128^3 step 893 -> 917 us).
-constexpr bool overlapped_launch(int s) { return !sch_roe(s); }
+// (128^3 step 893 -> 917 us).  So are the 3D kernels of the extended forms (walled
+// WENO3 stage, 128^3 151 -> 146 us without it, viscous 112^3 190 -> 181).
+constexpr bool overlapped_launch(int s, int dim) { return !sch_roe(s) && !(s == SCH_GENERAL_EXT && dim == 3); }
 // Families whose kernels reconstruct once per cell and direction (the face
 // values of a plane in shared memory): the default scheme and the run-time
 // Godunov schemes.
@@ -819,7 +820,7 @@ template <typename T, int DIM, bool VISC, int BX, int BY, int SCH>
 __device__ __forceinline__ void stage_tile(const StageArgs<T>& A, const Gas<T>& g, int bx, int by, int bz,
                                            T* smem) {
   using G = Geo<BX, BY, DIM, VISC>;
-  constexpr bool WALLS = sch_ext(SCH), NC = !overlapped_launch(SCH);
+  constexpr bool WALLS = sch_ext(SCH), NC = !overlapped_launch(SCH, DIM);
   T* ring = smem;
   T* Fx = ring + G::RING * G::PLANE;      // [5][BY][BX+1]
   T* Fy = Fx + 5 * G::NFX;                // [5][BY+1][BX]
@@ -1438,7 +1439,7 @@ __global__ void __launch_bounds__(Geo<BX, BY, DIM, VISC>::NT, MINB)
     stage_kernel(const StageArgs<T> A0, const SimDesc<T>* sims, const WorkItem* work,
                  int nwork, int stage, const Gas<T> g) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if constexpr (overlapped_launch(SCH)) follow_predecessor();
+  if constexpr (overlapped_launch(SCH, DIM)) follow_predecessor();
 #ifdef JF_DEBUG_BOUNDS
   {
     unsigned dyn;

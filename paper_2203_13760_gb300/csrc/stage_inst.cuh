@@ -22,11 +22,25 @@ cudaError_t prepare_stage() {
                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
-template <int SCH, typename... P, typename... A>
+// NEXT: with programmatic dependence (launch_next), if the kernel allows it.
+template <bool NEXT, typename... P, typename... A>
 cudaError_t launch_stage_kernel(void (*k)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A... args) {
-  if constexpr (overlapped_launch(SCH)) return launch_next(k, grid, threads, smem, s, args...);
+  if constexpr (NEXT) return launch_next(k, grid, threads, smem, s, args...);
   k<<<grid, threads, smem, s>>>(static_cast<P>(args)...);
   return cudaGetLastError();
+}
+
+// CTAs that arrive while the predecessor's still run take the slots these leave,
+// so that a launch that fills some slots of every SM but not all may come to rest
+// on a few SMs.  An FP64 stage, which the SM's FP64 pipe bounds, then takes as long
+// as its fullest SM: 160^2 (270 CTAs, three slots per SM) 86 us against 61 by plain
+// launches, 20000 cells (667, eight) 29.6 against 20.1.  Such launches are plain;
+// fewer CTAs than SMs spread out either way, and full SMs leave no choice.
+inline bool spreads_evenly(long long ctas, int slots) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return false;
+  return ctas <= sms || (ctas + sms - 1) / sms >= slots;
 }
 
 // A.zchunk: planes per CTA of a z-march (DIM_Y2: rows of the 2D grid).
@@ -37,8 +51,12 @@ cudaError_t launch_stage(const StageArgs<T>& A0, const Gas<T>& g, cudaStream_t s
   if constexpr (DIM == DIM_Y2) rows_as_planes(A);
   const dim3 grid((A.nx + BX - 1) / BX, plane_dims(DIM) == 2 ? (A.ny + BY - 1) / BY : 1,
                   marches(DIM) ? (A.nz + A.zchunk - 1) / A.zchunk : 1);
-  return launch_stage_kernel<SCH>(stage_kernel<T, DIM, VISC, BX, BY, MINB, SCH>, grid, Geo<BX, BY, DIM, VISC>::NT,
-                                  smem, s, A, nullptr, nullptr, 0, 0, g);
+  constexpr bool next = overlapped_launch(SCH, DIM);
+  auto k = stage_kernel<T, DIM, VISC, BX, BY, MINB, SCH>;
+  constexpr unsigned nt = Geo<BX, BY, DIM, VISC>::NT;
+  if (next && sizeof(T) == 8 && MINB > 1 && !spreads_evenly((long long)grid.x * grid.y * grid.z, MINB))
+    return launch_stage_kernel<false>(k, grid, nt, smem, s, A, nullptr, nullptr, 0, 0, g);
+  return launch_stage_kernel<next>(k, grid, nt, smem, s, A, nullptr, nullptr, 0, 0, g);
 }
 
 template <typename T, int DIM, bool VISC, int BX, int BY, int MINB, int SCH>
@@ -63,8 +81,12 @@ cudaError_t launch_batch(const SimDesc<T>* sims, const WorkItem* work, int nwork
 #ifdef JF_DEBUG_BOUNDS
   A.trace = debug_trace_dev();
 #endif
-  return launch_stage_kernel<SCH>(stage_kernel<T, DIM, VISC, BX, BY, MINB, SCH>, dim3(grid),
-                                  Geo<BX, BY, DIM, VISC>::NT, smem, s, A, sims, work, nwork, stage, g);
+  // plain: persistent CTAs fill the SMs, and programmatic dependence costs a step of
+  // 64 walled 64^2 grids 7 %, viscous 10 %; the network's stages of a training step
+  // (20 boxes of 32^2, a CTA per SM) follow one another with it (2427 -> 2312 us)
+  return launch_stage_kernel<SCH == SCH_NN && overlapped_launch(SCH, DIM)>(stage_kernel<T, DIM, VISC, BX, BY, MINB, SCH>, dim3(grid),
+                                                                           Geo<BX, BY, DIM, VISC>::NT, smem, s, A, sims,
+                                                                           work, nwork, stage, g);
 }
 
 template <typename T, int DIM, bool VISC, int BX, int BY, int MINB, int SCH>
