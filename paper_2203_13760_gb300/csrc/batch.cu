@@ -11,6 +11,7 @@
 // the simulations' field pointers from device descriptors, so rebinding new
 // fields only rewrites the descriptors.
 #include <cstdio>
+#include <algorithm>
 #include <cstring>
 #include <vector>
 
@@ -72,6 +73,23 @@ std::vector<std::pair<int, int>> batch_variant_list(int dim, bool visc, int kind
   return out;
 }
 
+// Planes of the fullest of `slots` persistent CTAs that share the 3D items (tile
+// columns by chunks of `rows` planes) round robin, a chunk's prologue counting
+// 1.5 planes.
+double round_robin_planes(const std::vector<jf_grid>& grids, int bx, int by, int rows, int slots) {
+  std::vector<double> load(slots > 0 ? slots : 1, 0.0);
+  size_t next = 0;
+  for (const jf_grid& g : grids) {
+    const long long cols = (long long)((g.nx + bx - 1) / bx) * ((g.ny + by - 1) / by);
+    for (int z = 0; z < g.nz; z += rows)
+      for (long long c = 0; c < cols; ++c) {
+        load[next] += (g.nz - z < rows ? g.nz - z : rows) + 1.5;
+        next = next + 1 == load.size() ? 0 : next + 1;
+      }
+  }
+  return *std::max_element(load.begin(), load.end());
+}
+
 // (Re)build the work list for the tile shape of the selected variant.
 template <typename T>
 jf_status setup_variant(jf_ctx* h, int v) {
@@ -91,6 +109,14 @@ jf_status setup_variant(jf_ctx* h, int v) {
       } else if (sizeof(T) == 4 && h->dim == 2 && scheme_kind(h) == SCH_GENERAL_EXT && tab[list[i].first].by == 8) {
         const StageVariant<T>& t0 = tab[list[0].first];
         if (tall_tiles_preferred(h->grids.data(), h->nsim, t0.bx, t0.by, 8, 2 * h->sms)) v = i;
+      } else if (sizeof(T) == 4 && h->dim == 3 && scheme_kind(h) == SCH_GENERAL_EXT && tab[list[i].first].by == 8) {
+        // the weights of tall_tiles_preferred_3d (walled WENO3 step, 32 x 7 and 32 x 8: eight
+        // 64^3 grids 827 and 534 us, sixteen of 24 to 64 cells a side 807 and 702)
+        const StageVariant<T>& t0 = tab[list[0].first];
+        const int slots = t0.minb * h->sms, rows = list[i].second;
+        if ((visc ? 1.21 : 1.13) * round_robin_planes(h->grids, t0.bx, 8, rows, slots) <
+            round_robin_planes(h->grids, t0.bx, t0.by, rows, slots)) v = i;
+        break;
       }
   }
   if (v >= (int)list.size()) { set_error(h, "batch: variant index out of range"); return JF_ERR_ARG; }
