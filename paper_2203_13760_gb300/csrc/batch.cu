@@ -114,7 +114,7 @@ jf_status setup_variant(jf_ctx* h, int v) {
         // 64^3 grids 827 and 534 us, sixteen of 24 to 64 cells a side 807 and 702)
         const StageVariant<T>& t0 = tab[list[0].first];
         const int slots = t0.minb * h->sms, rows = list[i].second;
-        if ((visc ? 1.21 : 1.13) * round_robin_planes(h->grids, t0.bx, 8, rows, slots) <
+        if ((visc ? 1.24 : 1.13) * round_robin_planes(h->grids, t0.bx, 8, rows, slots) <
             round_robin_planes(h->grids, t0.bx, t0.by, rows, slots)) v = i;
         break;
       }

@@ -270,19 +270,19 @@ bool tall_tiles_preferred(const jf_grid* grids, int n, int bx, int by, int tall,
 
 // The same choice for single 3D grids (32 x 8 in the place of 32 x 7): the shorter
 // schedule of planes, a plane of the taller tile taking 1.13 times one of the
-// lower (inviscid; viscous 1.21, reconstructed per face), and a CTA 1.5 planes
-// for its prologue; and the taller tile wherever only its CTAs fit one per SM.
-// Measured, walled WENO3 stage in us, 32 x 7 and 32 x 8: inviscid 32^3 13.2 and 12.5,
-// 40^3 17.4 and 18.7, 48^3 21.7 and 19.0, 64^3 30.2 and 28.9, 112^3 143 and 122, 128^3 150
-// and 200; viscous 48^3 27.2 and 25.6, 64^3 39.5 and 40.6, 112^3 192 and 181, 128^3 201 and
-// 302.
+// lower (inviscid; viscous 1.24, reconstructed per face), and a CTA 1.5 planes
+// for its prologue; inviscid also wherever only its CTAs fit one per SM.
+// Measured, walled WENO3 stage in us, 32 x 7 and 32 x 8: inviscid 32^3 12.9 and 12.8,
+// 40^3 17.3 and 18.7, 48^3 21.6 and 19.2, 64^3 30.6 and 28.9, 112^3 143 and 119, 128^3 146
+// and 196, 256^3 1154 and 1102; viscous 48^3 27.1 and 26.0, 64^3 39.6 and 41.0, 80^3 69.5
+// and 72.0, 112^3 195 and 181, 128^3 201 and 306, 256^3 1527 and 1833.
 bool tall_tiles_preferred_3d(const jf_grid& g, int bx, int by, int tall, bool visc, int ctas_per_sm, int sms) {
   const long long c = (g.nx + bx - 1) / bx, t = c * ((g.ny + by - 1) / by), q = c * ((g.ny + tall - 1) / tall);
   const int zt = zchunk_rule(g.nx, g.ny, g.nz, bx, by, ctas_per_sm, sms);
   const int zq = zchunk_rule(g.nx, g.ny, g.nz, bx, tall, ctas_per_sm, sms);
   const long long nt = t * ((g.nz + zt - 1) / zt), nq = q * ((g.nz + zq - 1) / zq);
-  if (nq <= sms && nt > sms) return true;
-  const double plane = visc ? 1.21 : 1.13;
+  if (!visc && nq <= sms && nt > sms) return true;
+  const double plane = visc ? 1.24 : 1.13;
   if (nt > 400000) return plane * q < t;  // many waves (bounds the host's work)
   const long long slots = (long long)sms * ctas_per_sm;
   return plane * schedule_length(q, g.nz, zq, slots, 1.5) < schedule_length(t, g.nz, zt, slots, 1.5);
