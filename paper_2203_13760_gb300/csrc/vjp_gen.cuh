@@ -264,15 +264,19 @@ constexpr int kHRow = NN_HIDDEN + 4;
 
 // acc += sum_j h[j] W[j][:] over the rows of W (pitch PITCH), h (16-byte
 // aligned) read four at a time; a loop, so that the code of a network pass
-// stays small.
-template <int PITCH, typename T>
+// stays small.  SPARSE: h holds zeros for inactive units, whose rows FP64 skips
+// (the FP64 pipe bounds it, and the faces of a warp share most of them: adjoint
+// step with the network, 128^2, 2321 us without, 2050 with; its parameter gradient too
+// 4383 and 3807).
+template <int PITCH, bool SPARSE = false, typename T>
 __device__ __forceinline__ void nn_rows(const T* W, const T* h, HRow<T>& acc) {
 #pragma unroll 1
   for (int j = 0; j < NN_HIDDEN; j += 4) {
     T q[4];
     ld4(h + j, q);
 #pragma unroll
-    for (int m = 0; m < 4; ++m) acc.axpy(W + (j + m) * PITCH, q[m]);
+    for (int m = 0; m < 4; ++m)
+      if (!SPARSE || sizeof(T) == 4 || q[m] != T(0)) acc.axpy(W + (j + m) * PITCH, q[m]);
   }
 }
 
@@ -327,12 +331,12 @@ __device__ __forceinline__ T nn_alpha_grad(const T* th, const T x[4], T dx[4], T
   for (int j = 0; j < NN_HIDDEN; ++j) h.set(j, h.get(j) > T(0) ? alpha * th[kNnW4 + j] : T(0));
   h.store(h2);
   h.fill(T(0));
-  nn_rows<NN_HIDDEN>(th + kNnW3, h2, h);
+  nn_rows<NN_HIDDEN, true>(th + kNnW3, h2, h);
 #pragma unroll
   for (int j = 0; j < NN_HIDDEN; ++j) h.set(j, (m2 >> j) & 1u ? h.get(j) : T(0));
   h.store(h1);
   h.fill(T(0));
-  nn_rows<NN_HIDDEN>(th + kNnW2, h1, h);
+  nn_rows<NN_HIDDEN, true>(th + kNnW2, h1, h);
 #pragma unroll
   for (int m = 0; m < 4; ++m) dx[m] = T(0);
 #pragma unroll
@@ -679,7 +683,7 @@ __global__ void __launch_bounds__(32 * kNnWarps, sizeof(T) == 4 ? 2 : 1) nn_para
     for (int r = 0; r < 32; ++r) a3.outer(R3 + r * kHRow + br, R2 + r * kHRow + bc);
     // G2 into R3: g2[j] = [h2_j > 0] sum_i W3[i][j] g3[i]
     v.fill(T(0));
-    nn_rows<NN_HIDDEN>(TH + kNnW3, r3, v);
+    nn_rows<NN_HIDDEN, true>(TH + kNnW3, r3, v);
 #pragma unroll
     for (int j = 0; j < NN_HIDDEN; j += 4) {
       T q[4];
@@ -699,7 +703,7 @@ __global__ void __launch_bounds__(32 * kNnWarps, sizeof(T) == 4 ? 2 : 1) nn_para
     __syncwarp();
     // G1 into R3: g1[k] = [h1_k > 0] sum_j W2[j][k] g2[j]
     v.fill(T(0));
-    nn_rows<NN_HIDDEN>(TH + kNnW2, r3, v);
+    nn_rows<NN_HIDDEN, true>(TH + kNnW2, r3, v);
 #pragma unroll
     for (int j = 0; j < NN_HIDDEN; j += 4) {
       T q[4];
