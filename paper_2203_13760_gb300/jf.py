@@ -474,8 +474,11 @@ class Batch:
                 if (not t_.is_cuda or t_.dtype != self.dtype or not t_.is_contiguous()
                         or tuple(t_.shape) != (int(nsteps) + 1, 5, g.nz, g.ny, g.nx)):
                     raise ValueError(f"trajectory {i} has the wrong shape / dtype / device")
-        if dt.dtype != torch.float64 or not dt.is_cuda or dt.numel() != self.nsim:
-            raise ValueError("dt must be a float64 CUDA tensor of one step per simulation")
+        if dt.dtype != torch.float64 or not dt.is_cuda or not dt.is_contiguous() or dt.numel() != self.nsim:
+            raise ValueError("dt must be a contiguous float64 CUDA tensor of one step per simulation")
+        if theta_bar is not None and (theta_bar.dtype != self.dtype or not theta_bar.is_cuda
+                                      or not theta_bar.is_contiguous() or theta_bar.numel() != NN_PARAMS):
+            raise ValueError(f"theta_bar must be a contiguous CUDA {self.dtype} tensor of {NN_PARAMS} values")
         lam0 = [torch.empty(tuple(t_.shape[1:]), dtype=self.dtype, device="cuda") for t_ in trajs]
         arr = lambda ts: (ctypes.c_void_p * self.nsim)(*[x.data_ptr() for x in ts])  # noqa: E731
         _check(lib().jf_batch_feed_forward_vjp(self.h, arr(trajs), arr(grads), int(nsteps), _ptr(dt), arr(lam0),
