@@ -790,7 +790,7 @@ template <> JF_HD double tlog<double>(double x) { return log(x); }
 // Not inlined: one copy of the ~2200 multiply-adds serves every face
 // direction, and its 64 hidden values do not add to the register pressure
 // of the tile code around the call.
-#ifdef __CUDACC__
+#if defined(__CUDACC__) || defined(JF_HOST_FLOAT4)  // (a host build that has float4)
 // Four consecutive network parameters (or hidden-row values) from a 16-byte
 // aligned address: every weight row of the parameter layout starts at a
 // multiple of 4 elements, and the kernels place the parameters at a 16-byte
@@ -885,7 +885,7 @@ JF_HD int nn_transposed(int i) {
   return -1;
 }
 
-#ifdef __CUDACC__
+#if defined(__CUDACC__) || defined(JF_HOST_FLOAT4)
 // nn_alpha of two faces (the lanes of x), from the parameters th and the
 // transposed weights tt (16-byte aligned): per face the operations of nn_alpha
 // in its order, so the same bits.  Two outputs of a layer share a packed FP32x2
