@@ -331,7 +331,7 @@ jf_status jf_batch_step(jf_handle batch, void* const* U_ptrs, int nsteps, double
  * per simulation since sizes may differ).  dt_dev: device array of nsim FP64
  * steps.  The integrator of the scheme is used; the arithmetic is that of
  * jf_batch_step and jf_rk3_step, so slot t equals t fixed-dt steps of the
- * single-grid path bit for bit.  Asynchronous on `stream`, which must not be
+ * single-grid path with the same tile shape (jf_set_variant) bit for bit.  Asynchronous on `stream`, which must not be
  * in capture. */
 jf_status jf_batch_feed_forward(jf_handle batch, void* const* U0_ptrs, void* const* traj_ptrs, int nsteps,
                                 const double* dt_dev, void* stream);

@@ -288,12 +288,16 @@ bool tall_tiles_preferred_3d(const jf_grid& g, int bx, int by, int tall, bool vi
   return plane * schedule_length(q, g.nz, zq, slots, 1.5) < schedule_length(t, g.nz, zt, slots, 1.5);
 }
 
-// 2D FP64 grids: the FP64 pipe is shared by an SM's warps, so a launch takes
-// the busiest SM's tiles times the warp tasks of a tile (2 BY + 3
+// Single 2D FP64 grids: the FP64 pipe is shared by an SM's warps, so a launch
+// takes the busiest SM's tiles times the warp tasks of a tile (2 BY + 3
 // reconstructions and 2 BY + 2 faces).  The tile shape with the fewest: small
 // grids are spread over the SMs with 32 x 3 or 32 x 4 tiles, large ones take
-// 32 x 8.  Measured, walled WENO3 stage: 128^2 31.0 us with 32 x 4 (rule: 21
-// tasks), 46.9 with 32 x 8 (37); 256^2 99.1 (84) and 93.0 (74).
+// 32 x 8.  Measured over 32^2 to 1024^2 and ragged grids of the default, run-time,
+// walled (WENO5, WENO3) and ROE families, inviscid and viscous: never more than
+// 0.3 % off the best shape.  Stage in us with 32 x 3, 32 x 4, 32 x 8: default 64^2 37.4,
+// 45.3, 68.6, 128^2 61.5, 45.5, 68.7, 160^2 61.5, 72.9, 68.9, 256^2 146, 143, 136; walled
+// WENO3 64^2 25.5, 29.3, 44.4, 128^2 39.9, 29.2, 44.5, 256^2 94.6, 94.3, 88.1; ROE (no
+// 32 x 3) 64^2 84.2, 137, 256^2 308, 274.
 template <typename T>
 int f64_tile(const jf_ctx* h, const std::vector<std::pair<int, int>>& list) {
   int count = 0, best = 0;

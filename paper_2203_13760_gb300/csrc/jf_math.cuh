@@ -34,10 +34,11 @@ namespace jf {
 // read-only during the whole kernel and may move above the wait.  A launch after a
 // copy, a memset or another library's kernel waits for that as usual.
 //
-// Before and after: FP64 step of a 200-cell tube 39.5 -> 31 us (four dependent
-// launches of a few us each), 97 x 61 x 43 step 139 -> 132 us, gradient of eight
-// 256^2 steps 2.90 -> 2.4 ms, a training step on a 32^2 batch 2.63 -> 2.49 ms;
-// steps of a millisecond and more within 1 %.
+// Before and after: FP64 step of a 200-cell tube 39 -> 32 us (four dependent
+// launches of a few us each), 107 x 61 x 45 step 139 -> 132 us, gradient of 24
+// 256^2 steps 2.78 -> 2.50 ms, a training step on a 32^2 batch 2.53 -> 2.31 ms;
+// steps of a millisecond and more within 1 %.  Where it costs time the launch is
+// plain (overlapped_launch, spreads_evenly and launch_batch).
 
 __device__ __forceinline__ void follow_predecessor() {
 #ifdef __CUDA_ARCH__
@@ -303,11 +304,11 @@ JF_HD void weno5_cell_lean(T vm2, T vm1, T v0, T vp1, T vp2, T eps, T& right, T&
   }
 }
 
-// The FP32 tile kernels (1D, 2D, 3D) keep an earlier grouping of the same
-// formulas, with three independent indicators: their states enter numbers
-// that are reported in FP64 (the CFL step, the loss at the end of a
-// trajectory), which another FP32 rounding moves by 1e-9 to 1e-7.  The lean
-// form above serves the row tiles and FP64 (see cell_recon).
+// The FP32 tile kernels (1D, 2D, 3D) have an earlier grouping of the same
+// formulas, with three independent indicators, of the same accuracy.  The lean
+// form above, which serves the row tiles and FP64 (see cell_recon), would take
+// 4 to 6 % off them; its other rounding moves a loss that is formed in FP64 from
+// FP32 states by 1e-9 to 1e-7.
 template <typename T>
 JF_HD void weno5_cell(T vm2, T vm1, T v0, T vp1, T vp2, T eps, T& right, T& left, int z = 0) {
   if constexpr (sizeof(T) == 8) {

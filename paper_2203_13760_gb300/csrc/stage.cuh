@@ -778,7 +778,7 @@ __device__ __forceinline__ void cell_recon(const RingView<T, BX, BY, DIM, VISC>&
   }
   if constexpr (sizeof(T) == 4) {
     // row tiles: the lean form (5 % less time per stage: 1024^2 62.5 -> 59.1 us,
-    // 64 uneven grids 261 -> 248 us); the tiles keep their rounding (weno5_cell)
+    // 64 uneven grids 261 -> 248 us); the tiles: weno5_cell
     constexpr bool LEAN = DIM == DIM_Y2;
     auto two = [&](int a, int b) {
       auto pr = [&](int n) { return make_float2(val(a, n), val(b, n)); };
@@ -1464,7 +1464,7 @@ __global__ void __launch_bounds__(Geo<BX, BY, DIM, VISC>::NT, MINB)
   if constexpr (SCH == SCH_NN) {
     // the Rusanov-NN parameters, after the stage buffers at a 16-byte
     // aligned offset (the launch adds them to the dynamic shared memory)
-    // (and, FP32 tiles spanning y, once more with every value twice)
+    // (FP32 tiles spanning y: W1, W2 and W3 once more, transposed)
     T* th = reinterpret_cast<T*>(smem_raw) + nn_smem_offset<T, DIM, VISC, BX, BY>();
     block_copy(g.nn, NN_PARAMS, [&](int i, T v) {
       th[i] = v;
