@@ -26,7 +26,7 @@ constexpr long long kChunk = 16384;  // cells per CFL CTA (a whole number of vec
 // pointers read from the device descriptors so that rebinding stays valid.
 template <typename T>
 __global__ void __launch_bounds__(256) batch_copy_kernel(const SimDesc<T>* sims) {
-  follow_predecessor();
+  follow_predecessor<sizeof(T) == 4>();
   const SimDesc<T> d = sims[blockIdx.y];
   const long long n = 5 * d.N;
 #ifdef JF_DEBUG_BOUNDS
@@ -43,7 +43,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) batch_copy_pairs_kernel(const T* const* src,
                                                                T* const* dst,
                                                                const long long* count) {
-  follow_predecessor();
+  follow_predecessor<sizeof(T) == 4>();
   const T* a = src[blockIdx.y];
   T* b = dst[blockIdx.y];
   const long long n = count[blockIdx.y];

@@ -17,24 +17,31 @@ struct CflChunk {
   long long begin, end;
 };
 
-// CTAs of a single-grid pass over N cells: one vector of cells per thread,
-// at most two CTAs per SM.  Their atomics on one address, not the loads, took
-// most of the pass on mid-size grids: with up to eight CTAs of 256 threads
+// Threads and CTAs of a single-grid pass over N cells: one vector of cells per
+// thread, at most two CTAs per SM.  Their atomics on one address, not the loads,
+// took most of the pass on mid-size grids: with up to eight CTAs of 256 threads
 // per SM (and the CTA count set by cells, so that three quarters of them had
-// no vector) it took 18 us at 1024^2 FP32.
+// no vector) it took 18 us at 1024^2 FP32.  CTAs of 512 threads in FP32; in FP64,
+// where a cell's division and root keep the SM's FP64 pipe busy, as few as leave no
+// SM idle, from 128 on (24^3: 13.8 us with 14 CTAs of 512, 7.4 with 54 of 128).
+// Tiny grids take one CTA of whole warps.
+template <typename T>
+inline unsigned cfl_threads(long long N, int sms) {
+  constexpr int V = 16 / (int)sizeof(T);
+  const long long units = N % V == 0 ? N / V : N;
+  long long t = kCflThreads;
+  if (sizeof(T) == 8) {
+    t = ((units + sms - 1) / sms + 31) / 32 * 32;
+    t = t < 128 ? 128 : (t > kCflThreads ? kCflThreads : t);
+  }
+  return (unsigned)(units >= t ? t : (units + 31) / 32 * 32);
+}
 template <typename T>
 inline unsigned cfl_blocks(long long N, int sms) {
   constexpr int V = 16 / (int)sizeof(T);
-  const long long units = N % V == 0 ? N / V : N;
-  const long long b = (units + kCflThreads - 1) / kCflThreads, cap = 2LL * sms;
-  return (unsigned)(b < 1 ? 1 : (b > cap ? cap : b));
-}
-// Threads of its CTAs: whole warps with a vector each (one CTA for tiny grids).
-template <typename T>
-inline unsigned cfl_threads(long long N) {
-  constexpr int V = 16 / (int)sizeof(T);
-  const long long units = N % V == 0 ? N / V : N;
-  return units >= kCflThreads ? kCflThreads : (unsigned)((units + 31) / 32 * 32);
+  const long long units = N % V == 0 ? N / V : N, t = cfl_threads<T>(N, sms);
+  const long long b = (units + t - 1) / t, cap = 2LL * sms;
+  return (unsigned)(b > cap ? cap : b);
 }
 
 template <typename T>
@@ -44,7 +51,7 @@ __global__ void __launch_bounds__(kCflThreads) cfl_kernel(const T* U0, CflArgs a
                                                   const CflChunk* chunks,
                                                   const CflArgs* args, ReduceScratch* red,
                                                   double* dts) {
-  follow_predecessor();
+  follow_predecessor<sizeof(T) == 4>();
   const T* U;
   CflArgs a;
   ReduceScratch* sc;

@@ -422,7 +422,7 @@ template <typename T>
 jf_status cfl_impl(jf_ctx* h, const void* U, double* dt_out, double* dt_out2, cudaStream_t s) {
   const CflArgs a = make_cfl(h->grid, h->gas, h->scheme);
   const cudaError_t e =
-      launch_next(cfl_kernel<T>, dim3(cfl_blocks<T>(a.N, h->sms)), cfl_threads<T>(a.N), 0, s, static_cast<const T*>(U), a,
+      launch_next(cfl_kernel<T>, dim3(cfl_blocks<T>(a.N, h->sms)), cfl_threads<T>(a.N, h->sms), 0, s, static_cast<const T*>(U), a,
                   h->red_cfl, dt_out, dt_out2, h->flag, nullptr, nullptr, nullptr, nullptr, nullptr);
   if (e != cudaSuccess) return cuda_fail(h, e, "cfl kernel launch");
   return JF_OK;

@@ -40,10 +40,16 @@ namespace jf {
 // steps of a millisecond and more within 1 %.  Where it costs time the launch is
 // plain (overlapped_launch, spreads_evenly and launch_batch).
 
+// LET: let the successor's CTAs in now (else as this kernel ends).  FP64 kernels
+// other than the stages do not: a stage that fills one slot of most SMs comes to
+// rest two to an SM where its predecessor's CTAs leave fewer SMs empty than it
+// has CTAs (FP64 128^2 step, after the CFL pass: 224 us with the early release,
+// 147 without).
+template <bool LET = true>
 __device__ __forceinline__ void follow_predecessor() {
 #ifdef __CUDA_ARCH__
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (LET) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 #endif
 }
 

@@ -148,7 +148,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) loss_density_kernel(const T* U, const T* target,
                                                            long long N, double dV, ReduceScratch* sc,
                                                            double* loss, T* seed) {
-  follow_predecessor();
+  follow_predecessor<sizeof(T) == 4>();
   double s = 0.0;
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < N; q += stride) {

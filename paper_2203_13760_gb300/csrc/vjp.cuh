@@ -162,7 +162,7 @@ template <typename T, int DIM, bool VISC, int BX, int BY, int MINB, int NT>
 __global__ void __launch_bounds__(NT, MINB) vjp_stage_kernel(const VjpArgs<T> A, const Gas<T> g) {
   using G = VGeo<BX, BY, DIM, VISC>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  follow_predecessor();
+  follow_predecessor<sizeof(T) == 4>();
   T* Wb = reinterpret_cast<T*>(smem_raw);
   T* Mb = Wb + G::NCW * G::CS;
   T* acc = Mb + 5 * G::MCS;

@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(NT, MINB)
     vjp3_kernel(const VjpArgs<T> A, const Gas<T> g, T* __restrict__ Gacc, int zchunk) {
   using G = V3Geo<BX, BY, VISC>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  follow_predecessor();
+  follow_predecessor<sizeof(T) == 4>();
   T* Wr = reinterpret_cast<T*>(smem_raw);  // [RING][NCW][PY][PX]
   T* Ar = Wr + G::RING * G::PLANE;         // [ARING][NCW][PY][PX]
   T* Mr = Ar + G::ARING * G::PLANE;        // [2][5][MPY][MPX]
@@ -602,7 +602,7 @@ __global__ void __launch_bounds__(NT, MINB)
 template <typename T, bool VISC>
 __global__ void __launch_bounds__(256) vjp3_finish_kernel(const VjpArgs<T> A, const Gas<T> g,
                                                           const T* Gacc) {
-  follow_predecessor();
+  follow_predecessor<sizeof(T) == 4>();
   const long long N = A.N;
   const T dt = T(*A.dt);
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < N; q += (long long)gridDim.x * blockDim.x) {

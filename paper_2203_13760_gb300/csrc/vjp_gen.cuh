@@ -74,7 +74,7 @@ __device__ __forceinline__ int find_sim(const long long* base, int nsim, long lo
 // out = a1 x1 + a2 x2 + a3 x3 + s_in lam, every cell of every grid
 template <typename T>
 __global__ void __launch_bounds__(256) gvjp_point_kernel(const GVjpBatch<T> B) {
-  follow_predecessor();
+  follow_predecessor<sizeof(T) == 4>();
   const long long total = B.cell_base[B.nsim];
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
@@ -561,7 +561,7 @@ constexpr size_t gvjp_face_smem_bytes() {
 template <typename T, int DIM, int RECON, int FLUX>
 __global__ void __launch_bounds__(kGvjpThreads, sizeof(T) == 4 ? 5 : 1) gvjp_face_kernel(const GVjpBatch<T> B, const Gas<T> g) {
   extern __shared__ __align__(16) unsigned char gvjp_smem[];
-  follow_predecessor();
+  follow_predecessor<sizeof(T) == 4>();
   T* th = reinterpret_cast<T*>(gvjp_smem);  // the network parameters (Rusanov-NN)
   T* h1 = th + kNnShared + threadIdx.x * kHRow;
   T* h2 = h1 + kGvjpThreads * kHRow;
@@ -624,7 +624,7 @@ __global__ void __launch_bounds__(32 * kNnWarps, sizeof(T) == 4 ? 2 : 1) nn_para
                                                                       const T* rec, long long nrec,
                                                                       T* grad) {
   extern __shared__ __align__(16) unsigned char nn_smem[];
-  follow_predecessor();
+  follow_predecessor<sizeof(T) == 4>();
   T* TH = reinterpret_cast<T*>(nn_smem);
   nn_stage(theta, TH);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
