@@ -30,6 +30,16 @@ extern thread_local uint3 blockIdx;
 extern dim3 blockDim, gridDim;
 void emu_syncthreads();
 #define __syncthreads() emu_syncthreads()
+inline int __syncthreads_or(int p) {
+  static int any = 0;
+  if (p) __atomic_store_n(&any, 1, __ATOMIC_RELAXED);
+  emu_syncthreads();
+  const int r = __atomic_load_n(&any, __ATOMIC_RELAXED);
+  emu_syncthreads();
+  __atomic_store_n(&any, 0, __ATOMIC_RELAXED);
+  emu_syncthreads();
+  return r;
+}
 template <class T> inline T __ldg(const T* p) { return *p; }
 inline float __fdividef(float a, float b) { return a / b; }
 inline float2 __ffma2_rn(float2 a, float2 b, float2 c) { return float2{std::fmaf(a.x, b.x, c.x), std::fmaf(a.y, b.y, c.y)}; }
