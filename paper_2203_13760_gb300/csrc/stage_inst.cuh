@@ -71,12 +71,16 @@ cudaError_t launch_batch(const SimDesc<T>* sims, const WorkItem* work, int nwork
 #ifdef JF_DEBUG_BOUNDS
   A.trace = debug_trace_dev();
 #endif
-  // plain: persistent CTAs fill the SMs, and programmatic dependence costs a step of
-  // 64 walled 64^2 grids 7 %, viscous 10 %; the network's stages of a training step
-  // (20 boxes of 32^2, a CTA per SM) follow one another with it (2427 -> 2312 us)
-  return launch_stage_kernel<SCH == SCH_NN && overlapped_launch(SCH, DIM)>(stage_kernel<T, DIM, VISC, BX, BY, MINB, SCH>, dim3(grid),
-                                                                           Geo<BX, BY, DIM, VISC>::NT, smem, s, A, sims,
-                                                                           work, nwork, stage, g);
+  // Plain where the CTAs fill the SMs for several items: programmatic dependence
+  // costs a step of 64 walled 64^2 grids 7 %, viscous 10 %.  With an item per CTA (but for
+  // marches) it gives time: trajectories of eight 64^2 grids 319 us, 340 the plain
+  // way; so it does the network's stages of a training step (2312 us, 2427).
+  auto k = stage_kernel<T, DIM, VISC, BX, BY, MINB, SCH>;
+  constexpr unsigned nt = Geo<BX, BY, DIM, VISC>::NT;
+  if constexpr (overlapped_launch(SCH, DIM) && !marches(DIM))
+    if (SCH == SCH_NN || nwork <= grid)
+      return launch_stage_kernel<true>(k, dim3(grid), nt, smem, s, A, sims, work, nwork, stage, g);
+  return launch_stage_kernel<false>(k, dim3(grid), nt, smem, s, A, sims, work, nwork, stage, g);
 }
 
 template <typename T, int DIM, bool VISC, int BX, int BY, int MINB, int SCH>
