@@ -32,9 +32,9 @@
 // Summation order of the atomics, and so the last bits, may vary between
 // runs.
 //
-// Planes over which m is uniform have no x and y tasks, and equal neighbours no
-// reverse z pass (24^3 rollout of a uniform cotangent, FP64, 13.8 -> 6.0 ms; 1 % of
-// a dense one).
+// Planes over which m is uniform have no x and y tasks, and cells between equal
+// ones no reverse z pass (24^3 rollout of a uniform cotangent, FP64, 13.8 -> 6.0 ms;
+// a dense one the same within 1 %).
 //
 // Bound by latency at 18 warps per SM (one CTA fills the shared memory): a
 // scheduler issues in 50 % of its cycles (44 % with 512 threads), the rest are
@@ -329,8 +329,7 @@ __global__ void __launch_bounds__(NT, MINB)
   for (int t = threadIdx.x; t < G::ARING * G::PLANE; t += NT) Ar[t] = T(0);
   for (int t = threadIdx.x; t < G::NXY * G::CS + G::ZRING * G::NZ * G::ZC; t += NT) Cxy[t] = T(0);
   // a plane over which m is uniform (no cotangent has reached it yet, say) has no
-  // x or y face with one, two equal ones no z face between them: live, live1 for the
-  // planes k and k + 1, below for the face k - 1/2
+  // x or y face with one: live, live1 for the planes k and k + 1
   T first[5];
 #pragma unroll
   for (int c = 0; c < 5; ++c) first[c] = A.s_in * A.lam[((long long)z0 * ny + y0) * nx + x0 + c * A.N];
@@ -342,7 +341,6 @@ __global__ void __launch_bounds__(NT, MINB)
     for (int c = 0; c < 5; ++c) mref[c] = first[c];
   }
   bool live = __syncthreads_or(uneven0), live1 = __syncthreads_or(uneven1);
-  bool below = true;
 
   V3Tile<T, VISC, BX, BY> V;
   V.W = Wr;
@@ -556,7 +554,7 @@ __global__ void __launch_bounds__(NT, MINB)
     const bool more = k + 1 < kend;
     if (more) vjp3_fetch<T, VISC, BX, BY, NT>(A, nxt, x0, y0, k + 4, k + 2);
     // pass 3: reverse reconstruction of the cells
-    const int nz3 = ((k >= z0 && k < z1) || k == nz || (bottom && k < z0)) && (below || live || live1) ? ncol : 0;
+    const int nz3 = (k >= z0 && k < z1) || k == nz || (bottom && k < z0) ? ncol : 0;
     for (int t = threadIdx.x; t < ncx + ncy + nz3; t += NT) {
       int r = t, j, i;
       if (x_task(r, ncx, ncy + nz3, j, i)) {
@@ -567,7 +565,11 @@ __global__ void __launch_bounds__(NT, MINB)
       } else {
         r -= ncy;
         const int j = divu(r, mex), i = r - j * ex;
-        rev(Z{}, i, j, ez(k) + j * BX + i, G::ZC);
+        const T* e = ez(k) + j * BX + i;
+        bool any = false;  // a z face with a cotangent beside it
+#pragma unroll
+        for (int c = 0; c < 10; ++c) any |= e[c * G::ZC] != T(0);
+        if (any) rev(Z{}, i, j, e, G::ZC);
       }
     }
     __syncthreads();
@@ -606,7 +608,6 @@ __global__ void __launch_bounds__(NT, MINB)
     vjp3_flush<T, VISC, BX, BY, NT>(A, Ar + V.ap[0], Gacc, x0, y0, k - 2);
     bool uneven = false;
     if (more) vjp3_commit<T, VISC, BX, BY, NT>(A, g, nxt, Wr + V.wp[0], Mr + V.mp[0], mref, bad, uneven);
-    below = live || live1;
     live = live1;
     live1 = __syncthreads_or(uneven);
   }
